@@ -49,7 +49,10 @@ namespace beta {
 
 namespace {
 
-// 16-byte vector atomic add (sm_90+), into a 16-byte aligned slot
+// 8- and 16-byte vector atomic adds (sm_90+), into slots aligned to their size
+__device__ __forceinline__ void red_add_v2(float* p, float a, float b) {
+  asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
 __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c),
                "f"(d)
@@ -623,7 +626,7 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
             float* gdst = grad2d + (size_t)s_ridx[buf][s] * kGrad2dStride;
             red_add_v4(gdst + 0, G[0], G[1], G[2], G[3]);
             red_add_v4(gdst + 4, G[4], G[5], G[6], G[7]);
-            red_add_v4(gdst + 8, G[8], G[9], 0.0f, 0.0f);
+            red_add_v2(gdst + 8, G[8], G[9]);
           }
           if (kb < 0) break;
           wide &= ~(1u << kb);
@@ -656,13 +659,24 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
 // shared-memory record loads and, in the backward, one set of gradient
 // atomics serve both pixels (neighbouring pixels share most records), and the
 // warp-wide reductions of records covering many lanes serve 64 pixels.
+// The walks are bound by instruction issue (82% of the slots at half of the
+// lanes), so both pixels' arithmetic is packed (fma.rn.f32x2 and its kin, one
+// slot for two fp32 results; a record's scalar is broadcast by the
+// instruction).  Scalar to packed: 3.94e8 -> 3.49e8 forward and 5.80e8 ->
+// 5.07e8 backward instructions on 1M Betas x 4 x 1080p (16x8 / 64), the one
+// launch 3.78 -> 3.43 ms at 16 views, forward and backward 9.26 -> 8.40 and
+// 21.9 -> 20.3 ms on 6M Betas x 8 x 4K.
 // ---------------------------------------------------------------------------
 
 // Threads per SM asked of the register allocator for the pixel-pair kernels:
-// 1280 (48 registers) where the record buffers of 64-record batches leave
+// 1152 (56 registers) where the record buffers of 64-record batches leave
 // room for that many CTAs, 1024 (64 registers) for larger batches, whose
-// shared memory holds fewer CTAs anyway.
-constexpr int pair_threads_per_sm(int S) { return S <= 64 ? 1280 : 1024; }
+// shared memory holds fewer CTAs anyway.  Packed pairs take aligned register
+// pairs: at 1280 threads (48 registers) the 64-record kernels spill 4 to 40
+// bytes.  Measured at 16x8 / 64, 1280 / 1152 / 1024: one launch on 1M Betas x
+// 16 x 1080p 3.44 / 3.43 / 3.59 ms, backward on 6M x 8 x 4K 20.66 / 20.28 /
+// 21.00 ms.
+constexpr int pair_threads_per_sm(int S) { return S <= 64 ? 1152 : 1024; }
 
 // Do TW x TH tiles hold whole pixel-pair blocks (16 x 4 in tiles at least
 // 16 wide, 8 x 8 in 8-wide ones)?  Those use the pixel-pair kernels, the
@@ -710,23 +724,59 @@ __device__ __forceinline__ uint32_t pair_cover(float4 f0, float4 f1, float bxf, 
   return m;
 }
 
-// r^2 of a staged record at the lane's two pixel centres (xf, yf) and
-// (xf + 1, yf), with their whitened coordinates: each pixel's the values
-// rec_r2 gives it (the row term q1 dy is shared), so that every pixel
-// composites the same way whatever the tiling, and the forward and the
-// backward see the same values.
-__device__ __forceinline__ void rec_r2_pair(float4 f0, float4 f1, float xf, float yf, float& u0, float& v0,
-                                            float& u1, float& v1, float& r2a, float& r2b) {
-  const float dx0 = (xf - f0.x) + f0.z;
-  const float dx1 = ((xf + 1.0f) - f0.x) + f0.z;
+// Two floats in one 64-bit register (the lane's two pixels: lo = pixel 0) and
+// the packed fp32 instructions of sm_100+: one issue slot for both pixels, each
+// half rounded to nearest as the scalar instruction rounds it.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 both2(float x) { return pack2(x, x); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return lo + hi;
+}
+
+// 1 - r^2 of a staged record at the lane's two pixel centres, x2 = (xf, xf + 1)
+// in row yf, with their whitened coordinates: each pixel's the values rec_r2
+// gives it (the row term q1 dy is shared), so that every pixel composites the
+// same way whatever the tiling, and the forward and the backward see the same
+// values.  r^2 < 1 exactly where 1 - r^2 > 0 (the difference is at least 2^-24
+// there; NaN is neither).
+__device__ __forceinline__ f32x2 rec_om_pair(float4 f0, float4 f1, f32x2 x2, float yf, f32x2& u, f32x2& v) {
+  const f32x2 dx = add2(add2(x2, both2(-f0.x)), both2(f0.z));
   const float dy = (yf - f0.y) + f0.w;
-  const float qy = f1.y * dy;
-  u0 = f1.x * dx0;
-  v0 = fmaf(f1.z, dx0, qy);
-  u1 = f1.x * dx1;
-  v1 = fmaf(f1.z, dx1, qy);
-  r2a = fmaf(u0, u0, v0 * v0);
-  r2b = fmaf(u1, u1, v1 * v1);
+  u = mul2(both2(f1.x), dx);
+  v = fma2(both2(f1.z), dx, both2(f1.y * dy));
+  const f32x2 r2 = fma2(u, u, mul2(v, v));
+  return fma2(r2, both2(-1.0f), both2(1.0f));
+}
+
+// Is a record's colour free of infinities and NaN?  (A finite sum that
+// overflows reads as not finite, which only costs the slower path.)
+__device__ __forceinline__ bool finite_colour(float4 f2) {
+  return fabsf((f2.y + f2.z) + f2.w) < __int_as_float(0x7f800000);
 }
 
 // Per-lane state of the pixel-pair forward after a tile's walk: transmittance,
@@ -736,6 +786,7 @@ struct PairFwdState {
   float T0, T1, C00, C01, C02, C10, C11, C12;
   uint32_t last0, last1;
   int walked_batch, walked_buf;   // the last batch the walk composited and its s_rec buffer (-1: none)
+  bool odd_colours;               // a record the warp walked has a non-finite colour (warp-uniform)
 };
 
 // Forward walk of one tile's list [start, end) at the lane's pixel pair (xf,
@@ -775,15 +826,19 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
   }
   cp_async_commit();
 
-  float T0 = 1.0f, T1 = 1.0f, C00 = 0.0f, C01 = 0.0f, C02 = 0.0f, C10 = 0.0f, C11 = 0.0f, C12 = 0.0f;
+  // a pixel composites while T >= t_eps (>= 0); an off-image one starts below it
+  f32x2 T2 = pack2(in0 ? 1.0f : -1.0f, in1 ? 1.0f : -1.0f);
+  f32x2 Cr = 0ull, Cg = 0ull, Cb = 0ull;
+  const f32x2 x2 = pack2(xf, xf + 1.0f), one2 = both2(1.0f), neg2 = both2(-1.0f);
   uint32_t last0 = 0, last1 = 0;
-  bool done0 = !in0, done1 = !in1;
-  bool warp_done = __all_sync(0xffffffffu, done0 && done1);
+  bool done = !in0 && !in1;   // both pixels
+  bool warp_done = __all_sync(0xffffffffu, done);
+  bool odd_any = false;
 
   int buf = 0, batch = 0, walked_batch = -1, walked_buf = -1;
   for (uint32_t base = start; base < end; base += S, ++batch) {
     cp_async_wait_all();
-    if (!__syncthreads_or(!(done0 && done1))) break;
+    if (!__syncthreads_or(!done)) break;
     const uint32_t nb = base + S;
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
@@ -803,9 +858,15 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
       // pass 1: lane k finds the pairs of this warp's block that record
       // c + k may cover; the transpose gives every lane its records
       const int idx = c + lane;
-      const uint32_t cov =
-          idx < cnt ? pair_cover<PB::BW>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf) : 0u;
+uint32_t cov = 0u;
+      bool odd = false;
+      if (idx < cnt) {
+        cov = pair_cover<PB::BW>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf);
+        odd = !finite_colour(s_rec[buf][idx][2]);
+      }
       uint32_t mine = transpose32(cov, lane);
+      odd = __any_sync(0xffffffffu, odd);
+      odd_any = odd_any || odd;
       const int jc = (int)((base - start + c) >> 5);
       if (hslot && jc < hm_chunks) {
         uint32_t* slot = hslot + (size_t)jc * (NT + NW);
@@ -813,60 +874,75 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         slot[tid] = mine;
         if (lane == 0) slot[NT + warp] = wide;
       }
-      if (done0 && done1) mine = 0u;
-      // pass 2: every lane composites its records in list order at both
-      // of its pixels
+      if (done) mine = 0u;
+      // pass 2: every lane composites its records in list order at both of
+      // its pixels in packed arithmetic; a pixel that the record does not
+      // cover, or that is done, takes alpha = 0, which leaves T and C as they
+      // are (colours are finite, or `odd` selects)
       while (mine) {
         const int k = __ffs(mine) - 1;
         mine &= mine - 1;
         const int s = c + k;
         const float4 f0 = s_rec[buf][s][0];
         const float4 f1 = s_rec[buf][s][1];
-        float u0, v0, u1, v1, r2a, r2b;
-        rec_r2_pair(f0, f1, xf, yf, u0, v0, u1, v1, r2a, r2b);
-        const bool h0 = !done0 && r2a < 1.0f, h1 = !done1 && r2b < 1.0f;
-        if (!(h0 || h1)) continue;                    // outside the support (the cover is conservative)
         const float4 f2 = s_rec[buf][s][2];
+        f32x2 u, v;
+        const f32x2 om = rec_om_pair(f0, f1, x2, yf, u, v);
+        float om0, om1, T0, T1, e0, e1;
+        unpack2(om, om0, om1);
+        unpack2(T2, T0, T1);
+        const bool h0 = om0 > 0.0f && T0 >= t_eps, h1 = om1 > 0.0f && T1 >= t_eps;
+        unpack2(fma2(both2(f1.w), pack2(lg2_approx(om0), lg2_approx(om1)), both2(f2.x)), e0, e1);
+        const float a0 = h0 ? fminf(ex2_approx(e0), amax) : 0.0f;
+        const float a1 = h1 ? fminf(ex2_approx(e1), amax) : 0.0f;
+        const f32x2 a2 = pack2(a0, a1);
+        const f32x2 w2 = mul2(a2, T2);
+        if (!odd) {
+          Cr = fma2(w2, both2(f2.y), Cr);
+          Cg = fma2(w2, both2(f2.z), Cg);
+          Cb = fma2(w2, both2(f2.w), Cb);
+        } else {
+          float w0, w1, r0, r1, g0, g1, b0, b1;
+          unpack2(w2, w0, w1);
+          unpack2(Cr, r0, r1);
+          unpack2(Cg, g0, g1);
+          unpack2(Cb, b0, b1);
+          if (h0) {
+            r0 = fmaf(w0, f2.y, r0);
+            g0 = fmaf(w0, f2.z, g0);
+            b0 = fmaf(w0, f2.w, b0);
+          }
+          if (h1) {
+            r1 = fmaf(w1, f2.y, r1);
+            g1 = fmaf(w1, f2.z, g1);
+            b1 = fmaf(w1, f2.w, b1);
+          }
+          Cr = pack2(r0, r1);
+          Cg = pack2(g0, g1);
+          Cb = pack2(b0, b1);
+        }
+        T2 = mul2(T2, fma2(a2, neg2, one2));
         const uint32_t pos = base - start + (uint32_t)s + 1u;
-        if (h0) {
-          const float a = fminf(ex2_approx(fmaf(f1.w, lg2_approx(1.0f - r2a), f2.x)), amax);
-          const float w = a * T0;
-          C00 = fmaf(w, f2.y, C00);
-          C01 = fmaf(w, f2.z, C01);
-          C02 = fmaf(w, f2.w, C02);
-          T0 = T0 * (1.0f - a);
-          last0 = pos;
-          done0 = T0 < t_eps;
-        }
-        if (h1) {
-          const float a = fminf(ex2_approx(fmaf(f1.w, lg2_approx(1.0f - r2b), f2.x)), amax);
-          const float w = a * T1;
-          C10 = fmaf(w, f2.y, C10);
-          C11 = fmaf(w, f2.z, C11);
-          C12 = fmaf(w, f2.w, C12);
-          T1 = T1 * (1.0f - a);
-          last1 = pos;
-          done1 = T1 < t_eps;
-        }
-        if (done0 && done1) mine = 0u;
+        if (h0) last0 = pos;
+        if (h1) last1 = pos;
+        unpack2(T2, T0, T1);
+        done = T0 < t_eps && T1 < t_eps;
+        if (done) mine = 0u;
       }
-      warp_done = __all_sync(0xffffffffu, done0 && done1);
+      warp_done = __all_sync(0xffffffffu, done);
     }
     buf ^= 1;
   }
   cp_async_wait_all();   // no copy may still land in a buffer the next tile fills
-  st.T0 = T0;
-  st.T1 = T1;
-  st.C00 = C00;
-  st.C01 = C01;
-  st.C02 = C02;
-  st.C10 = C10;
-  st.C11 = C11;
-  st.C12 = C12;
+  unpack2(T2, st.T0, st.T1);
+  unpack2(Cr, st.C00, st.C10);
+  unpack2(Cg, st.C01, st.C11);
+  unpack2(Cb, st.C02, st.C12);
   st.last0 = last0;
   st.last1 = last1;
   st.walked_batch = walked_batch;
   st.walked_buf = walked_buf;
+  st.odd_colours = odd_any;
 }
 
 // Epilogue of the pixel-pair forward at pixels (x, y), (x + 1, y) of view v:
@@ -985,31 +1061,54 @@ __global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_thre
   leave<PERSIST>(ctr);
 }
 
-// One pixel's terms (bwd_terms with ZERO) from its whitened coordinates,
-// added to G when ADD.
-template <bool ADD>
-__device__ __forceinline__ bool pix_terms(float u, float vv, float r2, float4 f1, float4 f2, float amax, bool act,
-                                          float gx, float gy, float gz, float& T, float& GS, float G[kGrad2d]) {
-  act = act && r2 < 1.0f;
-  const float beta = f1.w;
-  const float base = fmaxf(1.0f - r2, 5.9604645e-8f);   // 1 - r^2 >= 2^-24 wherever r^2 < 1
-  const float lb = lg2_approx(base);
-  const float a0 = ex2_approx(fmaf(beta, lb, f2.x));   // the forward's alpha
-  const float a = fminf(a0, amax);
-  const float inv = rcp_approx(1.0f - a);
-  const float Tk = T * inv;
-  const float gc = fmaf(gx, f2.y, fmaf(gy, f2.z, gz * f2.w));
-  const float dLa = fmaf(Tk, gc, -GS * inv);
-  const float wgt = act ? a * Tk : 0.0f;
-  const float t = (a0 < amax && act) ? dLa * a0 : 0.0f;   // clamped alpha: no o/beta/r^2 gradient
-  const float kk = t * rcp_approx(base);
-  const float g0 = kk * u, g1 = kk * vv;
-  const float H[kGrad2d] = {g0, g1, g0 * u, g0 * vv, g1 * vv, t, t * lb, wgt * gx, wgt * gy, wgt * gz};
-#pragma unroll
-  for (int q = 0; q < kGrad2d; ++q) G[q] = ADD ? G[q] + H[q] : H[q];
-  GS = act ? fmaf(wgt, gc, GS) : GS;
-  T = act ? Tk : T;
-  return act;
+// The lane's two pixels' terms (bwd_terms with ZERO) of a staged record, summed
+// over the two into G; T2 and NG2 (the suffix colour term g . S, negated) move
+// on at the pixels where `pos` holds and the record covers the pixel.  There
+// alpha takes its value, elsewhere zero, so that 1 / (1 - alpha) = 1 leaves T
+// and a zero weight leaves NG2 and the colour terms (with a non-finite colour,
+// `odd`, g . c is dropped there).  Returns whether either pixel is covered.
+__device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x2 x2, float yf, float amax, bool odd,
+                                           bool pos0, bool pos1, f32x2 gx, f32x2 gy, f32x2 gz, f32x2& T2, f32x2& NG2,
+                                           float G[kGrad2d]) {
+  f32x2 u, v;
+  const f32x2 om = rec_om_pair(f0, f1, x2, yf, u, v);
+  float b0, b1, e0, e1, d0, d1, t0, t1;
+  unpack2(om, b0, b1);
+  const bool act0 = pos0 && b0 > 0.0f, act1 = pos1 && b1 > 0.0f;
+  b0 = fmaxf(b0, 5.9604645e-8f);   // 1 - r^2 >= 2^-24 wherever r^2 < 1
+  b1 = fmaxf(b1, 5.9604645e-8f);
+  const f32x2 lb = pack2(lg2_approx(b0), lg2_approx(b1));
+  unpack2(fma2(both2(f1.w), lb, both2(f2.x)), e0, e1);
+  const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);   // the forward's alpha
+  const f32x2 a2 = pack2(act0 ? fminf(p0, amax) : 0.0f, act1 ? fminf(p1, amax) : 0.0f);
+  unpack2(fma2(a2, both2(-1.0f), both2(1.0f)), d0, d1);
+  const f32x2 inv = pack2(rcp_approx(d0), rcp_approx(d1));
+  f32x2 gc = fma2(gx, both2(f2.y), fma2(gy, both2(f2.z), mul2(gz, both2(f2.w))));
+  if (odd) {
+    float c0, c1;
+    unpack2(gc, c0, c1);
+    gc = pack2(act0 ? c0 : 0.0f, act1 ? c1 : 0.0f);
+  }
+  const f32x2 dLa = mul2(fma2(T2, gc, NG2), inv);
+  T2 = mul2(T2, inv);
+  const f32x2 wgt = mul2(a2, T2);
+  unpack2(mul2(dLa, pack2(p0, p1)), t0, t1);
+  const f32x2 t = pack2(act0 && p0 < amax ? t0 : 0.0f,    // clamped alpha: no o/beta/r^2 gradient
+                        act1 && p1 < amax ? t1 : 0.0f);
+  const f32x2 kk = mul2(t, pack2(rcp_approx(b0), rcp_approx(b1)));
+  const f32x2 h0 = mul2(kk, u), h1 = mul2(kk, v);
+  G[0] = sum2(h0);
+  G[1] = sum2(h1);
+  G[2] = sum2(mul2(h0, u));
+  G[3] = sum2(mul2(h0, v));
+  G[4] = sum2(mul2(h1, v));
+  G[5] = sum2(t);
+  G[6] = sum2(mul2(t, lb));
+  G[7] = sum2(mul2(wgt, gx));
+  G[8] = sum2(mul2(wgt, gy));
+  G[9] = sum2(mul2(wgt, gz));
+  NG2 = fma2(mul2(wgt, both2(-1.0f)), gc, NG2);
+  return act0 || act1;
 }
 
 // Per-lane state the pixel-pair backward starts from: final transmittance,
@@ -1018,6 +1117,7 @@ __device__ __forceinline__ bool pix_terms(float u, float vv, float r2, float4 f1
 struct PairBwdState {
   float T0, T1, GS0, GS1, g0x, g0y, g0z, g1x, g1y, g1z;
   uint32_t nl0, nl1;
+  int odd_colours;   // 1 / 0: some / none of the records has a non-finite colour; -1: not known
 };
 
 // Reverse walk of one tile's list lst at the lane's pixel pair, from the CTA's
@@ -1043,8 +1143,9 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
   using PB = PairBlock<TW>;
   constexpr int NT = TW * TH / 2, NW = NT / 32, RPT = (S + NT - 1) / NT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float T0 = st.T0, T1 = st.T1, GS0 = st.GS0, GS1 = st.GS1;
-  const float g0x = st.g0x, g0y = st.g0y, g0z = st.g0z, g1x = st.g1x, g1y = st.g1y, g1z = st.g1z;
+  f32x2 T2 = pack2(st.T0, st.T1), NG2 = pack2(-st.GS0, -st.GS1);
+  const f32x2 gx = pack2(st.g0x, st.g1x), gy = pack2(st.g0y, st.g1y), gz = pack2(st.g0z, st.g1z);
+  const f32x2 x2 = pack2(xf, xf + 1.0f);
   const uint32_t nl0 = st.nl0, nl1 = st.nl1;
   const uint32_t nlm = max(nl0, nl1);
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, nlm);
@@ -1128,6 +1229,8 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         pf_wide = nslot[NT + warp];
         pf_chunk = j - 1;
       }
+      bool odd = st.odd_colours > 0;
+      if (st.odd_colours < 0) odd = __any_sync(0xffffffffu, c + lane < cnt && !finite_colour(s_rec[buf][c + lane][2]));
       const int lim = (int)nlm - (lo + c);           // only positions before a pixel's last contributor
       mine &= lim >= 32 ? 0xffffffffu : (lim <= 0 ? 0u : (1u << lim) - 1u);
       // pass 2, in reverse list order: between wide records every lane walks
@@ -1144,17 +1247,14 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
           seg &= ~(1u << k);
           const int s = c + k;
           const uint32_t pos = (uint32_t)(lo + s);
-          const float4 f0 = s_rec[buf][s][0], f1 = s_rec[buf][s][1], f2 = s_rec[buf][s][2];
-          float u0, v0, u1, v1, r2a, r2b;
-          rec_r2_pair(f0, f1, xf, yf, u0, v0, u1, v1, r2a, r2b);
           float G[kGrad2d];
-          const bool a0 = pix_terms<false>(u0, v0, r2a, f1, f2, amax, pos < nl0, g0x, g0y, g0z, T0, GS0, G);
-          const bool a1 = pix_terms<true>(u1, v1, r2b, f1, f2, amax, pos < nl1, g1x, g1y, g1z, T1, GS1, G);
-          if (!(a0 || a1)) continue;                  // outside the support (the cover is conservative)
+          if (!pair_terms(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, pos < nl0, pos < nl1,
+                          gx, gy, gz, T2, NG2, G))
+            continue;                                 // outside the support (the cover is conservative)
           float* gdst = grad2d + (size_t)s_ridx[buf][s] * kGrad2dStride;
           red_add_v4(gdst + 0, G[0], G[1], G[2], G[3]);
           red_add_v4(gdst + 4, G[4], G[5], G[6], G[7]);
-          red_add_v4(gdst + 8, G[8], G[9], 0.0f, 0.0f);
+          red_add_v2(gdst + 8, G[8], G[9]);
         }
         if (kb < 0) break;
         wide &= ~(1u << kb);
@@ -1162,12 +1262,9 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         mine &= ~(1u << kb);
         const int s = c + kb;
         const uint32_t pos = (uint32_t)(lo + s);
-        const float4 f0 = s_rec[buf][s][0], f1 = s_rec[buf][s][1], f2 = s_rec[buf][s][2];
-        float u0, v0, u1, v1, r2a, r2b;
-        rec_r2_pair(f0, f1, xf, yf, u0, v0, u1, v1, r2a, r2b);
         float G[kGrad2d];                              // zero where a pixel is not covered
-        pix_terms<false>(u0, v0, r2a, f1, f2, amax, mine_kb && pos < nl0, g0x, g0y, g0z, T0, GS0, G);
-        pix_terms<true>(u1, v1, r2b, f1, f2, amax, mine_kb && pos < nl1, g1x, g1y, g1z, T1, GS1, G);
+        pair_terms(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, mine_kb && pos < nl0,
+                   mine_kb && pos < nl1, gx, gy, gz, T2, NG2, G);
         const float tot = warp_sum10(G, lane);
         float* gdst = grad2d + (size_t)s_ridx[buf][s] * kGrad2dStride;
         if (my_field >= 0 && tot != 0.0f) atomicAdd(gdst + my_field, tot);
@@ -1209,7 +1306,7 @@ __global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_thre
     const uint32_t range0 = ranges[g];
     const uint32_t* const hslot = hit_tile<NT>(const_cast<uint32_t*>(hm), hm_words, range0, ranges[g + 1], g);
 
-    PairBwdState bs{1.0f, 1.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0u, 0u};
+    PairBwdState bs{1.0f, 1.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0u, 0u, -1};
     {
       const int64_t HW = (int64_t)W * H;
       const int64_t pix = vt.v[v].pix_off + (int64_t)y * W + x;
@@ -1316,6 +1413,7 @@ __global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_thre
     bs.g1z = gv[5];
     bs.nl0 = fs.last0;
     bs.nl1 = fs.last1;
+    bs.odd_colours = fs.odd_colours ? 1 : 0;
     bs.GS0 = in0 ? bs.T0 * (bs.g0x * bg[0] + bs.g0y * bg[1] + bs.g0z * bg[2]) : 0.0f;
     bs.GS1 = in1 ? bs.T1 * (bs.g1x * bg[0] + bs.g1y * bg[1] + bs.g1z * bg[2]) : 0.0f;
     pair_bwd_walk<TW, TH, S>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,

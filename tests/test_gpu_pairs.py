@@ -1,0 +1,63 @@
+"""The packed pixel-pair raster kernels against the one-pixel kernels (8x4
+tiles) where packed arithmetic could differ: a record with an infinite colour
+must leave the pixels it does not cover, its pair's other pixel among them,
+exactly as they are, in images and gradients."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2501_18630_gb300 import _lib, render, scenes
+from tests import gpu_common as gc
+
+pytestmark = pytest.mark.gpu
+
+
+def _scene(odd):
+    rng = np.random.Generator(np.random.PCG64(11))
+    planes = scenes.random_scene(60, 1, rng, mean_lo=-0.6, mean_hi=0.6, logscale=(-2.6, 0.5))
+    if odd:
+        k = int(np.argsort(planes[2, :60])[20])       # some Betas in front of it, some behind
+        planes[12, k] = 3e38                           # base colour + lobe colour overflow
+        planes[15 + 2, k] = -20.0                      # lobe exponent ~ 0: weight 1 where it faces the view
+        planes[18, k] = 3e38
+        planes[15, k], planes[16, k] = np.pi / 2, 0.0
+        d = planes[0:3, k] - np.array([0.0, 0.0, -3.0])
+        planes[15, k], planes[16, k] = np.arccos(d[2] / np.linalg.norm(d)), np.arctan2(d[1], d[0])
+    return planes
+
+
+def _run(planes_np, cam, tile, s, fused):
+    gc.ensure_built()
+    planes = torch.from_numpy(planes_np).cuda()
+    opts = _lib.default_opts(tile_w=tile[0], tile_h=tile[1], batch_s=s)
+    r = render.Rasterizer(60, planes.shape[1], 1, [cam], opts)
+    target = torch.from_numpy(scenes.target_images([cam], seed=3)[0].reshape(-1)).cuda()
+    r.forward(planes)
+    grad = torch.zeros_like(planes)
+    if fused:
+        r.raster_fwd_bwd_l1(planes, target)
+    else:
+        r.raster_fwd_l1(planes, target)
+        r.raster_bwd(planes, r.dL_dcolor)
+    r.project_bwd(planes, grad)
+    torch.cuda.synchronize()
+    return r.color.cpu().numpy(), grad.cpu().numpy()
+
+
+@pytest.mark.parametrize("odd", [False, True])
+@pytest.mark.parametrize("tile,s,fused", [((8, 8), 64, False), ((16, 8), 64, True), ((16, 16), 128, False),
+                                          ((16, 16), 256, True), ((32, 16), 64, True)])
+@pytest.mark.parametrize("w,h", [(37, 29), (64, 48)])
+def test_pair_kernels_equal_one_pixel_kernels(odd, tile, s, fused, w, h):
+    cam = scenes.pinhole(*scenes.look_at((0.0, 0.0, -3.0)), w, h)
+    planes = _scene(odd)
+    c0, g0 = _run(planes, cam, (8, 4), 64, False)
+    c1, g1 = _run(planes, cam, tile, s, fused)
+    assert np.isfinite(c0).all() != odd and (not odd or np.isfinite(c0).mean() > 0.2)
+    np.testing.assert_array_equal(c1, c0)              # NaN and infinities in the same places too
+    fin = np.isfinite(g0)
+    assert (np.isfinite(g1) == fin).all() and fin.any()
+    # fp32 terms summed in another order: 60 Betas on a few thousand pixels,
+    # each sum off by at most ~sqrt(terms) roundings of its largest partial sums
+    scale = np.max(np.abs(np.where(fin, g0, 0.0)), axis=1, keepdims=True) + 1e-30
+    assert np.max(np.abs(np.where(fin, g1 - g0, 0.0)) / scale) < 1e-4
