@@ -14,13 +14,22 @@
 //   b = 2 dS/dG*x^2 = -2 S / B2,   c = dS/dG*xy = 2 A1 d
 //   dL/dx = (1 - lambda) sign(x - y) / N - lambda / N (G*a + x G*b + y G*c).
 //
-// k_ssim_stats: one CTA per 32 x 32 pixel tile of one channel: x and y over
-//   the tile and a 5-pixel halo in shared memory, the
-//   horizontal and vertical 11-tap passes with each thread sliding a register
-//   window over 4 outputs (one shared-memory load per input instead of one per
-//   tap), then S, (a, b, c) to the workspace and the tile's sums of S and
-//   |x - y| as per-block partials.
-// k_ssim_grad:  the same tiling over (a, b, c): blur them and form dL/dx.
+// sigma_x^2 and sigma_y^2 enter S and its derivatives only as their sum, which is
+// 2 sigma_xy + Var(x - y), so four quantities are filtered: (x, y) and
+// ((x - y)^2, x y), two packed pairs.  With D = Var(x - y) and d = mu_x - mu_y,
+//   A1 = 2 mu_x mu_y + C1, A2 = 2 sigma_xy + C2, B1 = A1 + d^2, B2 = A2 + D,
+// so that S = (A1 / B1)(A2 / B2) loses least where the images are alike (error of
+// dL/dx against 64 bits on images 0.08 apart: 2.3e-6, from the five moments
+// 3.1e-6; on unrelated ones 1.1e-7 both).
+//
+// k_ssim_stats: one CTA per 32 x 54 pixel tile of one channel: x and y over the
+//   tile and a 5-pixel halo in shared memory, the horizontal pass (a thread
+//   slides a register window over 8 outputs of one of the 64 halo rows: 256
+//   threads are 64 rows x 4 runs), its results over the same shared memory, the
+//   vertical pass (a thread owns 7 outputs of one column), then S, (a, b, c) to
+//   the workspace and the tile's sum of S as a per-block partial.
+// k_ssim_grad:  the same tiling over (a, b, c): blur them, form dL/dx, and the
+//   tile's sum of |x - y|.
 // k_ssim_loss:  per view, the sum of its blocks' partials (fixed order: the
 //   loss is deterministic) and the loss.
 // HBM traffic per channel-pixel: x, y read twice, (a, b, c) written and read
@@ -35,16 +44,22 @@ namespace beta {
 
 namespace {
 
-constexpr int kTX = 32, kTY = 32, kR = 5, kWin = 2 * kR + 1;
-constexpr int kRun = 4;   // outputs per thread in each filter pass (sliding register window)
+// 64 halo rows by 4 runs of 8 columns are the CTA's 256 threads in the
+// horizontal pass; 32 columns by 8 groups of 7 rows (the last of 5) in the
+// vertical one.
+constexpr int kTX = 32, kTY = 54, kR = 5, kWin = 2 * kR + 1;
 constexpr int kHX = kTX + 2 * kR, kHY = kTY + 2 * kR;
-// row stride of the staged halo tiles: 45 = 1 (mod 4), so the four rows a
-// warp reads in the horizontal pass (8 lanes each, 4 columns apart) fall in
-// distinct banks
-constexpr int kSX = 45;
-// row stride of the horizontal-pass results: 33, so the same pass's stores
-// (rows apart by one, 4 columns apart) fall in distinct banks
-constexpr int kSH = kTX + 1;
+constexpr int kThreads2 = 256;
+constexpr int kRunH = kHY * kTX / kThreads2;              // 8 outputs a thread, horizontal pass
+constexpr int kRunV = (kTY * kTX + kThreads2 - 1) / kThreads2;   // 7 outputs a thread, vertical pass
+static_assert(kHY == 64 && kTX == 32 && kRunH == 8 && kRunV * (kThreads2 / kTX) >= kTY, "thread mapping");
+// Row strides of the staged tile and of the horizontal results: odd, so that
+// lanes on consecutive rows (the horizontal pass) fall in distinct banks for
+// 4-, 8- and 16-byte accesses.
+constexpr int kSX = kHX + 1, kSH = kTX + 1;
+// rows the vertical pass reads: the last group's outputs past the tile, which
+// are dropped, read rows past the halo that nothing has written
+constexpr int kRowsV = (kThreads2 / kTX) * kRunV + 2 * kR;
 constexpr float kC1 = 1e-4f, kC2 = 9e-4f;
 
 // normalised Gaussian taps (sigma 1.5), computed by the host launcher and
@@ -91,238 +106,364 @@ __device__ __forceinline__ double block_sum_d(float x, double* s_w) {
   return t;
 }
 
-// Horizontal pass over a staged (kHY x kHX) tile: row r, columns c0 .. c0 +
-// kRun - 1 of the output, from a register window of kRun + 2 kR inputs.
-// PRODUCTS: the sources are x and y, and the five filtered quantities are
-// x, y, x^2, y^2, x y (formed in registers).
-template <int Q, bool PRODUCTS>
-__device__ __forceinline__ void hpass_run(const float (*src)[kHY][kSX], const SsimWin& win, int r, int c0,
-                                          float (&out)[Q][kRun]) {
+// Packed fp32 pairs (sm_100+): one instruction for two results, each rounded
+// as the scalar instruction rounds it.  The filters are bound by issue slots
+// and the FMA pipe, so every tap is a packed multiply-add.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 both2(float x) { return pack2(x, x); }
+
+// 1 / x to one unit in the last place
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Asynchronous 4-byte global -> shared copy.
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+  const size_t ga = __cvta_generic_to_global(gmem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(ga) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// tap k of the symmetric window (0 outside)
+__device__ __forceinline__ float tap(const SsimWin& w, int k) {
+  return k < 0 || k >= kWin ? 0.0f : w.g[k <= kR ? k : kWin - 1 - k];
+}
+
+// One input (t-th of a run's window) added to the run's N outputs: a packed
+// pair of quantities `ab`, and one further quantity `c` whose outputs are
+// packed by neighbours (2 q, 2 q + 1).
+template <int N>
+__device__ __forceinline__ void taps_pair(const SsimWin& w, int t, f32x2 ab, f32x2 (&out)[N]) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q)
+  for (int j = 0; j < N; ++j)
+    if (t - j >= 0 && t - j < kWin) out[j] = fma2(pack2(tap(w, t - j), tap(w, t - j)), ab, out[j]);
+}
+template <int N>
+__device__ __forceinline__ void taps_single(const SsimWin& w, int t, float c, f32x2 (&out)[(N + 1) / 2]) {
 #pragma unroll
-    for (int j = 0; j < kRun; ++j) out[q][j] = 0.0f;
-#pragma unroll
-  for (int t = 0; t < kRun + 2 * kR; ++t) {
-    float v[Q];
-    if (PRODUCTS) {
-      const float xv = src[0][r][c0 + t], yv = src[1][r][c0 + t];
-      v[0] = xv;
-      v[1] = yv;
-      v[2] = xv * xv;
-      v[3] = yv * yv;
-      v[4] = xv * yv;
-    } else {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) v[q] = src[q][r][c0 + t];
-    }
-#pragma unroll
-    for (int j = 0; j < kRun; ++j) {
-      const int k = t - j;                 // tap of input t for output j
-      if (k >= 0 && k < kWin) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) out[q][j] = fmaf(win.g[k], v[q], out[q][j]);
-      }
+  for (int q = 0; q < (N + 1) / 2; ++q) {
+    const int k = t - 2 * q;           // tap of the input for output 2 q, k - 1 for output 2 q + 1
+    if (k >= 1 && k < kWin) {
+      out[q] = fma2(pack2(tap(w, k), tap(w, k - 1)), pack2(c, c), out[q]);
+    } else if (k == 0 || k == kWin) {  // one of the two only: no 0 * c, c may be infinite
+      float lo, hi;
+      unpack2(out[q], lo, hi);
+      if (k == 0) lo = fmaf(tap(w, 0), c, lo);
+      else hi = fmaf(tap(w, kWin - 1), c, hi);
+      out[q] = pack2(lo, hi);
     }
   }
 }
 
-__global__ void __launch_bounds__(256) k_ssim_stats(ViewTable vt, SsimWin win, const float* __restrict__ color,
-                                                    const float* __restrict__ target,
-                                                    float* __restrict__ abc, int64_t plane,
-                                                    double* __restrict__ acc) {
-  __shared__ float s_in[2][kHY][kSX];     // x, y over the tile and its halo
-  __shared__ float s_h[5][kHY][kSH];      // their horizontal pass
+// Loads of the CTA's halo tile, kLoads per thread: load(i, shared index,
+// offset in the channel, in image).  Columns 0 .. 31: warp w takes rows w,
+// w + 8, ... (i < 8); columns 32 .. 41: 10 threads a row.
+constexpr int kRowLoads = kHY / (kThreads2 / 32);
+constexpr int kLoads = kRowLoads + ((kHX - 32) * kHY + kThreads2 - 1) / kThreads2;
+template <typename F>
+__device__ __forceinline__ void for_halo(const SsimBlock& B, F load) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gx0 = B.x0 - kR + lane;
+  const bool in0 = gx0 >= 0 && gx0 < B.W;
+  int64_t at = (int64_t)(B.y0 - kR + warp) * B.W + gx0;
+#pragma unroll
+  for (int i = 0; i < kRowLoads; ++i, at += 8 * (int64_t)B.W) {
+    const int r = warp + 8 * i, gy = B.y0 - kR + r;
+    load(i, r * kSX + lane, at, in0 && gy >= 0 && gy < B.H);
+  }
+#pragma unroll
+  for (int i = kRowLoads; i < kLoads; ++i) {
+    const int k = threadIdx.x + (i - kRowLoads) * kThreads2;
+    const int r = k / (kHX - 32), c = 32 + k - r * (kHX - 32);
+    const int gx = B.x0 - kR + c, gy = B.y0 - kR + r;
+    load(i, r < kHY ? r * kSX + c : -1, (int64_t)gy * B.W + gx, r < kHY && gx < B.W && gy >= 0 && gy < B.H);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads2, 4) k_ssim_stats(ViewTable vt, SsimWin win, const float* __restrict__ color,
+                                                             const float* __restrict__ target,
+                                                             float2* __restrict__ ab, float* __restrict__ cc,
+                                                             double* __restrict__ acc) {
+  // the staged (x, y), then the horizontal results (x, y, (x - y)^2, x y)
+  __shared__ __align__(16) float4 s_buf[kRowsV * kSH];
   __shared__ double s_w[8];
+  static_assert(sizeof(float2) * kHY * kSX <= sizeof(float4) * kHY * kSH, "staged tile exceeds the buffer");
   const SsimBlock B = ssim_block(vt, blockIdx.x);
   const int64_t HW = (int64_t)B.W * B.H;
   const int64_t base = 3 * vt.v[B.v].pix_off + B.ch * HW;
   const float* xs = color + base;
   const float* ys = target + base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   {
-    constexpr int kLd = (kHY * kHX + 255) / 256;
-    float lx[kLd], ly[kLd];
+    // all of a thread's halo loads are issued before its shared-memory stores
+    // (4-byte asynchronous copies instead took 9% more instructions)
+    float2* s_in = reinterpret_cast<float2*>(s_buf);
+    float2 v[kLoads];
+    int to[kLoads];
+    for_halo(B, [&](int i, int dst, int64_t at, bool in) {
+      to[i] = dst;
+      v[i] = in ? make_float2(xs[at], ys[at]) : make_float2(0.0f, 0.0f);
+    });
 #pragma unroll
-    for (int i = 0; i < kLd; ++i) {
-      const int k = threadIdx.x + i * 256;
-      const int r = k / kHX, c = k - r * kHX;
-      const int gy = B.y0 - kR + r, gx = B.x0 - kR + c;
-      const bool in = k < kHY * kHX && gx >= 0 && gx < B.W && gy >= 0 && gy < B.H;
-      lx[i] = in ? xs[(int64_t)gy * B.W + gx] : 0.0f;
-      ly[i] = in ? ys[(int64_t)gy * B.W + gx] : 0.0f;
+    for (int i = 0; i < kLoads; ++i)
+      if (i < kRowLoads || to[i] >= 0) s_in[to[i]] = v[i];
+  }
+  __syncthreads();
+  {
+    const int r = (warp & 1) * 32 + lane, c0 = (warp >> 1) * kRunH;
+    const f32x2* src = reinterpret_cast<const f32x2*>(s_buf) + r * kSX + c0;
+    f32x2 hm[kRunH], hs[kRunH];
+#pragma unroll
+    for (int j = 0; j < kRunH; ++j) hm[j] = hs[j] = 0ull;
+#pragma unroll
+    for (int t = 0; t < kRunH + 2 * kR; ++t) {
+      const f32x2 xy = src[t];
+      float x, y;
+      unpack2(xy, x, y);
+      const float dif = x - y;
+      taps_pair<kRunH>(win, t, xy, hm);
+      taps_pair<kRunH>(win, t, pack2(dif * dif, x * y), hs);
     }
+    __syncthreads();   // every thread has read its window: the results replace the staged tile
 #pragma unroll
-    for (int i = 0; i < kLd; ++i) {
-      const int k = threadIdx.x + i * 256;
-      if (k < kHY * kHX) {
-        const int r = k / kHX, c = k - r * kHX;
-        s_in[0][r][c] = lx[i];
-        s_in[1][r][c] = ly[i];
-      }
+    for (int j = 0; j < kRunH; ++j) {
+      float4 h;
+      unpack2(hm[j], h.x, h.y);
+      unpack2(hs[j], h.z, h.w);
+      s_buf[r * kSH + c0 + j] = h;
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < kHY * (kTX / kRun); k += blockDim.x) {
-    const int r = k / (kTX / kRun), c0 = (k - r * (kTX / kRun)) * kRun;
-    float h[5][kRun];
-    hpass_run<5, true>(s_in, win, r, c0, h);
-#pragma unroll
-    for (int q = 0; q < 5; ++q)
-#pragma unroll
-      for (int j = 0; j < kRun; ++j) s_h[q][r][c0 + j] = h[q][j];
-  }
-  __syncthreads();
-  // vertical pass: column c, rows r0 .. r0 + kRun - 1 from a register window
-  // per-thread sums of 4 values in fp32 (GB300's FP64 rate is a small fraction
+  // per-thread sums of 7 values in fp32 (GB300's FP64 rate is a small fraction
   // of FP32); the block and view sums are FP64
-  float sum_s = 0.0f, sum_l1 = 0.0f;
+  float sum_s = 0.0f;
   {
-    const int c = threadIdx.x % kTX, r0 = (threadIdx.x / kTX) * kRun;
-    float m[5][kRun];
+    const int r0 = warp * kRunV;
+    f32x2 m[kRunV], q[kRunV];
 #pragma unroll
-    for (int q = 0; q < 5; ++q)
+    for (int j = 0; j < kRunV; ++j) m[j] = q[j] = 0ull;
 #pragma unroll
-      for (int j = 0; j < kRun; ++j) m[q][j] = 0.0f;
-#pragma unroll
-    for (int t = 0; t < kRun + 2 * kR; ++t) {
-      float v[5];
-#pragma unroll
-      for (int q = 0; q < 5; ++q) v[q] = s_h[q][r0 + t][c];
-#pragma unroll
-      for (int j = 0; j < kRun; ++j) {
-        const int k = t - j;
-        if (k >= 0 && k < kWin) {
-#pragma unroll
-          for (int q = 0; q < 5; ++q) m[q][j] = fmaf(win.g[k], v[q], m[q][j]);
-        }
-      }
+    for (int t = 0; t < kRunV + 2 * kR; ++t) {
+      const float4 h = s_buf[(r0 + t) * kSH + lane];
+      taps_pair<kRunV>(win, t, pack2(h.x, h.y), m);
+      taps_pair<kRunV>(win, t, pack2(h.z, h.w), q);
     }
-    const int gx = B.x0 + c;
+    // S and its partials of outputs j and j + 1, packed
+    const int gx = B.x0 + lane;
+    const int rows = gx < B.W ? min(min(kRunV, kTY - r0), B.H - B.y0 - r0) : 0;   // outputs inside tile and image
+    const int64_t at0 = base + (int64_t)(B.y0 + r0) * B.W + gx;
+    float2* abp = ab + at0;
+    float* ccp = cc + at0;
+    const f32x2 two = both2(2.0f), neg = both2(-1.0f);
 #pragma unroll
-    for (int j = 0; j < kRun; ++j) {
-      const int gy = B.y0 + r0 + j;
-      if (gx >= B.W || gy >= B.H) continue;
-      const float mx = m[0][j], my = m[1][j];
-      const float sxx = m[2][j] - mx * mx, syy = m[3][j] - my * my, sxy = m[4][j] - mx * my;
-      const float A1 = 2.0f * mx * my + kC1, A2 = 2.0f * sxy + kC2;
-      const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
-      const float iB1 = __frcp_rn(B1), iB2 = __frcp_rn(B2);
-      const float d = iB1 * iB2;
-      const float S = A1 * A2 * d;
-      const float a = 2.0f * my * A2 * d - 2.0f * mx * S * iB1 + 2.0f * mx * S * iB2 - 2.0f * my * A1 * d;
-      const int64_t at = base + (int64_t)gy * B.W + gx;
-      abc[at] = a;
-      abc[plane + at] = -2.0f * S * iB2;
-      abc[2 * plane + at] = 2.0f * A1 * d;
-      sum_s += S;
-      sum_l1 += fabsf(s_in[0][r0 + j + kR][c + kR] - s_in[1][r0 + j + kR][c + kR]);
+    for (int j = 0; j < kRunV; j += 2) {
+      constexpr int last = kRunV - 1;
+      const int k = j < last ? j + 1 : j;
+      float x0, y0, x1, y1, s0, p0, s1, p1;
+      unpack2(m[j], x0, y0);
+      unpack2(m[k], x1, y1);
+      unpack2(q[j], s0, p0);
+      unpack2(q[k], s1, p1);
+      const f32x2 mx = pack2(x0, x1), my = pack2(y0, y1);
+      const f32x2 md = fma2(my, neg, mx), nmd = fma2(mx, neg, my);
+      const f32x2 A1 = fma2(two, mul2(mx, my), both2(kC1)), B1 = fma2(md, md, A1);
+      const f32x2 A2 = fma2(two, fma2(mul2(mx, neg), my, pack2(p0, p1)), both2(kC2));
+      const f32x2 B2 = add2(A2, fma2(nmd, md, pack2(s0, s1)));
+      float b10, b11, b20, b21;
+      unpack2(B1, b10, b11);
+      unpack2(B2, b20, b21);
+      const f32x2 iB1 = pack2(rcp_approx(b10), rcp_approx(b11)), iB2 = pack2(rcp_approx(b20), rcp_approx(b21));
+      const f32x2 A1d = mul2(A1, mul2(iB1, iB2)), S = mul2(A2, A1d);
+      // a = 2 my d (A2 - A1) + 2 mx S (1 / B2 - 1 / B1),  b = -2 S / B2,  c = 2 A1 d
+      const f32x2 d = mul2(iB1, iB2);
+      const f32x2 a = mul2(two, fma2(mul2(my, d), fma2(A1, neg, A2), mul2(mul2(mx, S), fma2(iB1, neg, iB2))));
+      const f32x2 b = mul2(mul2(both2(-2.0f), S), iB2), c = mul2(two, A1d);
+      float a0, a1, b0, b1, c0, c1, S0, S1;
+      unpack2(a, a0, a1);
+      unpack2(b, b0, b1);
+      unpack2(c, c0, c1);
+      unpack2(S, S0, S1);
+      if (j < rows) {
+        abp[(int64_t)j * B.W] = make_float2(a0, b0);
+        ccp[(int64_t)j * B.W] = c0;
+        sum_s += S0;
+      }
+      if (j < last && k < rows) {
+        abp[(int64_t)k * B.W] = make_float2(a1, b1);
+        ccp[(int64_t)k * B.W] = c1;
+        sum_s += S1;
+      }
     }
   }
   const double ts = block_sum_d(sum_s, s_w);
-  __syncthreads();
-  const double tl = block_sum_d(sum_l1, s_w);
-  if (threadIdx.x == 0) {   // per-block partial sums, reduced per view by k_ssim_loss
-    acc[2 * blockIdx.x] = ts;
-    acc[2 * blockIdx.x + 1] = tl;
-  }
+  if (threadIdx.x == 0) acc[2 * blockIdx.x] = ts;   // per-block partial sums, reduced per view by k_ssim_loss
 }
 
-__global__ void __launch_bounds__(256) k_ssim_grad(ViewTable vt, SsimWin win, const float* __restrict__ color,
-                                                   const float* __restrict__ target,
-                                                   const float* __restrict__ abc, int64_t plane, float lambda,
-                                                   float* __restrict__ dLdC) {
-  __shared__ float s_m[3][kHY][kSX];
-  __shared__ float s_h[3][kHY][kSH];
+__global__ void __launch_bounds__(kThreads2, 4) k_ssim_grad(ViewTable vt, SsimWin win, const float* __restrict__ color,
+                                                            const float* __restrict__ target,
+                                                            const float2* __restrict__ ab, const float* __restrict__ cc,
+                                                            float lambda, float* __restrict__ dLdC,
+                                                            double* __restrict__ acc) {
+  // the staged (a, b) and c, then their horizontal pass
+  __shared__ __align__(16) float2 s_ab[kHY * kSX];
+  __shared__ float s_c[kHY * kSX];
+  __shared__ float s_xy[2][kRunV][kThreads2];   // x, y at the thread's outputs, copied in while it filters
+  __shared__ double s_w[8];
+  static_assert(kRowsV * kSH <= kHY * kSX, "horizontal results exceed the buffer");
   const SsimBlock B = ssim_block(vt, blockIdx.x);
   const int64_t HW = (int64_t)B.W * B.H;
   const int64_t base = 3 * vt.v[B.v].pix_off + B.ch * HW;
-  // all of a thread's halo loads are issued before any store (memory-level
-  // parallelism: the loads are the kernel's latency)
-  constexpr int kLd = (kHY * kHX + 255) / 256;
-  float ld[kLd][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gx = B.x0 + lane, r0 = warp * kRunV;
+  const int rows = gx < B.W ? min(min(kRunV, kTY - r0), B.H - B.y0 - r0) : 0;   // outputs inside tile and image
+  const int64_t at0 = base + (int64_t)(B.y0 + r0) * B.W + gx;
+  {
+    const float2* as = ab + base;
+    const float* cs = cc + base;
+    float2 v[kLoads];
+    float w[kLoads];
+    int to[kLoads];
+    for_halo(B, [&](int i, int dst, int64_t at, bool in) {
+      to[i] = dst;
+      v[i] = in ? as[at] : make_float2(0.0f, 0.0f);
+      w[i] = in ? cs[at] : 0.0f;
+    });
 #pragma unroll
-  for (int i = 0; i < kLd; ++i) {
-    const int k = threadIdx.x + i * 256;
-    const int r = k / kHX, c = k - r * kHX;
-    const int gy = B.y0 - kR + r, gx = B.x0 - kR + c;
-    const bool in = k < kHY * kHX && gx >= 0 && gx < B.W && gy >= 0 && gy < B.H;
-    const int64_t at = base + (int64_t)gy * B.W + gx;
+    for (int j = 0; j < kRunV; ++j)
+      if (j < rows) {
+        cp_async4(&s_xy[0][j][threadIdx.x], color + at0 + (int64_t)j * B.W);
+        cp_async4(&s_xy[1][j][threadIdx.x], target + at0 + (int64_t)j * B.W);
+      }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) ld[i][q] = in ? abc[q * plane + at] : 0.0f;
-  }
-#pragma unroll
-  for (int i = 0; i < kLd; ++i) {
-    const int k = threadIdx.x + i * 256;
-    if (k < kHY * kHX) {
-      const int r = k / kHX, c = k - r * kHX;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) s_m[q][r][c] = ld[i][q];
-    }
+    for (int i = 0; i < kLoads; ++i)
+      if (i < kRowLoads || to[i] >= 0) {
+        s_ab[to[i]] = v[i];
+        s_c[to[i]] = w[i];
+      }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < kHY * (kTX / kRun); k += blockDim.x) {
-    const int r = k / (kTX / kRun), c0 = (k - r * (kTX / kRun)) * kRun;
-    float h[3][kRun];
-    hpass_run<3, false>(s_m, win, r, c0, h);
+  {
+    const int r = (warp & 1) * 32 + lane, c0 = (warp >> 1) * kRunH;
+    const f32x2* src = reinterpret_cast<const f32x2*>(s_ab) + r * kSX + c0;
+    const float* srcc = s_c + r * kSX + c0;
+    f32x2 h[kRunH], hc[kRunH / 2];
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
+    for (int j = 0; j < kRunH; ++j) h[j] = 0ull;
 #pragma unroll
-      for (int j = 0; j < kRun; ++j) s_h[q][r][c0 + j] = h[q][j];
+    for (int j = 0; j < kRunH / 2; ++j) hc[j] = 0ull;
+#pragma unroll
+    for (int t = 0; t < kRunH + 2 * kR; ++t) {
+      taps_pair<kRunH>(win, t, src[t], h);
+      taps_single<kRunH>(win, t, srcc[t], hc);
+    }
+    __syncthreads();   // every thread has read its window: the results replace the staged tile
+#pragma unroll
+    for (int j = 0; j < kRunH; ++j) reinterpret_cast<f32x2*>(s_ab)[r * kSH + c0 + j] = h[j];
+#pragma unroll
+    for (int j = 0; j < kRunH / 2; ++j) {
+      float lo, hi;
+      unpack2(hc[j], lo, hi);
+      s_c[r * kSH + c0 + 2 * j] = lo;
+      s_c[r * kSH + c0 + 2 * j + 1] = hi;
+    }
   }
   __syncthreads();
   const float inv_n = 1.0f / (3.0f * (float)HW);
-  const int c = threadIdx.x % kTX, r0 = (threadIdx.x / kTX) * kRun;
-  float m[3][kRun];
+  f32x2 m[kRunV], mc[(kRunV + 1) / 2];
 #pragma unroll
-  for (int q = 0; q < 3; ++q)
+  for (int j = 0; j < kRunV; ++j) m[j] = 0ull;
 #pragma unroll
-    for (int j = 0; j < kRun; ++j) m[q][j] = 0.0f;
+  for (int j = 0; j < (kRunV + 1) / 2; ++j) mc[j] = 0ull;
 #pragma unroll
-  for (int t = 0; t < kRun + 2 * kR; ++t) {
-    float v[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) v[q] = s_h[q][r0 + t][c];
-#pragma unroll
-    for (int j = 0; j < kRun; ++j) {
-      const int k = t - j;
-      if (k >= 0 && k < kWin) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) m[q][j] = fmaf(win.g[k], v[q], m[q][j]);
-      }
-    }
+  for (int t = 0; t < kRunV + 2 * kR; ++t) {
+    const int at = (r0 + t) * kSH + lane;
+    taps_pair<kRunV>(win, t, reinterpret_cast<const f32x2*>(s_ab)[at], m);
+    taps_single<kRunV>(win, t, s_c[at], mc);
   }
-  const int gx = B.x0 + c;
+  cp_async_wait_all();   // x, y: the thread reads its own copies only
+  float sum_l1 = 0.0f;
 #pragma unroll
-  for (int j = 0; j < kRun; ++j) {
-    const int gy = B.y0 + r0 + j;
-    if (gx >= B.W || gy >= B.H) continue;
-    const int64_t at = base + (int64_t)gy * B.W + gx;
-    const float xv = color[at], yv = target[at];
+  for (int j = 0; j < kRunV; ++j) {
+    if (j >= rows) continue;
+    const float xv = s_xy[0][j][threadIdx.x], yv = s_xy[1][j][threadIdx.x];
     const float dif = xv - yv;
     const float sgn = dif > 0.0f ? 1.0f : (dif < 0.0f ? -1.0f : 0.0f);
-    const float dS = m[0][j] + xv * m[1][j] + yv * m[2][j];
-    dLdC[at] = inv_n * ((1.0f - lambda) * sgn - lambda * dS);
+    float ga, gb, c0, c1;
+    unpack2(m[j], ga, gb);
+    unpack2(mc[j / 2], c0, c1);
+    const float dS = ga + xv * gb + yv * (j % 2 ? c1 : c0);
+    dLdC[at0 + (int64_t)j * B.W] = inv_n * ((1.0f - lambda) * sgn - lambda * dS);
+    sum_l1 += fabsf(dif);
   }
+  const double tl = block_sum_d(sum_l1, s_w);
+  if (threadIdx.x == 0) acc[2 * blockIdx.x + 1] = tl;
 }
 
 // per view: the sums of its blocks' partials (fixed order), then the loss
-__global__ void __launch_bounds__(256) k_ssim_loss(ViewTable vt, const double* __restrict__ acc, int nb,
+__global__ void __launch_bounds__(512) k_ssim_loss(ViewTable vt, const double* __restrict__ acc, int nb,
                                                    float lambda, float* __restrict__ loss) {
   const int v = blockIdx.x;
   const int b0 = vt.v[v].pad0, b1 = v + 1 < vt.n_views ? vt.v[v + 1].pad0 : nb;
   double ss = 0.0, sl = 0.0;
-  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-    ss += acc[2 * b];
-    sl += acc[2 * b + 1];
+  constexpr int kAhead = 4;   // loads in flight
+  for (int64_t c = b0; c < b1; c += kAhead * 512) {
+    double2 x[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      const int64_t b = c + q * 512 + threadIdx.x;
+      x[q] = b < b1 ? *reinterpret_cast<const double2*>(acc + 2 * b) : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q)
+      if (c + q * 512 < b1) {
+        ss += x[q].x;
+        sl += x[q].y;
+      }
   }
-  // one CTA per view: FP64 throughout (a few thousand values)
-  __shared__ double s_a[256], s_b[256];
-  s_a[threadIdx.x] = ss;
-  s_b[threadIdx.x] = sl;
+  // one CTA per view, FP64 throughout (a few thousand values): warp sums by
+  // shuffles, then the warps' sums in order (256 values added by one thread
+  // were 27 us of a training iteration's 430)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    sl += __shfl_xor_sync(0xffffffffu, sl, o);
+  }
+  __shared__ double s_a[32], s_b[32];
+  if ((threadIdx.x & 31) == 0) {
+    s_a[threadIdx.x >> 5] = ss;
+    s_b[threadIdx.x >> 5] = sl;
+  }
   __syncthreads();
   double ts = 0.0, tl = 0.0;
   if (threadIdx.x == 0)
-    for (int t = 0; t < (int)blockDim.x; ++t) {
+    for (int t = 0; t < (int)(blockDim.x >> 5); ++t) {
       ts += s_a[t];
       tl += s_b[t];
     }
@@ -366,11 +507,12 @@ cudaError_t launch_ssim_loss(const ViewTable& vt_in, const float* color, const f
   const int nb = ssim_blocks(vt);
   if (nb <= 0) return cudaSuccess;
   const int64_t plane = 3 * vt.total_pixels;
-  float* abc = (float*)ws;
+  float2* ab = (float2*)ws;                 // (a, b) of every value, then c
+  float* cc = (float*)ws + 2 * plane;
   double* acc = (double*)((char*)ws + ((size_t)9 * vt.total_pixels * sizeof(float) + 255) / 256 * 256);
-  k_ssim_stats<<<nb, 256, 0, s>>>(vt, win, color, target, abc, plane, acc);
-  k_ssim_grad<<<nb, 256, 0, s>>>(vt, win, color, target, abc, plane, lambda, dL_dcolor);
-  k_ssim_loss<<<vt.n_views, 256, 0, s>>>(vt, acc, nb, lambda, loss);
+  k_ssim_stats<<<nb, kThreads2, 0, s>>>(vt, win, color, target, ab, cc, acc);
+  k_ssim_grad<<<nb, kThreads2, 0, s>>>(vt, win, color, target, ab, cc, lambda, dL_dcolor, acc);
+  k_ssim_loss<<<vt.n_views, 512, 0, s>>>(vt, acc, nb, lambda, loss);
   return cudaGetLastError();
 }
 
