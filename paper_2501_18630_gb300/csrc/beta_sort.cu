@@ -15,12 +15,12 @@
 //   3. k_tile_scatter: every record appends the 64-bit item
 //                      (depth key << 32 | record) to each of its tiles' lists,
 //                      slots taken with atomics (arbitrary order inside a list);
-//   4. k_tile_sort:    each list is sorted by its items (a register sorting
-//                      network per thread, then a shuffle bitonic network
-//                      across the warp, or merge-path merges in shared memory
-//                      for 16 items a lane and for CTA sorts), one warp per
-//                      list up to kWarpMax items, one CTA per longer list, and
-//                      the record ids are written out.
+//   4. k_tile_sort:    each list is sorted by its items, one warp per list up
+//                      to kWarpMax items (a shuffle bitonic network over
+//                      32-bit words that stand for the items, checked and put
+//                      right against the items), one CTA per longer list
+//                      (warp-sorted runs, then merge-path merges in shared
+//                      memory), and the record ids are written out.
 // The items of a list are distinct (the record index is part of them), so the
 // sorted list does not depend on the order the atomics gave: it is the order
 // (tile, depth key, record index), a stable sort of the pairs by depth in
@@ -43,12 +43,12 @@ typedef unsigned long long u64;
 
 constexpr int kSortThreads = 256;
 constexpr int kScanItems = 8;
-constexpr int kScanTile = kSortThreads * kScanItems;   // tiles per scan block
-static_assert(kScanItems == 8, "the scan moves a thread's tiles as two 16-byte vectors");
+constexpr int kScanTile = kSortThreads * kScanItems;   // tiles per scan block of the largest scan (k_tile_scan<8>)
 constexpr int kWarpMax = 512;                      // longest list one warp sorts (16 items a lane)
 constexpr int kCtaItems = 16;
 constexpr int kCtaMax = kSortThreads * kCtaItems;      // longest list sorted in one shared-memory pass
-constexpr int kTicketLists = 4;                    // short lists per warp ticket
+constexpr int kTicketLists = 4;                    // short lists per warp ticket, at most
+constexpr int kSortCtasPerSM = 3;
 constexpr int kSub = 16;                           // counters per tile (record index mod kSub): spreads
                                                    // the atomics on a busy tile over kSub addresses
 constexpr int kSpinLimit = 1 << 20;
@@ -210,11 +210,45 @@ __device__ __forceinline__ u64 block_excl_scan(u64 x, u64* s_w, u64& total) {
   return pre + inc - x;
 }
 
+// ITEMS consecutive words (1, 2, 4 or 8, aligned to their size or 16 bytes)
+template <int ITEMS>
+__device__ __forceinline__ void load_tiles(const uint32_t* p, uint32_t (&x)[ITEMS]) {
+  if constexpr (ITEMS == 1) {
+    x[0] = *p;
+  } else if constexpr (ITEMS == 2) {
+    const uint2 a = *reinterpret_cast<const uint2*>(p);
+    x[0] = a.x; x[1] = a.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < ITEMS; k += 4) {
+      const uint4 a = *reinterpret_cast<const uint4*>(p + k);
+      x[k] = a.x; x[k + 1] = a.y; x[k + 2] = a.z; x[k + 3] = a.w;
+    }
+  }
+}
+template <int ITEMS>
+__device__ __forceinline__ void store_tiles(uint32_t* p, const uint32_t (&x)[ITEMS]) {
+  if constexpr (ITEMS == 1) {
+    *p = x[0];
+  } else if constexpr (ITEMS == 2) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(x[0], x[1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < ITEMS; k += 4)
+      *reinterpret_cast<uint4*>(p + k) = make_uint4(x[k], x[k + 1], x[k + 2], x[k + 3]);
+  }
+}
+
 // 2. exclusive scan of the tile counters: each CTA takes the next block of
-// kScanTile tiles from a ticket, reduces it, chains its offset to the
-// preceding blocks by decoupled look-back (warp 0 inspects 32 predecessors
+// kSortThreads x ITEMS tiles from a ticket, reduces it, chains its offset to
+// the preceding blocks by decoupled look-back (warp 0 inspects 32 predecessors
 // at a time; bounded waits) and writes ranges and cursors.  The last block
 // writes ranges[total_tiles] and the pair count and flags a capacity overflow.
+// ITEMS is the fewest tiles a thread (1, 2, 4 or 8) whose look-back entries
+// fit in the workspace's: a single 1080p view has 8160 tiles, four CTAs of
+// 2048, whose 32 dependent rounds of loads took 13-15 us; as 32 CTAs of 256
+// it is one round per CTA.
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __restrict__ cnt, int total_tiles,
                                                         u64* look, uint32_t* counters,
                                                         uint32_t* __restrict__ ranges,
@@ -222,6 +256,7 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __re
                                                         uint32_t* __restrict__ longl, int64_t cap,
                                                         int64_t* d_count, int32_t* status,
                                                         int spin_limit, int64_t withhold) {
+  constexpr int kTile = kSortThreads * ITEMS;
   __shared__ u64 s_w[kSortThreads / 32];
   __shared__ u64 s_base;
   __shared__ uint32_t s_blk;
@@ -229,34 +264,39 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __re
   if (threadIdx.x == 0) s_blk = atomicAdd(&counters[0], 1u);
   __syncthreads();
   const int64_t blk = s_blk;
-  const int64_t nb = cdiv(total_tiles, kScanTile);
+  const int64_t nb = cdiv(total_tiles, kTile);
   if (blk >= nb) return;
-  const int64_t base = blk * kScanTile + threadIdx.x * kScanItems;
-  // the thread's kScanItems tiles: per class two 16-byte loads (rows are
-  // padded to a multiple of kScanItems and zeroed, so no tail guard)
+  const int64_t base = blk * kTile + threadIdx.x * ITEMS;
+  // the thread's tiles: per class one load of ITEMS words (two 16-byte ones
+  // for 8; rows are padded to a multiple of kScanItems and zeroed, so no tail guard)
   const int64_t row = crow(total_tiles);
   const bool mine = base < total_tiles;
-  uint32_t c[kScanItems];
+  uint32_t c[ITEMS], part[ITEMS <= 2 ? kSub : 1][ITEMS <= 2 ? ITEMS : 1];
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) c[k] = 0u;
-  if (mine)
-#pragma unroll 4
+  for (int k = 0; k < ITEMS; ++k) c[k] = 0u;
+  if (mine) {
+#pragma unroll(ITEMS <= 2 ? kSub : 4)
     for (int q = 0; q < kSub; ++q) {
-      const uint4* src = reinterpret_cast<const uint4*>(cnt + q * row + base);
-      const uint4 a = src[0], b = src[1];
-      c[0] += a.x; c[1] += a.y; c[2] += a.z; c[3] += a.w;
-      c[4] += b.x; c[5] += b.y; c[6] += b.z; c[7] += b.w;
+      uint32_t x[ITEMS];
+      load_tiles<ITEMS>(cnt + q * row + base, x);
+#pragma unroll
+      for (int k = 0; k < ITEMS; ++k) {
+        c[k] += x[k];
+        if constexpr (ITEMS <= 2) part[q][k] = x[k];
+      }
     }
+  }
   u64 sum = 0;
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) sum += c[k];
+  for (int k = 0; k < ITEMS; ++k) sum += c[k];
   u64 total;
   const u64 excl = block_excl_scan(sum, s_w, total);
   if (warp == 0) {
     u64 prefix = 0;
-    // `withhold` (a test hook, -1 normally) names a block that never posts
-    // its look-back entry, so that its successors' bounded waits run out
-    const bool post = blk != withhold;
+    // `withhold` (a test hook, -1 normally; in units of kScanTile tiles) names
+    // blocks that never post their look-back entries, so that their
+    // successors' bounded waits run out
+    const bool post = blk * kTile / kScanTile != withhold;
     if (blk == 0) {
       if (lane == 0 && post) atomicExch(&look[0], kInc | total);
     } else {
@@ -301,9 +341,9 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __re
   __syncthreads();
   u64 run = s_base + excl;
   if (!mine) return;
-  uint32_t start[kScanItems];
+  uint32_t start[ITEMS];
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
+  for (int k = 0; k < ITEMS; ++k) {
     const int64_t g = base + k;
     start[k] = (uint32_t)run;
     if (g < total_tiles) {
@@ -313,15 +353,18 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __re
     run += c[k];
   }
   // class q's part of a list starts after classes 0 .. q-1
-#pragma unroll 4
+#pragma unroll(ITEMS <= 2 ? kSub : 4)
   for (int q = 0; q < kSub; ++q) {
-    const uint4* src = reinterpret_cast<const uint4*>(cnt + q * row + base);
-    uint4* dst = reinterpret_cast<uint4*>(cursor + q * row + base);
-    const uint4 a = src[0], b = src[1];
-    dst[0] = make_uint4(start[0], start[1], start[2], start[3]);
-    dst[1] = make_uint4(start[4], start[5], start[6], start[7]);
-    start[0] += a.x; start[1] += a.y; start[2] += a.z; start[3] += a.w;
-    start[4] += b.x; start[5] += b.y; start[6] += b.z; start[7] += b.w;
+    uint32_t x[ITEMS];
+    if constexpr (ITEMS <= 2) {
+#pragma unroll
+      for (int k = 0; k < ITEMS; ++k) x[k] = part[q][k];
+    } else {
+      load_tiles<ITEMS>(cnt + q * row + base, x);
+    }
+    store_tiles<ITEMS>(cursor + q * row + base, start);
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) start[k] += x[k];
   }
 }
 
@@ -391,8 +434,8 @@ __device__ __forceinline__ void group_sync() {
 }
 
 // Ascending bitonic sorting network over a thread's E registers.
-template <int E>
-__device__ __forceinline__ void sort_regs(u64 (&k)[E]) {
+template <int E, typename K>
+__device__ __forceinline__ void sort_regs(K (&k)[E]) {
 #pragma unroll
   for (int size = 2; size <= E; size <<= 1)
 #pragma unroll
@@ -402,7 +445,7 @@ __device__ __forceinline__ void sort_regs(u64 (&k)[E]) {
         const int j = i ^ stride;
         if (j > i) {
           const bool up = (i & size) == 0;
-          const u64 a = k[i], b = k[j];
+          const K a = k[i], b = k[j];
           const bool sw = up ? (a > b) : (a < b);
           k[i] = sw ? b : a;
           k[j] = sw ? a : b;
@@ -410,15 +453,15 @@ __device__ __forceinline__ void sort_regs(u64 (&k)[E]) {
       }
 }
 
-// Merge sort across a group of G threads, each holding a sorted run of E
-// items: at every level thread t produces outputs t*E .. t*E+E-1 of the
+// Merges across a group of G threads, thread t holding items t*E .. t*E+E-1 of
+// sorted runs of RUN0 items: at every level thread t produces outputs t*E .. t*E+E-1 of the
 // merge of two neighbouring runs, starting where the merge path crosses its
 // first output (binary search), ties to the left run.  `sm` holds G*E items
 // (padded by sidx).
-template <int G, int E>
+template <int G, int E, int RUN0>
 __device__ __forceinline__ void group_merge(u64 (&k)[E], u64* sm, int t) {
 #pragma unroll 1
-  for (int run = E; run < G * E; run <<= 1) {
+  for (int run = RUN0; run < G * E; run <<= 1) {
 #pragma unroll
     for (int j = 0; j < E; ++j) sm[sidx(t * E + j)] = k[j];
     group_sync<G>();
@@ -454,13 +497,13 @@ __device__ __forceinline__ void group_merge(u64 (&k)[E], u64* sm, int t) {
 // with lane ^ (stride / E) through shuffles and strides < E are
 // compare-exchanges inside the lane; a run's direction is bit log2(size) of
 // its first item.  No shared memory and no dependent loads.
-template <int E>
-__device__ __forceinline__ void warp_bitonic(u64 (&k)[E], int lane) {
+template <int E, typename K>
+__device__ __forceinline__ void warp_bitonic(K (&k)[E], int lane) {
   // lane runs must alternate ascending / descending for the first merge
   if (lane & 1) {
 #pragma unroll
     for (int j = 0; j < E / 2; ++j) {
-      const u64 t = k[j];
+      const K t = k[j];
       k[j] = k[E - 1 - j];
       k[E - 1 - j] = t;
     }
@@ -474,7 +517,7 @@ __device__ __forceinline__ void warp_bitonic(u64 (&k)[E], int lane) {
       const bool take_min = ((lane & lm) == 0) == up;
 #pragma unroll
       for (int j = 0; j < E; ++j) {
-        const u64 o = __shfl_xor_sync(0xffffffffu, k[j], lm);
+        const K o = __shfl_xor_sync(0xffffffffu, k[j], lm);
         k[j] = (take_min == (o < k[j])) ? o : k[j];
       }
     }
@@ -484,7 +527,7 @@ __device__ __forceinline__ void warp_bitonic(u64 (&k)[E], int lane) {
       for (int j = 0; j < E; ++j) {
         const int jj = j ^ stride;
         if (jj > j) {
-          const u64 a = k[j], b = k[jj];
+          const K a = k[j], b = k[jj];
           const bool sw = up ? (a > b) : (a < b);
           k[j] = sw ? b : a;
           k[jj] = sw ? a : b;
@@ -493,48 +536,103 @@ __device__ __forceinline__ void warp_bitonic(u64 (&k)[E], int lane) {
   }
 }
 
-// Sorts list items[0, n) (n <= 32 E) with one warp and writes the record ids:
-// E <= 8 by the shuffle network, E = 16 by merge-path merges in shared memory.
+// Are the warp's items (lane L: items L E .. L E + E - 1) in ascending order?
+template <int E>
+__device__ __forceinline__ bool warp_sorted(const u64 (&k)[E], int lane) {
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j + 1 < E; ++j) ok = ok && k[j] <= k[j + 1];
+  const u64 prev = __shfl_up_sync(0xffffffffu, k[E - 1], 1);
+  return __all_sync(0xffffffffu, ok && (lane == 0 || prev <= k[0]));
+}
+
+// Sorts 32 E items at sm[sidx(s0 + 0 .. 32 E - 1)] (pads, kPad, last) with one
+// warp; on return lane L holds items L E .. L E + E - 1 of the order.
+// The network runs on 32-bit words instead of the 64-bit items: the item's
+// depth key minus the list's least, shifted right until it fits above the
+// item's position in the list.  A compare-exchange is then a third of the
+// 64-bit one (1156 instructions a list before, at 98 items on average).  The
+// items are gathered by position and checked: keys that the shift (or the
+// scene) made equal can be out of order, and a few odd-even passes over
+// neighbours put such pairs right; if that is not enough the items are sorted
+// outright.
+template <int E>
+__device__ __forceinline__ void warp_sort_items(u64 (&k)[E], const u64* sm, int s0, int lane) {
+  constexpr int kPosBits = 5 + (E >= 2) + (E >= 4) + (E >= 8) + (E >= 16);
+  static_assert(32 * E == 1 << kPosBits, "positions fill their bits");
+  uint32_t c[E], lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const u64 it = sm[sidx(s0 + j * 32 + lane)];
+    c[j] = (uint32_t)(it >> 32);             // 0xffffffff for a pad, below 2^31 otherwise
+    lo = min(lo, c[j]);
+    hi = max(hi, c[j] == 0xffffffffu ? 0u : c[j]);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  const int shift = hi > lo ? max(0, kPosBits - __clz(hi - lo)) : 0;
+#pragma unroll
+  for (int j = 0; j < E; ++j)
+    c[j] = c[j] == 0xffffffffu ? c[j] : ((c[j] - lo) >> shift) << kPosBits | (uint32_t)(j * 32 + lane);
+  sort_regs<E>(c);
+  warp_bitonic<E>(c, lane);
+  // a pad's word has all position bits set: the last position, itself a pad
+#pragma unroll
+  for (int j = 0; j < E; ++j) k[j] = sm[sidx(s0 + (int)(c[j] & (32 * E - 1)))];
+  if (warp_sorted<E>(k, lane)) return;
+  if (E >= 2) {
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+#pragma unroll
+      for (int odd = 0; odd < 2; ++odd)
+#pragma unroll
+        for (int j = odd; j + 1 < E; j += 2) {
+          const u64 a = k[j], b = k[j + 1];
+          k[j] = a < b ? a : b;
+          k[j + 1] = a < b ? b : a;
+        }
+      // a lane's last item against the next lane's first
+      const u64 next = __shfl_down_sync(0xffffffffu, k[0], 1), prev = __shfl_up_sync(0xffffffffu, k[E - 1], 1);
+      if (lane < 31 && next < k[E - 1]) k[E - 1] = next;
+      if (lane > 0 && k[0] < prev) k[0] = prev;
+      if (warp_sorted<E>(k, lane)) return;
+    }
+  }
+  sort_regs<E>(k);
+  warp_bitonic<E>(k, lane);
+}
+
+// Sorts list items[0, n) (n <= 32 E) with one warp and writes the record ids.
 template <int E>
 __device__ __forceinline__ void warp_list_sort(const u64* items, int n, uint32_t* __restrict__ out,
                                                u64* sm, int lane) {
   u64 k[E];
-  if (E <= 8) {
 #pragma unroll
-    for (int j = 0; j < E; ++j) {
-      const int p = lane * E + j;
-      k[j] = p < n ? items[p] : kPad;
-    }
-    sort_regs<E>(k);
-    warp_bitonic<E>(k, lane);
-  } else {
-    for (int p = lane; p < 32 * E; p += 32) sm[sidx(p)] = p < n ? items[p] : kPad;
-    __syncwarp();
+  for (int j = 0; j < E; ++j) k[j] = j * 32 + lane < n ? items[j * 32 + lane] : kPad;
 #pragma unroll
-    for (int j = 0; j < E; ++j) k[j] = sm[sidx(lane * E + j)];
-    __syncwarp();
-    sort_regs<E>(k);
-    group_merge<32, E>(k, sm, lane);
-  }
-#pragma unroll
-  for (int j = 0; j < E; ++j) sm[sidx(lane * E + j)] = k[j];
+  for (int j = 0; j < E; ++j) sm[sidx(j * 32 + lane)] = k[j];
   __syncwarp();
-  for (int p = lane; p < n; p += 32) out[p] = (uint32_t)sm[sidx(p)];
+  warp_sort_items<E>(k, sm, 0, lane);
+  __syncwarp();
+  uint32_t* ids = reinterpret_cast<uint32_t*>(sm);   // sidx: E words a lane apart without bank conflicts
+#pragma unroll
+  for (int j = 0; j < E; ++j) ids[sidx(lane * E + j)] = (uint32_t)k[j];
+  __syncwarp();
+  for (int p = lane; p < n; p += 32) out[p] = ids[sidx(p)];
   __syncwarp();
 }
 
 // Sorts up to kSortThreads * E items of `src` (m of them) with the whole
-// CTA; the sorted items are left in sm[sidx(0 .. m-1)].
+// CTA: each warp sorts a run of 32 E, then the runs are merged; the sorted
+// items are left in sm[sidx(0 .. m-1)].
 template <int E>
 __device__ __forceinline__ void cta_chunk_sort(const u64* src, int m, u64* sm, int tid) {
   for (int p = tid; p < kSortThreads * E; p += kSortThreads) sm[sidx(p)] = p < m ? src[p] : kPad;
   __syncthreads();
   u64 k[E];
-#pragma unroll
-  for (int j = 0; j < E; ++j) k[j] = sm[sidx(tid * E + j)];
+  warp_sort_items<E>(k, sm, (tid >> 5) * 32 * E, tid & 31);
   __syncthreads();
-  sort_regs<E>(k);
-  group_merge<kSortThreads, E>(k, sm, tid);
+  group_merge<kSortThreads, E, 32 * E>(k, sm, tid);
 #pragma unroll
   for (int j = 0; j < E; ++j) sm[sidx(tid * E + j)] = k[j];
   __syncthreads();
@@ -602,13 +700,16 @@ __device__ void cta_list_sort(u64* items, u64* tmp, uint32_t n, uint32_t* __rest
 }
 
 // 4. per-list sort.  Long lists first (one CTA each, from a ticket), then
-// short lists (one warp each, kTicketLists tiles per ticket).
-__global__ void __launch_bounds__(kSortThreads, 3) k_tile_sort(const uint32_t* __restrict__ ranges,
+// short lists (one warp each, ticket_lists tiles per ticket: kTicketLists, or
+// fewer where there are not that many lists for every warp, so that a single
+// view's lists spread over all of them).
+__global__ void __launch_bounds__(kSortThreads, kSortCtasPerSM) k_tile_sort(const uint32_t* __restrict__ ranges,
                                                            int total_tiles,
                                                            const uint32_t* __restrict__ longl,
                                                            uint32_t* counters, u64* items, u64* tmp,
                                                            uint32_t* __restrict__ vals,
-                                                           const int32_t* __restrict__ status) {
+                                                           const int32_t* __restrict__ status,
+                                                           int ticket_lists) {
   constexpr int kWarpSm = kWarpMax + kWarpMax / 16;
   __shared__ u64 sm[kCtaMax + kCtaMax / 16];
   __shared__ uint32_t s_t;
@@ -629,10 +730,10 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_tile_sort(const uint32_t* _
   u64* wsm = sm + warp * kWarpSm;
   for (;;) {
     uint32_t t0 = 0;
-    if (lane == 0) t0 = atomicAdd(&counters[2], (uint32_t)kTicketLists);
+    if (lane == 0) t0 = atomicAdd(&counters[2], (uint32_t)ticket_lists);
     t0 = __shfl_sync(0xffffffffu, t0, 0);
     if (t0 >= (uint32_t)total_tiles) break;
-    for (int q = 0; q < kTicketLists; ++q) {
+    for (int q = 0; q < ticket_lists; ++q) {
       const int g = (int)t0 + q;
       if (g >= total_tiles) break;
       const uint32_t s = ranges[g];
@@ -679,16 +780,27 @@ cudaError_t launch_bin_sort(const ViewTable& vt, int pitch, ProjBuffers pb, uint
   const int64_t grid_p = std::min<int64_t>(cdiv(std::max<int64_t>((int64_t)kSub * crow(total_tiles), nb_scan), kSortThreads), 1024);
   const int64_t grid_r = std::max<int64_t>(1, std::min<int64_t>(cdiv(n_items, kSortThreads), 1 << 20));
 
-  k_sort_prep<<<(unsigned)std::max<int64_t>(grid_p, 1), kSortThreads, 0, s>>>(w.cnt, total_tiles, w.look, nb_scan,
+  k_sort_prep<<<(unsigned)std::max<int64_t>(grid_p, 1), kSortThreads, 0, s>>>(w.cnt, total_tiles, w.look,
+                                                                          (int64_t)(align256((size_t)nb_scan * 8) / 8),
                                                                           w.counters, d_count, d_status);
   k_tile_count<<<(unsigned)grid_r, kSortThreads, 0, s>>>(pb.rect, pb.tiles, n_items, pitch, vt, total_tiles, w.cnt);
-  k_tile_scan<<<(unsigned)nb_scan, kSortThreads, 0, s>>>(w.cnt, total_tiles, w.look, w.counters, ranges, w.cursor,
-                                                     w.longl, cap, d_count, d_status, g_spin_limit.load(),
-                                                     g_withhold.load());
+  // look-back entries the workspace holds (its pieces are 256-byte aligned)
+  const int64_t entries = (int64_t)(align256((size_t)nb_scan * 8) / 8);
+  auto scan = [&](auto kernel, int items) {
+    kernel<<<(unsigned)cdiv(total_tiles, kSortThreads * items), kSortThreads, 0, s>>>(
+        w.cnt, total_tiles, w.look, w.counters, ranges, w.cursor, w.longl, cap, d_count, d_status,
+        g_spin_limit.load(), g_withhold.load());
+  };
+  if (cdiv(total_tiles, kSortThreads) <= entries) scan(k_tile_scan<1>, 1);
+  else if (cdiv(total_tiles, kSortThreads * 2) <= entries) scan(k_tile_scan<2>, 2);
+  else if (cdiv(total_tiles, kSortThreads * 4) <= entries) scan(k_tile_scan<4>, 4);
+  else scan(k_tile_scan<kScanItems>, kScanItems);
   k_tile_scatter<<<(unsigned)grid_r, kSortThreads, 0, s>>>(pb.rect, pb.tiles, pb.key, n_items, pitch, vt, total_tiles,
                                                        w.cursor, w.items, cap, d_status);
-  k_tile_sort<<<(unsigned)(device_sm_count() * 3), kSortThreads, 0, s>>>(ranges, total_tiles, w.longl, w.counters, w.items,
-                                                              w.tmp, pair_vals, d_status);
+  const int sort_grid = device_sm_count() * kSortCtasPerSM;
+  const int tickets = std::max(1, std::min(kTicketLists, total_tiles / (sort_grid * (kSortThreads / 32))));
+  k_tile_sort<<<(unsigned)sort_grid, kSortThreads, 0, s>>>(ranges, total_tiles, w.longl, w.counters, w.items, w.tmp,
+                                                           pair_vals, d_status, tickets);
   return cudaGetLastError();
 }
 
