@@ -222,12 +222,19 @@ cudaError_t launch_adam(int n_lobes, float* planes, const float* grad, float* m,
 // random word r of a dead primitive picks t = floor(r W_total / 2^32), the
 // source being the first i with W_i > t.
 //
-//   k_reloc_weights  weights (bit 31: dead) and per-block sums
-//   k_reloc_scan     exclusive scan of the block sums (one CTA)
-//   k_reloc_cdf      per-primitive inclusive prefix W
-//   k_reloc_sample   binary search per dead primitive, copy counts
-//   k_reloc_opacity  new opacity logit of every source
-//   k_reloc_copy     the copies (after the sources' new logits)
+//   k_reloc_weights  weights (bit 31: dead), old logits, zeroed copy counts,
+//                    per-block weight sums and dead counts
+//   k_reloc_scan     exclusive scan of the block sums, totals (one CTA)
+//   k_reloc_sample   a warp per dead primitive: its source (a 32-way search of
+//                    the block offsets, then the block's 256 weights), copy counts
+//   k_reloc_copy     the copies, kCopyPlanes planes of one primitive a thread,
+//                    and the new opacity logits of sources and copies (from the
+//                    old logits, so in any order)
+// Bound by scattered 4-byte reads and writes: 3% dead among 1M touch a fifth of
+// all 32-byte sectors of parameters and moments, 260 MB of DRAM traffic.  A
+// thread per dead primitive walking all 33 planes x 3 arrays took 92 us, a warp
+// per dead one (lane = plane) 113; one counter for the number of dead and a
+// binary search of 1M cumulative weights per dead thread took 38.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -252,32 +259,56 @@ __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long x
   return t;
 }
 
-__global__ void __launch_bounds__(256) k_reloc_weights(const float* __restrict__ planes, int n, int pitch,
-                                                       float min_opacity, uint32_t* __restrict__ w,
-                                                       unsigned long long* __restrict__ bsum) {
+constexpr int kRelocBlock = 256;   // primitives per block of weights
+
+__global__ void __launch_bounds__(kRelocBlock) k_reloc_weights(const float* __restrict__ planes, int n, int pitch,
+                                                               float min_opacity, uint32_t* __restrict__ w,
+                                                               uint32_t* __restrict__ copies,
+                                                               float* __restrict__ logit,
+                                                               unsigned long long* __restrict__ bsum,
+                                                               uint32_t* __restrict__ bdead) {
   __shared__ unsigned long long s_w[8];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t wi = 0;
   if (i < n) {
-    const float o = rule_opacity(planes[(size_t)10 * pitch + i]);
+    const float x = planes[(size_t)10 * pitch + i];
+    logit[i] = x;
+    const float o = rule_opacity(x);
     wi = o < min_opacity ? kDeadBit : (uint32_t)__fmul_rn(o, 16777216.0f);
     w[i] = wi;
+    copies[i] = 0u;
   }
+  const int dead = __syncthreads_count((wi & kDeadBit) != 0u);
   const unsigned long long t = block_sum_u64(wi & ~kDeadBit, s_w);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = t;
+  if (threadIdx.x == 0) {
+    bsum[blockIdx.x] = t;
+    bdead[blockIdx.x] = (uint32_t)dead;
+  }
 }
 
-__global__ void __launch_bounds__(1024) k_reloc_scan(unsigned long long* __restrict__ bsum, int nb,
-                                                     unsigned long long* __restrict__ total) {
+// Exclusive scan of the nb block sums in place, their total, and the number of
+// relocated primitives (the dead ones, if anything is live).  Four sums a
+// thread: 1M primitives are one round.
+__global__ void __launch_bounds__(1024) k_reloc_scan(unsigned long long* __restrict__ bsum,
+                                                     const uint32_t* __restrict__ bdead, int nb,
+                                                     unsigned long long* __restrict__ total,
+                                                     int32_t* __restrict__ d_count) {
+  constexpr int kPer = 4;
   __shared__ unsigned long long s_w[32];
-  __shared__ unsigned long long s_carry;
+  __shared__ unsigned int s_d[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int c0 = 0; c0 < nb; c0 += 1024) {
-    const int i = c0 + threadIdx.x;
-    const unsigned long long x = i < nb ? bsum[i] : 0ull;
-    unsigned long long inc = x;
+  unsigned long long carry = 0;
+  unsigned int dead = 0;
+  for (int c0 = 0; c0 < nb; c0 += 1024 * kPer) {
+    const int i0 = c0 + threadIdx.x * kPer;
+    unsigned long long x[kPer], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      x[q] = i0 + q < nb ? bsum[i0 + q] : 0ull;
+      dead += i0 + q < nb ? bdead[i0 + q] : 0u;
+      sum += x[q];
+    }
+    unsigned long long inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
@@ -290,123 +321,160 @@ __global__ void __launch_bounds__(1024) k_reloc_scan(unsigned long long* __restr
       if (w < warp) pre += s_w[w];
       tot += s_w[w];
     }
-    const unsigned long long carry = s_carry;
-    if (i < nb) bsum[i] = carry + pre + inc - x;   // exclusive block offsets, in place
-    __syncthreads();
-    if (threadIdx.x == 0) s_carry = carry + tot;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *total = s_carry;
-}
-
-__global__ void __launch_bounds__(256) k_reloc_cdf(const uint32_t* __restrict__ w, int n,
-                                                   const unsigned long long* __restrict__ boff,
-                                                   unsigned long long* __restrict__ cdf) {
-  __shared__ unsigned long long s_w[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned long long x = i < n ? (unsigned long long)(w[i] & ~kDeadBit) : 0ull;
-  unsigned long long inc = x;
+    unsigned long long run = carry + pre + inc - sum;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += y;
-  }
-  if (lane == 31) s_w[warp] = inc;
-  __syncthreads();
-  unsigned long long pre = 0;
-  for (int ww = 0; ww < warp; ++ww) pre += s_w[ww];
-  if (i < n) cdf[i] = boff[blockIdx.x] + pre + inc;
-}
-
-__global__ void __launch_bounds__(256) k_reloc_sample(const uint32_t* __restrict__ w, int n,
-                                                      const unsigned long long* __restrict__ cdf,
-                                                      const unsigned long long* __restrict__ total,
-                                                      const uint32_t* __restrict__ rnd,
-                                                      int32_t* __restrict__ src, uint32_t* __restrict__ copies,
-                                                      int32_t* __restrict__ d_count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const unsigned long long T = *total;
-  int32_t s = -1;
-  if ((w[i] & kDeadBit) && T > 0) {
-    // t = floor(r T / 2^32), exactly: T = hi 2^32 + lo
-    const unsigned long long r = rnd[i];
-    const unsigned long long t = r * (T >> 32) + ((r * (T & 0xffffffffull)) >> 32);
-    int lo = 0, hi = n - 1;                      // first index with cdf > t
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (cdf[mid] > t) hi = mid; else lo = mid + 1;
+    for (int q = 0; q < kPer; ++q) {
+      if (i0 + q < nb) bsum[i0 + q] = run;
+      run += x[q];
     }
-    s = lo;
-    atomicAdd(&copies[s], 1u);
-    atomicAdd(d_count, 1);
+    carry += tot;
+    __syncthreads();   // s_w is written again
   }
-  src[i] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dead += __shfl_xor_sync(0xffffffffu, dead, o);
+  if (lane == 0) s_d[warp] = dead;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned int d = 0;
+    for (int w = 0; w < 32; ++w) d += s_d[w];
+    *total = carry;
+    *d_count = carry > 0 ? (int32_t)d : 0;
+  }
 }
 
-__global__ void __launch_bounds__(256) k_reloc_opacity(float* __restrict__ planes, int n, int pitch,
-                                                       const uint32_t* __restrict__ copies) {
+__global__ void __launch_bounds__(kRelocBlock) k_reloc_sample(const uint32_t* __restrict__ w, int n,
+                                                              const unsigned long long* __restrict__ boff, int nb,
+                                                              const unsigned long long* __restrict__ total,
+                                                              const uint32_t* __restrict__ rnd,
+                                                              int32_t* __restrict__ src,
+                                                              uint32_t* __restrict__ copies) {
+  const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || copies[i] == 0u) return;
-  const float inv_n = 1.0f / (float)(copies[i] + 1u);
-  float* lp = planes + (size_t)10 * pitch + i;
-  // -log(1 - o) = softplus(logit), from the logit (1 - o by subtraction loses
-  // the digits of an opacity near 1); q = -log(1 - o') = softplus / N
-  const float x = *lp;
-  const float q = (x > 0.0f ? x + log1pf(expf(-x)) : log1pf(expf(x))) * inv_n;
-  const float o_new = -expm1f(-q);                       // 1 - (1 - o)^(1/N)
-  *lp = logf(o_new) + q;                                 // log o' - log(1 - o')
+  const unsigned long long T = *total;
+  const bool dead = i < n && (w[i] & kDeadBit) && T > 0;
+  int32_t mine = -1;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, dead); todo; todo &= todo - 1u) {
+    const int from = __ffs(todo) - 1;
+    const int d = __shfl_sync(0xffffffffu, i, from);
+    // t = floor(r T / 2^32), exactly: T = hi 2^32 + lo
+    const unsigned long long r = rnd[d];
+    const unsigned long long t = r * (T >> 32) + ((r * (T & 0xffffffffull)) >> 32);
+    // the last block whose offset is <= t: t < T, so its weights reach past t
+    int lo = 0, len = nb;
+    while (len > 1) {
+      const int step = (len + 31) >> 5;
+      const bool le = lane * step < len && boff[lo + lane * step] <= t;
+      const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
+      lo += k * step;
+      len = min(step, len - k * step);
+    }
+    // first primitive of the block whose inclusive sum exceeds t
+    const unsigned long long rem = t - boff[lo];
+    const int base = lo * kRelocBlock + lane * (kRelocBlock / 32);
+    uint32_t x[kRelocBlock / 32];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int q = 0; q < kRelocBlock / 32; ++q) {
+      x[q] = base + q < n ? w[base + q] & ~kDeadBit : 0u;
+      sum += x[q];
+    }
+    unsigned long long inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const int who = __ffs(__ballot_sync(0xffffffffu, inc > rem)) - 1;
+    unsigned long long run = inc - sum;
+    int at = 0;
+#pragma unroll
+    for (int q = 0; q < kRelocBlock / 32; ++q) {
+      run += x[q];
+      at += run <= rem ? 1 : 0;
+    }
+    const int s = __shfl_sync(0xffffffffu, base + at, who);
+    if (lane == 0) atomicAdd(&copies[s], 1u);
+    if (lane == from) mine = s;
+  }
+  if (i < n) src[i] = mine;
 }
 
+// Block row y < gridDim.y - 1 copies planes y kCopyPlanes .. (the opacity plane
+// apart) of 256 primitives, consecutive blocks sweeping along the planes; the
+// last row writes the new opacity logits.  Sources are live: nothing but their
+// logit changes.
+constexpr int kCopyPlanes = 9;
 __global__ void __launch_bounds__(256) k_reloc_copy(float* __restrict__ planes, float* __restrict__ m,
                                                     float* __restrict__ v, int n, int pitch, int np,
-                                                    const int32_t* __restrict__ src) {
+                                                    const int32_t* __restrict__ src,
+                                                    const uint32_t* __restrict__ copies,
+                                                    const float* __restrict__ logit) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int s = src[i];
-  if (s < 0) return;
-  for (int k = 0; k < np; ++k) {
-    const size_t at = (size_t)k * pitch;
-    planes[at + i] = planes[at + s];
-    if (m) m[at + i] = 0.0f;
-    if (v) v[at + i] = 0.0f;
+  const int32_t s = src[i];
+  if (blockIdx.y + 1 == gridDim.y) {
+    const int from = s >= 0 ? s : i;
+    const uint32_t c = copies[from];
+    if (c != 0u) {
+      const float inv_n = 1.0f / (float)(c + 1u);
+      // -log(1 - o) = softplus(logit), from the logit (1 - o by subtraction loses
+      // the digits of an opacity near 1); q = -log(1 - o') = softplus / N
+      const float x = logit[from];
+      const float q = (x > 0.0f ? x + log1pf(expf(-x)) : log1pf(expf(x))) * inv_n;
+      const float o_new = -expm1f(-q);                       // 1 - (1 - o)^(1/N)
+      planes[(size_t)10 * pitch + i] = logf(o_new) + q;      // log o' - log(1 - o')
+    }
+    if (s >= 0) {
+      if (m) m[(size_t)10 * pitch + i] = 0.0f;
+      if (v) v[(size_t)10 * pitch + i] = 0.0f;
+    }
+    return;
   }
+  if (s < 0) return;
+  const int k0 = blockIdx.y * kCopyPlanes;
+  float x[kCopyPlanes];
+#pragma unroll
+  for (int k = 0; k < kCopyPlanes; ++k)
+    if (k0 + k < np && k0 + k != 10) x[k] = planes[(size_t)(k0 + k) * pitch + s];
+#pragma unroll
+  for (int k = 0; k < kCopyPlanes; ++k)
+    if (k0 + k < np && k0 + k != 10) {
+      const size_t at = (size_t)(k0 + k) * pitch + i;
+      planes[at] = x[k];
+      if (m) m[at] = 0.0f;
+      if (v) v[at] = 0.0f;
+    }
 }
 
 }  // namespace
 
-// workspace carve-up: weights u32[n], cdf u64[n], block sums u64[nb], total
-// u64, copies u32[n], sources i32[n] (256-byte aligned pieces)
+// workspace carve-up: weights u32[n], old logits f32[n], block sums u64[nb], dead
+// counts u32[nb], total u64, copies u32[n], sources i32[n] (256-byte aligned pieces)
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 size_t reloc_ws_bytes(int n) {
-  const size_t nb = (size_t)(n + 255) / 256;
-  return al256((size_t)n * 4) + al256((size_t)n * 8) + al256(nb * 8) + al256(8) + al256((size_t)n * 4) +
-         al256((size_t)n * 4);
+  const size_t nb = (size_t)(n + kRelocBlock - 1) / kRelocBlock;
+  return al256((size_t)n * 4) * 4 + al256(nb * 8) + al256(nb * 4) + al256(8);
 }
 
 cudaError_t launch_relocate(int n, int pitch, int n_planes, float* planes, float* m, float* v,
                             const uint32_t* rnd, float min_opacity, void* ws, int32_t* src_out,
                             int32_t* d_count, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int nb = (n + 255) / 256;
+  const int nb = (n + kRelocBlock - 1) / kRelocBlock;
   char* p = (char*)ws;
   uint32_t* w = (uint32_t*)p;                   p += al256((size_t)n * 4);
-  unsigned long long* cdf = (unsigned long long*)p; p += al256((size_t)n * 8);
+  float* logit = (float*)p;                     p += al256((size_t)n * 4);
   unsigned long long* bsum = (unsigned long long*)p; p += al256((size_t)nb * 8);
+  uint32_t* bdead = (uint32_t*)p;               p += al256((size_t)nb * 4);
   unsigned long long* total = (unsigned long long*)p; p += al256(8);
   uint32_t* copies = (uint32_t*)p;              p += al256((size_t)n * 4);
   int32_t* src = src_out ? src_out : (int32_t*)p;
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(copies, 0, (size_t)n * 4, s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(d_count, 0, 4, s)) != cudaSuccess) return e;
-  k_reloc_weights<<<nb, 256, 0, s>>>(planes, n, pitch, min_opacity, w, bsum);
-  k_reloc_scan<<<1, 1024, 0, s>>>(bsum, nb, total);
-  k_reloc_cdf<<<nb, 256, 0, s>>>(w, n, bsum, cdf);
-  k_reloc_sample<<<nb, 256, 0, s>>>(w, n, cdf, total, rnd, src, copies, d_count);
-  k_reloc_opacity<<<nb, 256, 0, s>>>(planes, n, pitch, copies);
-  k_reloc_copy<<<nb, 256, 0, s>>>(planes, m, v, n, pitch, n_planes, src);
+  k_reloc_weights<<<nb, kRelocBlock, 0, s>>>(planes, n, pitch, min_opacity, w, copies, logit, bsum, bdead);
+  k_reloc_scan<<<1, 1024, 0, s>>>(bsum, bdead, nb, total, d_count);
+  k_reloc_sample<<<nb, kRelocBlock, 0, s>>>(w, n, bsum, nb, total, rnd, src, copies);
+  const dim3 grid((n + 255) / 256, (n_planes + kCopyPlanes - 1) / kCopyPlanes + 1);
+  k_reloc_copy<<<grid, 256, 0, s>>>(planes, m, v, n, pitch, n_planes, src, copies, logit);
   return cudaGetLastError();
 }
 
