@@ -73,6 +73,8 @@ int build_views(const beta_camera* cams, int32_t n_views, const beta_opts* opt, 
     d.nty = (c.height + opt->tile_h - 1) / opt->tile_h;
     d.tile_off = (int32_t)tiles;
     d.pix_off = pix;
+    d.l1_scale = 1.0f / (3.0f * (float)((int64_t)c.width * c.height));
+    d.inv_ntx = 1.0f / (float)d.ntx;
     tiles += (int64_t)d.ntx * d.nty;
     pix += (int64_t)c.width * c.height;
   }

@@ -33,6 +33,8 @@ struct ViewDev {
   int32_t tile_off;
   int32_t pad0;
   int64_t pix_off;
+  float l1_scale;      // 1 / (3 width height), rounded as the kernels that divide round it
+  float inv_ntx;       // 1 / ntx
 };
 
 struct ViewTable {
@@ -61,6 +63,23 @@ __device__ __forceinline__ int view_of_tile(const ViewTable& vt, int g) {
     if (vt.v[mid].tile_off <= g) lo = mid; else hi = mid - 1;
   }
   return lo;
+}
+
+// Column and row of global tile g in its view: the quotient by the view's
+// reciprocal (off by a few at the most for the largest grids), put right against
+// the remainder.
+__device__ __forceinline__ void tile_xy(const ViewDev& V, int g, int& tx, int& ty) {
+  const int lt = g - V.tile_off, ntx = V.ntx;
+  ty = (int)((float)lt * V.inv_ntx);
+  tx = lt - ty * ntx;
+  while (tx < 0) {
+    --ty;
+    tx += ntx;
+  }
+  while (tx >= ntx) {
+    ++ty;
+    tx -= ntx;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -472,8 +491,8 @@ struct ProjBuffers {
   uint2* rect;       // [V * pitch]  (tx0 | tx1 << 16, ty0 | ty1 << 16), tx0 > tx1 if empty
   uint32_t* key;     // [V * pitch]  depth key, 0xFFFFFFFF if not binned
   uint32_t* tiles;   // [V * pitch]  rule B2 tiles of the rectangle (bit r w + q; all ones: every tile)
-  uint32_t* work;    // records rule B2 applies to (k_tiles' worklist): projection block b owns
-                     // entries [b kProjRegion V, (b + 1) kProjRegion V), in arbitrary order
+  uint32_t* work;    // records rule B2 applies to: projection block b owns entries
+                     // [b kProjRegion V, (b + 1) kProjRegion V), in arbitrary order
   uint32_t* n_work;  // [projection blocks] entries of each block's region
 };
 
