@@ -635,13 +635,13 @@ def main():
                 "full_frame_4096_betas_256x256": c1}
 
     # kernel launches of ours inside the timed region (all inside the replayed graph on
-    # one GPU): project 3 (worklist reset, projection, rule-B2 tiles); bin_sort 5 (prep,
-    # tile counts, scan, scatter, list sort); schedule 3 (persistent); raster fwd with
+    # one GPU): project 1 (with the rule-B2 tiles); bin_sort 5 (prep, tile counts,
+    # scan, scatter, list sort); schedule 3 (persistent); raster fwd with
     # the L1 term 2 and raster bwd 1, or the one-launch raster kernel and the L1
     # reduce 2; project bwd 1 (one per chunk on several GPUs)
     from paper_2501_18630_gb300.distributed import chunk_ranges
     n_pbwd = len(chunk_ranges(sc.n, max(4, (sc.n + 7) // 8))) if world > 1 else 1
-    per_step = 3 + 5 + (3 if rast.persistent else 0) + (2 if fused else 3) + n_pbwd
+    per_step = 1 + 5 + (3 if rast.persistent else 0) + (2 if fused else 3) + n_pbwd
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",

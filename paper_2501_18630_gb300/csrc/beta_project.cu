@@ -137,14 +137,47 @@ __device__ __forceinline__ void sb_colour(const float* p, const PrimAttr<M>& a, 
   }
 }
 
-constexpr int kFwdThreads = 256, kFwdBlocksPerSM = 1;
+constexpr int kFwdThreads = 256;
+// CTAs per SM asked of the register allocator: 64 registers up to 3 lobes, 80
+// above.  Fused with rule B2's latency-bound tail the kernel wants warps: at
+// 1 / 2 / 3 / 4 CTAs per SM, 1M primitives x 1 view take 80 / 80 / 63 / 53 us
+// with 1 lobe, 90 / 90 / 70 / 62 with 3, 94 / 94 / 74 / 68 with 4, 193 / 113 /
+// 103 / 102 with 8; 500k x 8 views 134 / 134 / 115 / 109, 139 / 139 / 121 / 123,
+// 142 / 143 / 125 / 134 and 238 / 159 / 172 / 174 us.
+constexpr int fwd_blocks_per_sm(int lobes) { return lobes <= 3 ? 4 : 3; }
 
+// Rule B2 for one record of the block's worklist: the rule chain recomputed (the
+// same fp32 operations as the view loop, so the same rectangle) and the tiles
+// of the rectangle the support reaches.
+__device__ __forceinline__ void narrow_tiles(const float* __restrict__ planes, int pitch, const ViewTable& vt,
+                                             const RenderOpts& ro, uint32_t r, uint32_t* tiles) {
+  const int sw = __ffs(ro.tile_w) - 1, sh = __ffs(ro.tile_h) - 1;
+  const int v = (int)(r / (uint32_t)pitch), i = (int)(r - (uint32_t)v * (uint32_t)pitch);
+  float p[10];
+#pragma unroll
+  for (int q = 0; q < 10; ++q) p[q] = planes[(size_t)q * pitch + i];
+  PrimGeo pg;
+  ViewGeo g;
+  uint32_t kk;
+  int rc[4];
+  const ViewDev& V = vt.v[v];
+  if (rule_prim(p, pg) && rule_depth(pg, V, g, kk) && rule_view(pg, V, ro.blur_eps, sw, sh, g, rc))
+    tiles[r] = rule_tiles(g, V, ro.blur_eps, sw, ro.tile_h, rc);
+}
+
+// Projection of one primitive a thread over all views, then (in the same CTA)
+// rule B2 for the records it applies to: a worklist packs them into full warps,
+// which evaluating the rule's correctly rounded divisions and roots inline would
+// not.
 template <int M>
-__global__ void __launch_bounds__(kFwdThreads, kFwdBlocksPerSM) k_project(const float* __restrict__ planes, int n, int pitch,
+__global__ void __launch_bounds__(kFwdThreads, fwd_blocks_per_sm(M)) k_project(const float* __restrict__ planes, int n, int pitch,
                                                  ViewTable vt, RenderOpts ro,
                                                  float4* __restrict__ rec, uint2* __restrict__ rect,
-                                                 uint32_t* __restrict__ key, uint32_t* __restrict__ tiles,
-                                                 uint32_t* __restrict__ work, uint32_t* __restrict__ n_work) {
+                                                 uint32_t* __restrict__ key, uint32_t* tiles,
+                                                 uint32_t* work, uint32_t* __restrict__ n_work) {
+  __shared__ uint32_t s_nw;
+  if (threadIdx.x == 0) s_nw = 0u;
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = i < pitch;   // threads past the pitch write nothing but join the warp's append
   float p[15 + 6 * M];
@@ -205,7 +238,7 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdBlocksPerSM) k_project(const 
       rec[r * kRecordF4 + 2] = o2;
       rect[r] = make_uint2((uint32_t)rc[0] | ((uint32_t)rc[1] << 16), (uint32_t)rc[2] | ((uint32_t)rc[3] << 16));
       key[r] = kk;
-      tiles[r] = rule_all_tiles(rc);   // k_tiles narrows it where rule B2 applies
+      tiles[r] = rule_all_tiles(rc);   // narrowed below where rule B2 applies
     } else if (live) {
       rect[r] = make_uint2(1u, 1u);
       key[r] = 0xffffffffu;
@@ -213,9 +246,8 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdBlocksPerSM) k_project(const 
     }
     if (bin && rule_tiles_apply(rc)) need |= 1ull << v;
   }
-  // the records rule B2 applies to go on k_tiles' worklist, in this block's
-  // region: one atomic per warp, after the view loop (every thread of the
-  // warp gets here: none returned early)
+  // the records rule B2 applies to go on the block's worklist: one atomic per
+  // warp, after the view loop (every thread gets here: none returned early)
   const int lane = threadIdx.x & 31;
   const int cnt = __popcll(need);
   int incl = cnt;
@@ -224,43 +256,15 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdBlocksPerSM) k_project(const 
     const int y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
-  const int total = __shfl_sync(0xffffffffu, incl, 31);
-  if (total == 0) return;
   uint32_t base = 0;
-  if (lane == 31) base = atomicAdd(&n_work[blockIdx.x], (uint32_t)total);
+  if (lane == 31) base = atomicAdd(&s_nw, (uint32_t)incl);
   base = __shfl_sync(0xffffffffu, base, 31) + (uint32_t)(incl - cnt);
   uint32_t* region = work + (size_t)blockIdx.x * kProjRegion * vt.n_views;
   for (uint64_t m = need; m; m &= m - 1ull) region[base++] = (uint32_t)(__ffsll((long long)m) - 1) * (uint32_t)pitch + (uint32_t)i;
-}
-
-__global__ void k_proj_prep(uint32_t* n_work, int nb) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) n_work[b] = 0u;
-}
-
-// Rule B2 for the records on the worklist: the rule chain recomputed (the
-// same fp32 operations as k_project, so the same rectangle) and the tiles of
-// the rectangle the support reaches.  The worklist packs the records that
-// need it into full warps; CTA b takes projection block b's region.
-__global__ void __launch_bounds__(256) k_tiles(const float* __restrict__ planes, int pitch, ViewTable vt,
-                                               RenderOpts ro, const uint32_t* __restrict__ work,
-                                               const uint32_t* __restrict__ n_work, uint32_t* __restrict__ tiles) {
-  const uint32_t nw = n_work[blockIdx.x];
-  const uint32_t* region = work + (size_t)blockIdx.x * kProjRegion * vt.n_views;
-  const int sw = __ffs(ro.tile_w) - 1, sh = __ffs(ro.tile_h) - 1;
-  for (uint32_t k = threadIdx.x; k < nw; k += blockDim.x) {
-    const uint32_t r = region[k];
-    const int v = (int)(r / (uint32_t)pitch), i = (int)(r - (uint32_t)v * (uint32_t)pitch);
-    float p[10];
-#pragma unroll
-    for (int q = 0; q < 10; ++q) p[q] = planes[(size_t)q * pitch + i];
-    PrimGeo pg;
-    ViewGeo g;
-    uint32_t kk;
-    int rc[4];
-    const ViewDev& V = vt.v[v];
-    if (rule_prim(p, pg) && rule_depth(pg, V, g, kk) && rule_view(pg, V, ro.blur_eps, sw, sh, g, rc))
-      tiles[r] = rule_tiles(g, V, ro.blur_eps, sw, ro.tile_h, rc);
-  }
+  __syncthreads();   // the list, and the tile masks of the view loop, which are written again
+  const uint32_t nw = s_nw;
+  if (threadIdx.x == 0) n_work[blockIdx.x] = nw;
+  for (uint32_t k = threadIdx.x; k < nw; k += blockDim.x) narrow_tiles(planes, pitch, vt, ro, region[k], tiles);
 }
 
 // Per-view geometry for the backward: the same quantities as the rule chain
@@ -518,10 +522,8 @@ static cudaError_t launch_project_m(const float* planes, int n, int pitch, const
   int grid = (pitch + kFwdThreads - 1) / kFwdThreads;
   if (grid < 1) return cudaSuccess;
   static_assert(kFwdThreads == kProjRegion, "a projection block owns one worklist region");
-  k_proj_prep<<<(grid + 255) / 256, 256, 0, s>>>(pb.n_work, grid);
   k_project<M><<<grid, kFwdThreads, 0, s>>>(planes, n, pitch, vt, ro, pb.rec, pb.rect, pb.key, pb.tiles,
                                             pb.work, pb.n_work);
-  k_tiles<<<grid, 256, 0, s>>>(planes, pitch, vt, ro, pb.work, pb.n_work, pb.tiles);
   return cudaGetLastError();
 }
 
