@@ -18,7 +18,8 @@ def _vp(t):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle: a torch.cuda.Stream object costs 3 us a call
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 class Rasterizer:
@@ -49,8 +50,15 @@ class Rasterizer:
         dev = self.device
         self.proj = torch.empty(int(L.beta_proj_bytes(self.pitch, self.V)), dtype=torch.uint8, device=dev)
         self.ranges = torch.empty(self.total_tiles + 1, dtype=torch.int32, device=dev)
-        self.count = torch.zeros(1, dtype=torch.int64, device=dev)
-        self.status = torch.zeros(1, dtype=torch.int32, device=dev)
+        # pair count and status word side by side, so that one copy reads both
+        # back (into pinned memory: the copy does not block the host)
+        self._state = torch.zeros(2, dtype=torch.int64, device=dev)
+        self.count = self._state[:1]
+        self.status = self._state.view(torch.int32)[2:3]
+        self._host_state = torch.zeros(2, dtype=torch.int64).pin_memory()
+        self._host_count = self._host_state.numpy()[:1]
+        self._host_status = self._host_state.numpy().view("int32")[2:3]
+        self._state_read = torch.cuda.Event()
         self.color = torch.empty(3 * self.total_pixels, dtype=torch.float32, device=dev)
         self.T_final = torch.empty(self.total_pixels, dtype=torch.float32, device=dev)
         self.n_contrib = torch.empty(self.total_pixels, dtype=torch.int32, device=dev)
@@ -210,32 +218,58 @@ class Rasterizer:
             ctypes.c_void_p(grad_planes.data_ptr() + 4 * c0), _vp(self.status), _stream()))
 
     # -- composite calls ---------------------------------------------------
+    def _read_state(self):
+        """Starts the copy of (pair count, status) to the host."""
+        self._host_state.copy_(self._state, non_blocking=True)
+
     def device_status(self):
         """(status, pair count); synchronises the current stream."""
+        self._read_state()
         torch.cuda.current_stream().synchronize()
-        return int(self.status.item()), int(self.count.item())
+        return int(self._host_status[0]), int(self._host_count[0])
 
-    def forward(self, planes, check_capacity: bool = True):
-        """project + bin/sort + raster.  With check_capacity the pair count is
-        read back (one host sync) and the pair buffers grow if needed."""
-        self.project(planes)
-        self.bin_sort(planes)
-        if check_capacity:
-            st, k = self.device_status()
-            if st == _lib.BETA_ERR_CAPACITY:
-                self._alloc_pairs(int(math.ceil(k * 1.25)) + 1024)
-                self.bin_sort(planes)
-                st, k = self.device_status()
-            if st != _lib.BETA_OK:
-                raise _lib.BetaError("beta_bin_sort", st, self.L.beta_status_string(st).decode())
+    def _composite(self, planes):
         if self.persistent:
             self.schedule()
         self.raster_fwd(planes)
+
+    def forward(self, planes, check_capacity: bool = True):
+        """project + bin/sort + raster.  With check_capacity the pair count is
+        read back and the pair buffers grow if needed.  The host waits for the
+        binning only: the raster kernels are launched behind it first (they
+        write nothing when the binning reports an overflow), so the GPU does not
+        idle while the host reads the count and goes on to the next launch."""
+        self.project(planes)
+        self.bin_sort(planes)
+        if not check_capacity:
+            self._composite(planes)
+            return self.color
+        self._read_state()
+        self._state_read.record()
+        self._composite(planes)
+        self._state_read.synchronize()
+        st, k = int(self._host_status[0]), int(self._host_count[0])
+        if st == _lib.BETA_ERR_CAPACITY:
+            self._alloc_pairs(int(math.ceil(k * 1.25)) + 1024)
+            self.bin_sort(planes)
+            st, k = self.device_status()
+            if st == _lib.BETA_OK:
+                self._composite(planes)
+        if st != _lib.BETA_OK:
+            raise _lib.BetaError("beta_bin_sort", st, self.L.beta_status_string(st).decode())
         return self.color
+
+    def _empty_grad(self, planes):
+        """Gradient planes for project_bwd to fill: zeros where it writes nothing
+        (the padding columns)."""
+        grad = torch.empty_like(planes)
+        if self.n < self.pitch:
+            grad[:, self.n:].zero_()
+        return grad
 
     def backward(self, planes, dL_dcolor, grad_planes=None):
         if grad_planes is None:
-            grad_planes = torch.zeros_like(planes)
+            grad_planes = self._empty_grad(planes)
         self.raster_bwd(planes, dL_dcolor)
         self.project_bwd(planes, grad_planes)
         return grad_planes
