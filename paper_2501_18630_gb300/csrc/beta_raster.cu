@@ -656,46 +656,76 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
 }
 
 // ---------------------------------------------------------------------------
-// Pixel-pair raster kernels: every lane owns two horizontally adjacent pixels.
-// Warp w of a tile owns a BW x BH block (16 x 4 in tiles at least 16 wide,
-// else 8 x 8); lane L owns pixels (2 pc, r) and (2 pc + 1, r) of it, with
+// Pixel-pair raster kernels: every lane owns NP pairs of horizontally adjacent
+// pixels, one above the other (NP = 1, or 2: a 2 x 2 quad).  Warp w of a tile
+// owns a BW x BH block (16 x 4 NP in tiles at least 16 wide, else 8 x 8); lane L
+// owns pixels (2 pc, NP r + i) and (2 pc + 1, NP r + i), i < NP, of it, with
 // pc = L mod PC, r = L / PC, PC = BW / 2 pair columns.  A record's cover mask
-// has one bit per pair (bit L: the record may cover either pixel of lane L),
-// and the lanes walk the union of their two pixels' records: one set of
-// shared-memory record loads and, in the backward, one set of gradient
-// atomics serve both pixels (neighbouring pixels share most records), and the
-// warp-wide reductions of records covering many lanes serve 64 pixels.
+// has one bit per lane (bit L: the record may cover a pixel of lane L), and the
+// lanes walk the union of their pixels' records: one set of shared-memory
+// record loads and, in the backward, one set of gradient atomics serve them all
+// (neighbouring pixels share most records), and the warp-wide reductions of
+// records covering many lanes serve 64 NP pixels.
 // The walks are bound by instruction issue (82% of the slots at half of the
-// lanes), so both pixels' arithmetic is packed (fma.rn.f32x2 and its kin, one
-// slot for two fp32 results; a record's scalar is broadcast by the
-// instruction).  Scalar to packed: 3.94e8 -> 3.49e8 forward and 5.80e8 ->
-// 5.07e8 backward instructions on 1M Betas x 4 x 1080p (16x8 / 64), the one
-// launch 3.78 -> 3.43 ms at 16 views, forward and backward 9.26 -> 8.40 and
-// 21.9 -> 20.3 ms on 6M Betas x 8 x 4K.
+// lanes) and, as those fall, by the L1 data pipe (record loads and atomics), so
+// a pair's arithmetic is packed (fma.rn.f32x2 and its kin, one slot for two fp32
+// results; a record's scalar is broadcast by the instruction) and NP = 2 shares
+// the loads and atomics of four pixels.  Scalar to packed: 3.94e8 -> 3.49e8
+// forward and 5.80e8 -> 5.07e8 backward instructions on 1M Betas x 4 x 1080p
+// (16x8 / 64), the one launch 3.78 -> 3.43 ms at 16 views, forward and backward
+// 9.26 -> 8.40 and 21.9 -> 20.3 ms on 6M Betas x 8 x 4K.  NP 1 -> 2 (after the
+// packed cover pass): one launch 3.38 -> 2.84 ms, forward and backward of 6M x 8
+// x 4K 7.2 -> 7.0 and 20.3 -> 14.2 ms.
 // ---------------------------------------------------------------------------
-
-// Threads per SM asked of the register allocator for the pixel-pair kernels:
-// 1152 (56 registers) where the record buffers of 64-record batches leave
-// room for that many CTAs, 1024 (64 registers) for larger batches, whose
-// shared memory holds fewer CTAs anyway.  Packed pairs take aligned register
-// pairs: at 1280 threads (48 registers) the 64-record kernels spill 4 to 40
-// bytes.  Measured at 16x8 / 64, 1280 / 1152 / 1024: one launch on 1M Betas x
-// 16 x 1080p 3.44 / 3.43 / 3.59 ms, backward on 6M x 8 x 4K 20.66 / 20.28 /
-// 21.00 ms.
-constexpr int pair_threads_per_sm(int S) { return S <= 64 ? 1152 : 1024; }
 
 // Do TW x TH tiles hold whole pixel-pair blocks (16 x 4 in tiles at least
 // 16 wide, 8 x 8 in 8-wide ones)?  Those use the pixel-pair kernels, the
 // others (8 x 4) the one-pixel-per-lane ones; the hit-mask layout follows.
 constexpr bool pair_tiles(int tw, int th) { return th % (tw % 16 == 0 ? 4 : 8) == 0; }
 
-template <int TW>
+// Pairs a lane owns.  Two need 16 x 8 blocks and record batches of at most two
+// records per thread (larger ones leave room for too few CTAs: 16x16 / 256
+// forward 1.38 -> 1.59 ms at 1M Betas x 16 x 1080p), and enough blocks to fill
+// the chip with half the warps.  At 16x8 / 64 the one launch takes, NP 1 / 2: 9840
+// blocks (4 x 641x479, clustered lists) 130 / 151 us; 16200 (one 1080p view)
+// 253 / 223; 32400 466 / 407; 64800 877 / 752; at 32x16 / 128, 10080 blocks
+// 199 / 220 us, 16320 392 / 333.
+constexpr int kQuadBlocks = 16000;
+constexpr bool quad_shape(int tw, int th, int S) {
+  return tw % 16 == 0 && th % 8 == 0 && S <= 2 * (tw * th / 4);
+}
+inline int lane_pairs(const RenderOpts& ro, int total_tiles) {
+  return quad_shape(ro.tile_w, ro.tile_h, ro.batch_s) &&
+                 (int64_t)total_tiles * (ro.tile_w * ro.tile_h / 128) >= kQuadBlocks
+             ? 2 : 1;
+}
+
+template <int TW, int TH, int NP>
 struct PairBlock {
   static constexpr int BW = TW % 16 == 0 ? 16 : 8;   // block width in pixels
-  static constexpr int BH = 64 / BW;                 // block height
+  static constexpr int BH = 64 * NP / BW;            // block height
   static constexpr int PC = BW / 2;                  // pair columns
   static constexpr int WX = TW / BW;                 // blocks per tile row
+  static constexpr int NT = TW * TH / (2 * NP);      // threads of a tile's CTA
+  static constexpr int NW = NT / 32;
+  // Records covering more lanes than this are reduced across the warp.  With
+  // quads a lane's atomics serve four pixels, so more lanes add their own: 12 /
+  // 16 / 20 / 24 / 28 took 3.17 / 2.96 / 2.87 / 2.84 / 2.82 ms (one launch, 1M
+  // Betas x 16 x 1080p) and 18.4 / 16.1 / 14.7 / 14.2 / 14.7 ms (backward, 6M x 8
+  // x 4K).
+  static constexpr int kWide = NP == 1 ? kLaneAtomics : 24;
 };
+
+// CTAs per SM asked of the register allocator.  One pair: 1152 threads (56
+// registers) where the record buffers of 64-record batches leave room for that
+// many CTAs, 1024 (64) for larger batches (at 16x8 / 64, 1280 / 1152 / 1024
+// threads: one launch 3.44 / 3.43 / 3.59 ms, backward of 6M x 8 x 4K 20.66 / 20.28
+// / 21.00 ms: packed pairs take aligned register pairs, and 48 registers spill).
+// Two pairs: 704 threads (80 registers; 1024 / 800 / 704 / 640: 3.93 / 3.34 /
+// 3.17 / 3.2 ms with kWide 12), 768 for larger batches.
+constexpr int pair_ctas_per_sm(int tw, int th, int S, int np) {
+  return min_blocks(tw * th / (2 * np), np == 1 ? (S <= 64 ? 1152 : 1024) : (S <= 64 ? 704 : 768));
+}
 
 // Two floats in one 64-bit register (the lane's two pixels: lo = pixel 0) and
 // the packed fp32 instructions of sm_100+: one issue slot for both pixels, each
@@ -755,12 +785,10 @@ __device__ __forceinline__ uint32_t bit_run(uint32_t pos, uint32_t width) {
 // pair column pc.  Per row the support is the interval of block_cover (same
 // closed form and margins, so every pixel the exact test accepts is covered);
 // the pairs are those holding a column of it.  Two rows at a time in packed
-// arithmetic and bit runs by one instruction (with the transpose the pass was a
-// fifth of the forward's instructions: 3.49e8 -> 2.94e8 on 1M Betas x 4 x 1080p,
-// 16x8 / 64; forward of 6M Betas x 8 x 4K 8.40 -> 7.15 ms).
-template <int BW>
+// arithmetic (the pass was a fifth of the forward's instructions).
+template <int BW, int NP>
 __device__ __forceinline__ uint32_t pair_cover(float4 f0, float4 f1, float bxf, float byf) {
-  constexpr int BH = 64 / BW, PC = BW / 2;
+  constexpr int BH = 64 * NP / BW, PC = BW / 2;
   constexpr int kMagic = 0x4B400000;                 // bits of kRoundMagic: integer k reads kMagic + k
   const float p = f1.x, q1 = f1.y, q2 = f1.z;
   const float X0 = (bxf - f0.x) + f0.z;              // dx of the block's first column
@@ -794,22 +822,25 @@ __device__ __forceinline__ uint32_t pair_cover(float4 f0, float4 f1, float bxf, 
     // pairs (il >> 1) .. (ih >> 1); kMagic is even, so it halves exactly
     const int n0 = d0 > 0.0f && il0 <= ih0 ? (ih0 >> 1) - (il0 >> 1) + 1 : 0;
     const int n1 = d1 > 0.0f && il1 <= ih1 ? (ih1 >> 1) - (il1 >> 1) + 1 : 0;
-    m |= bit_run((uint32_t)((il0 >> 1) - (kMagic >> 1) + PC * r), (uint32_t)n0);
-    m |= bit_run((uint32_t)((il1 >> 1) - (kMagic >> 1) + PC * (r + 1)), (uint32_t)n1);
+    m |= bit_run((uint32_t)((il0 >> 1) - (kMagic >> 1) + PC * (r / NP)), (uint32_t)n0);
+    m |= bit_run((uint32_t)((il1 >> 1) - (kMagic >> 1) + PC * ((r + 1) / NP)), (uint32_t)n1);
   }
   return m;
 }
 
-// 1 - r^2 of a staged record at the lane's two pixel centres, x2 = (xf, xf + 1)
-// in row yf, with their whitened coordinates: each pixel's the values rec_r2
-// gives it (the row term q1 dy is shared), so that every pixel composites the
-// same way whatever the tiling, and the forward and the backward see the same
-// values.  r^2 < 1 exactly where 1 - r^2 > 0 (the difference is at least 2^-24
-// there; NaN is neither).
-__device__ __forceinline__ f32x2 rec_om_pair(float4 f0, float4 f1, f32x2 x2, float yf, f32x2& u, f32x2& v) {
-  const f32x2 dx = add2(add2(x2, both2(-f0.x)), both2(f0.z));
-  const float dy = (yf - f0.y) + f0.w;
+// A staged record at the lane's two pixel columns: dx and u = p dx, the same
+// for every row of the lane.
+__device__ __forceinline__ void rec_cols(float4 f0, float4 f1, f32x2 x2, f32x2& dx, f32x2& u) {
+  dx = add2(add2(x2, both2(-f0.x)), both2(f0.z));
   u = mul2(both2(f1.x), dx);
+}
+// 1 - r^2 of the record at the two pixel centres of row yf, with their second
+// whitened coordinate: each pixel's the values rec_r2 gives it (the row term
+// q1 dy is shared), so that every pixel composites the same way whatever the
+// tiling, and the forward and the backward see the same values.  r^2 < 1 exactly
+// where 1 - r^2 > 0 (the difference is at least 2^-24 there; NaN is neither).
+__device__ __forceinline__ f32x2 rec_om(float4 f0, float4 f1, f32x2 dx, f32x2 u, float yf, f32x2& v) {
+  const float dy = (yf - f0.y) + f0.w;
   v = fma2(both2(f1.z), dx, both2(f1.y * dy));
   const f32x2 r2 = fma2(u, u, mul2(v, v));
   return fma2(r2, both2(-1.0f), both2(1.0f));
@@ -823,33 +854,35 @@ __device__ __forceinline__ bool finite_colour(float4 f2) {
 
 // Per-lane state of the pixel-pair forward after a tile's walk: transmittance,
 // accumulated colour and last contributor (1-based list position, 0 for none)
-// of the lane's two pixels.
+// of the lane's pixels (pixel 2 i + h: column h of pair i).
+template <int NP>
 struct PairFwdState {
-  float T0, T1, C00, C01, C02, C10, C11, C12;
-  uint32_t last0, last1;
+  float T[2 * NP], C[2 * NP][3];
+  uint32_t last[2 * NP];
   int walked_batch, walked_buf;   // the last batch the walk composited and its s_rec buffer (-1: none)
   bool odd_colours;               // a record the warp walked has a non-finite colour (warp-uniform)
 };
 
-// Forward walk of one tile's list [start, end) at the lane's pixel pair (xf,
-// yf), (xf + 1, yf) of the warp block whose first pixel is (bxf, byf): records
-// staged S per batch (double-buffered cp.async, the list entries of the next
-// batch loaded one batch ahead); per 32-record chunk the warp's cover pass and
-// bit transpose, then every lane composites its records in list order at both
-// pixels (Eq. C), until T < t_eps at every pixel of the CTA.  With hslot the
+// Forward walk of one tile's list [start, end) at the lane's pixel pairs (xf,
+// yf + i), (xf + 1, yf + i) of the warp block whose first pixel is (bxf, byf):
+// records staged S per batch (double-buffered cp.async, the list entries of the
+// next batch loaded one batch ahead); per 32-record chunk the warp's cover pass
+// and bit transpose, then every lane composites its records in list order at
+// its pixels (Eq. C), until T < t_eps at every pixel of the CTA.  With hslot the
 // cover masks of the list's first hm_chunks chunks are stored for the
 // backward; with ridx (a [2][S] array) the staged records' indices as well,
 // so that a backward can start from the last batch still in s_rec.  Returns
 // with every copy landed; the caller synchronises the CTA before s_rec is
 // staged again.
-template <int TW, int TH, int S>
+template <int TW, int TH, int S, int NP>
 __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], uint32_t* ridx,
                                               const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
                                               uint32_t start, uint32_t end, uint32_t* hslot, int hm_chunks,
-                                              float xf, float yf, float bxf, float byf, bool in0, bool in1,
-                                              float t_eps, float amax, PairFwdState& st) {
-  using PB = PairBlock<TW>;
-  constexpr int NT = TW * TH / 2, NW = NT / 32, RPT = (S + NT - 1) / NT;
+                                              float xf, float yf, float bxf, float byf,
+                                              const bool (&in)[2 * NP], float t_eps, float amax,
+                                              PairFwdState<NP>& st) {
+  using PB = PairBlock<TW, TH, NP>;
+  constexpr int NT = PB::NT, NW = PB::NW, RPT = (S + NT - 1) / NT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   // batch 0 goes to buffer 0 now; the list entries of batch 1 are loaded
@@ -869,12 +902,19 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
   cp_async_commit();
 
   // a pixel composites while T >= t_eps (>= 0); an off-image one starts below it
-  f32x2 T2 = pack2(in0 ? 1.0f : -1.0f, in1 ? 1.0f : -1.0f);
-  f32x2 Cr = 0ull, Cg = 0ull, Cb = 0ull;
+  f32x2 T2[NP], Cr[NP], Cg[NP], Cb[NP];
+  uint32_t last[2 * NP];
+  bool live[2 * NP], done = true;   // T >= t_eps (< 1); no pixel is live
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    T2[i] = pack2(in[2 * i] ? 1.0f : -1.0f, in[2 * i + 1] ? 1.0f : -1.0f);
+    Cr[i] = Cg[i] = Cb[i] = 0ull;
+    last[2 * i] = last[2 * i + 1] = 0u;
+    live[2 * i] = in[2 * i];
+    live[2 * i + 1] = in[2 * i + 1];
+    done = done && !in[2 * i] && !in[2 * i + 1];
+  }
   const f32x2 x2 = pack2(xf, xf + 1.0f), one2 = both2(1.0f), neg2 = both2(-1.0f);
-  uint32_t last0 = 0, last1 = 0;
-  bool live0 = in0, live1 = in1;   // T >= t_eps (< 1)
-  bool done = !in0 && !in1;        // both pixels
   bool warp_done = __all_sync(0xffffffffu, done);
   bool odd_any = false;
 
@@ -898,13 +938,13 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
     walked_buf = buf;
     const int cnt = (int)min((uint32_t)S, end - base);
     for (int c = 0; c < cnt && !warp_done; c += 32) {
-      // pass 1: lane k finds the pairs of this warp's block that record
+      // pass 1: lane k finds the lanes of this warp's block that record
       // c + k may cover; the transpose gives every lane its records
       const int idx = c + lane;
-uint32_t cov = 0u;
+      uint32_t cov = 0u;
       bool odd = false;
       if (idx < cnt) {
-        cov = pair_cover<PB::BW>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf);
+        cov = pair_cover<PB::BW, NP>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf);
         odd = !finite_colour(s_rec[buf][idx][2]);
       }
       uint32_t mine = transpose32(cov, lane);
@@ -913,15 +953,15 @@ uint32_t cov = 0u;
       const int jc = (int)((base - start + c) >> 5);
       if (hslot && jc < hm_chunks) {
         uint32_t* slot = hslot + (size_t)jc * (NT + NW);
-        const uint32_t wide = __ballot_sync(0xffffffffu, __popc(cov) > kLaneAtomics);
+        const uint32_t wide = __ballot_sync(0xffffffffu, __popc(cov) > PB::kWide);
         slot[tid] = mine;
         if (lane == 0) slot[NT + warp] = wide;
       }
       if (done) mine = 0u;
-      // pass 2: every lane composites its records in list order at both of
-      // its pixels in packed arithmetic; a pixel that the record does not
-      // cover, or that is done, takes alpha = 0, which leaves T and C as they
-      // are (colours are finite, or `odd` selects)
+      // pass 2: every lane composites its records in list order at its pixels
+      // in packed arithmetic; a pixel that the record does not cover, or that is
+      // done, takes alpha = 0, which leaves T and C as they are (colours are
+      // finite, or `odd` selects)
       while (mine) {
         const int k = __ffs(mine) - 1;
         mine &= mine - 1;
@@ -929,48 +969,54 @@ uint32_t cov = 0u;
         const float4 f0 = s_rec[buf][s][0];
         const float4 f1 = s_rec[buf][s][1];
         const float4 f2 = s_rec[buf][s][2];
-        f32x2 u, v;
-        const f32x2 om = rec_om_pair(f0, f1, x2, yf, u, v);
-        float om0, om1, T0, T1, e0, e1;
-        unpack2(om, om0, om1);
-        const bool h0 = live0 && om0 > 0.0f, h1 = live1 && om1 > 0.0f;
-        unpack2(fma2(both2(f1.w), pack2(lg2_approx(om0), lg2_approx(om1)), both2(f2.x)), e0, e1);
-        const float a0 = h0 ? fminf(ex2_approx(e0), amax) : 0.0f;
-        const float a1 = h1 ? fminf(ex2_approx(e1), amax) : 0.0f;
-        const f32x2 a2 = pack2(a0, a1);
-        const f32x2 w2 = mul2(a2, T2);
-        if (!odd) {
-          Cr = fma2(w2, both2(f2.y), Cr);
-          Cg = fma2(w2, both2(f2.z), Cg);
-          Cb = fma2(w2, both2(f2.w), Cb);
-        } else {
-          float w0, w1, r0, r1, g0, g1, b0, b1;
-          unpack2(w2, w0, w1);
-          unpack2(Cr, r0, r1);
-          unpack2(Cg, g0, g1);
-          unpack2(Cb, b0, b1);
-          if (h0) {
-            r0 = fmaf(w0, f2.y, r0);
-            g0 = fmaf(w0, f2.z, g0);
-            b0 = fmaf(w0, f2.w, b0);
-          }
-          if (h1) {
-            r1 = fmaf(w1, f2.y, r1);
-            g1 = fmaf(w1, f2.z, g1);
-            b1 = fmaf(w1, f2.w, b1);
-          }
-          Cr = pack2(r0, r1);
-          Cg = pack2(g0, g1);
-          Cb = pack2(b0, b1);
-        }
-        T2 = mul2(T2, fma2(a2, neg2, one2));
         const uint32_t pos = base - start + (uint32_t)s + 1u;
-        if (h0) last0 = pos;
-        if (h1) last1 = pos;
-        unpack2(T2, T0, T1);
-        live0 = T0 >= t_eps;
-        live1 = T1 >= t_eps;
-        done = !live0 && !live1;
+        f32x2 dx, u;
+        rec_cols(f0, f1, x2, dx, u);
+        done = true;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          f32x2 v;
+          const f32x2 om = rec_om(f0, f1, dx, u, i == 0 ? yf : yf + (float)i, v);
+          float om0, om1, T0, T1, e0, e1;
+          unpack2(om, om0, om1);
+          const bool h0 = live[2 * i] && om0 > 0.0f, h1 = live[2 * i + 1] && om1 > 0.0f;
+          unpack2(fma2(both2(f1.w), pack2(lg2_approx(om0), lg2_approx(om1)), both2(f2.x)), e0, e1);
+          const float a0 = h0 ? fminf(ex2_approx(e0), amax) : 0.0f;
+          const float a1 = h1 ? fminf(ex2_approx(e1), amax) : 0.0f;
+          const f32x2 a2 = pack2(a0, a1);
+          const f32x2 w2 = mul2(a2, T2[i]);
+          if (!odd) {
+            Cr[i] = fma2(w2, both2(f2.y), Cr[i]);
+            Cg[i] = fma2(w2, both2(f2.z), Cg[i]);
+            Cb[i] = fma2(w2, both2(f2.w), Cb[i]);
+          } else {
+            float w0, w1, r0, r1, g0, g1, b0, b1;
+            unpack2(w2, w0, w1);
+            unpack2(Cr[i], r0, r1);
+            unpack2(Cg[i], g0, g1);
+            unpack2(Cb[i], b0, b1);
+            if (h0) {
+              r0 = fmaf(w0, f2.y, r0);
+              g0 = fmaf(w0, f2.z, g0);
+              b0 = fmaf(w0, f2.w, b0);
+            }
+            if (h1) {
+              r1 = fmaf(w1, f2.y, r1);
+              g1 = fmaf(w1, f2.z, g1);
+              b1 = fmaf(w1, f2.w, b1);
+            }
+            Cr[i] = pack2(r0, r1);
+            Cg[i] = pack2(g0, g1);
+            Cb[i] = pack2(b0, b1);
+          }
+          T2[i] = mul2(T2[i], fma2(a2, neg2, one2));
+          if (h0) last[2 * i] = pos;
+          if (h1) last[2 * i + 1] = pos;
+          unpack2(T2[i], T0, T1);
+          live[2 * i] = T0 >= t_eps;
+          live[2 * i + 1] = T1 >= t_eps;
+          done = done && !live[2 * i] && !live[2 * i + 1];
+        }
         if (done) mine = 0u;
       }
       warp_done = __all_sync(0xffffffffu, done);
@@ -978,30 +1024,33 @@ uint32_t cov = 0u;
     buf ^= 1;
   }
   cp_async_wait_all();   // no copy may still land in a buffer the next tile fills
-  unpack2(T2, st.T0, st.T1);
-  unpack2(Cr, st.C00, st.C10);
-  unpack2(Cg, st.C01, st.C11);
-  unpack2(Cb, st.C02, st.C12);
-  st.last0 = last0;
-  st.last1 = last1;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    unpack2(T2[i], st.T[2 * i], st.T[2 * i + 1]);
+    unpack2(Cr[i], st.C[2 * i][0], st.C[2 * i + 1][0]);
+    unpack2(Cg[i], st.C[2 * i][1], st.C[2 * i + 1][1]);
+    unpack2(Cb[i], st.C[2 * i][2], st.C[2 * i + 1][2]);
+    st.last[2 * i] = last[2 * i];
+    st.last[2 * i + 1] = last[2 * i + 1];
+  }
   st.walked_batch = walked_batch;
   st.walked_buf = walked_buf;
   st.odd_colours = odd_any;
 }
 
-// Epilogue of the pixel-pair forward at pixels (x, y), (x + 1, y) of view v:
-// the colour C + T bg to color; T and the last contributor to Tout / ncontrib
-// when those are given; with a target (tgt[ch][2 tid + i]: pixel i, channel
+// Epilogue of the pixel-pair forward at the lane's pixels (x + h, y + i) of view
+// v: the colour C + T bg to color; T and the last contributor to Tout / ncontrib
+// when those are given; with a target (tgt[ch][2 NP tid + q]: pixel q, channel
 // ch, landed in shared memory) the L1 term, whose gradient
-// sign(C - target) / (3 H W) goes to dLdC when given and to gv (pixel i,
-// channel ch at gv[3 i + ch]; zero off the image or without a target).
+// sign(C - target) / (3 H W) goes to dLdC when given and to gv (pixel q,
+// channel ch at gv[3 q + ch]; zero off the image or without a target).
 // Returns the lane's sum of |C - target|.
-template <int NT>
-__device__ __forceinline__ float pair_fwd_out(const PairFwdState& st, const ViewTable& vt, int v, int x, int y,
-                                              bool in0, bool in1, bool with_target, const float (&tgt)[3][2 * NT],
-                                              float* __restrict__ color, float* __restrict__ Tout,
-                                              uint32_t* __restrict__ ncontrib, float* __restrict__ dLdC,
-                                              float (&gv)[6]) {
+template <int NT, int NP>
+__device__ __forceinline__ float pair_fwd_out(const PairFwdState<NP>& st, const ViewTable& vt, int v, int x, int y,
+                                              const bool (&in)[2 * NP], bool with_target,
+                                              const float (&tgt)[3][2 * NP * NT], float* __restrict__ color,
+                                              float* __restrict__ Tout, uint32_t* __restrict__ ncontrib,
+                                              float* __restrict__ dLdC, float (&gv)[6 * NP]) {
   const int tid = threadIdx.x;
   const int W = vt.v[v].width, H = vt.v[v].height;
   const int64_t HW = (int64_t)W * H;
@@ -1010,30 +1059,59 @@ __device__ __forceinline__ float pair_fwd_out(const PairFwdState& st, const View
   const float scale = vt.v[v].l1_scale;
   float l1 = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+  for (int q = 0; q < 2 * NP; ++q) {
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) gv[3 * i + ch] = 0.0f;
-    if (!(i == 0 ? in0 : in1)) continue;
-    const float T = i == 0 ? st.T0 : st.T1;
-    const float c[3] = {(i == 0 ? st.C00 : st.C10) + T * vt.v[v].bg[0], (i == 0 ? st.C01 : st.C11) + T * vt.v[v].bg[1],
-                        (i == 0 ? st.C02 : st.C12) + T * vt.v[v].bg[2]};
+    for (int ch = 0; ch < 3; ++ch) gv[3 * q + ch] = 0.0f;
+    if (!in[q]) continue;
+    const int64_t at = (int64_t)(q / 2) * W + (q & 1);
+    const float T = st.T[q];
+    const float c[3] = {st.C[q][0] + T * vt.v[v].bg[0], st.C[q][1] + T * vt.v[v].bg[1], st.C[q][2] + T * vt.v[v].bg[2]};
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) color[o + i + ch * HW] = c[ch];
-    if (Tout) Tout[pix + i] = T;
-    if (ncontrib) ncontrib[pix + i] = i == 0 ? st.last0 : st.last1;
+    for (int ch = 0; ch < 3; ++ch) color[o + at + ch * HW] = c[ch];
+    if (Tout) Tout[pix + at] = T;
+    if (ncontrib) ncontrib[pix + at] = st.last[q];
     if (with_target) {
       // the per-pixel L1 term and its gradient, as beta_l1_loss computes them
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
-        const float d = c[ch] - tgt[ch][2 * tid + i];
+        const float d = c[ch] - tgt[ch][2 * NP * tid + q];
         l1 += fabsf(d);
         const float gd = d > 0.0f ? scale : (d < 0.0f ? -scale : 0.0f);
-        gv[3 * i + ch] = gd;
-        if (dLdC) dLdC[o + i + ch * HW] = gd;
+        gv[3 * q + ch] = gd;
+        if (dLdC) dLdC[o + at + ch * HW] = gd;
       }
     }
   }
   return l1;
+}
+
+// Column x and row y of the lane's first pixel, and which of its pixels (x + h,
+// y + i) lie inside the view.
+template <int TW, int TH, int NP>
+__device__ __forceinline__ void lane_pixels(const ViewDev& V, int tx, int ty, int& bx, int& by, int& x, int& y,
+                                            bool (&in)[2 * NP]) {
+  using PB = PairBlock<TW, TH, NP>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bx = tx * TW + (warp % PB::WX) * PB::BW;
+  by = ty * TH + (warp / PB::WX) * PB::BH;
+  x = bx + 2 * (lane % PB::PC);
+  y = by + NP * (lane / PB::PC);
+#pragma unroll
+  for (int q = 0; q < 2 * NP; ++q) in[q] = x + (q & 1) < V.width && y + q / 2 < V.height;
+}
+
+// Starts the copies of the lane's target values into shared memory.
+template <int NT, int NP>
+__device__ __forceinline__ void copy_targets(const ViewDev& V, const float* __restrict__ target, int x, int y,
+                                             const bool (&in)[2 * NP], float (&tgt)[3][2 * NP * NT]) {
+  const int64_t HW = (int64_t)V.width * V.height;
+  const int64_t o = 3 * V.pix_off + (int64_t)y * V.width + x;
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch)
+#pragma unroll
+    for (int q = 0; q < 2 * NP; ++q)
+      if (in[q])
+        cp_async4(&tgt[ch][2 * NP * threadIdx.x + q], target + o + (int64_t)(q / 2) * V.width + (q & 1) + ch * HW);
 }
 
 // The CTA's sum of the lanes' l1 in a fixed order (warp shuffles, then the
@@ -1055,143 +1133,142 @@ __device__ __forceinline__ void tile_l1_partial(float l1, float (&s_l1)[NW], flo
   __syncthreads();
 }
 
-template <int TW, int TH, int S, bool PERSIST>
-__global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_threads_per_sm(S))) k_raster_fwd2(
+template <int TW, int TH, int S, int NP, bool PERSIST>
+__global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_fwd2(
     ViewTable vt, RenderOpts ro, const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
     const uint32_t* __restrict__ ranges, float* __restrict__ color, float* __restrict__ Tout,
     uint32_t* __restrict__ ncontrib, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const float* __restrict__ target, float* __restrict__ dLdC,
     float* __restrict__ l1_partial, uint32_t* __restrict__ hm, size_t hm_words) {
-  using PB = PairBlock<TW>;
-  constexpr int NT = TW * TH / 2, NW = NT / 32;
+  using PB = PairBlock<TW, TH, NP>;
+  constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ float s_l1[NW];
-  __shared__ float s_tgt[3][2 * NT];   // the pixels' targets, copied in while the tile composites
+  __shared__ float s_tgt[3][2 * NP * NT];   // the pixels' targets, copied in while the tile composites
   __shared__ int s_item;
   if (*status != 0) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float t_eps = ro.t_eps, amax = ro.alpha_max;
   for (int iter = 0;; ++iter) {
     const int g = next_tile<PERSIST>(iter, vt.total_tiles, ctr, order, &s_item);
     if (g < 0) break;
     const int v = view_of_tile(vt, g);
-    const int W = vt.v[v].width, H = vt.v[v].height;
-    int tx, ty;
+    int tx, ty, bx, by, x, y;
+    bool in[2 * NP];
     tile_xy(vt.v[v], g, tx, ty);
-    const int bx = tx * TW + (warp % PB::WX) * PB::BW, by = ty * TH + (warp / PB::WX) * PB::BH;
-    const int x = bx + 2 * (lane % PB::PC), y = by + lane / PB::PC;   // pixels (x, y), (x + 1, y)
-    const bool in0 = x < W && y < H, in1 = x + 1 < W && y < H;
+    lane_pixels<TW, TH, NP>(vt.v[v], tx, ty, bx, by, x, y, in);
     const uint32_t start = ranges[g], end = ranges[g + 1];
     uint32_t* const hslot = hit_tile<NT>(hm, hm_words, start, end, g);
-    if (target) {
-      const int64_t HW = (int64_t)W * H;
-      const int64_t o = 3 * vt.v[v].pix_off + (int64_t)y * W + x;
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        if (in0) cp_async4(&s_tgt[ch][2 * tid], target + o + ch * HW);
-        if (in1) cp_async4(&s_tgt[ch][2 * tid + 1], target + o + 1 + ch * HW);
-      }
-    }
-    PairFwdState fs;
-    pair_fwd_walk<TW, TH, S>(s_rec, nullptr, rec, vals, start, end, hslot, INT_MAX, (float)x, (float)y, (float)bx,
-                             (float)by, in0, in1, t_eps, amax, fs);
-    float gv[6];
-    const float l1 = pair_fwd_out<NT>(fs, vt, v, x, y, in0, in1, target != nullptr, s_tgt, color, Tout, ncontrib,
-                                      dLdC, gv);
+    if (target) copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
+    PairFwdState<NP> fs;
+    pair_fwd_walk<TW, TH, S, NP>(s_rec, nullptr, rec, vals, start, end, hslot, INT_MAX, (float)x, (float)y, (float)bx,
+                             (float)by, in, t_eps, amax, fs);
+    float gv[6 * NP];
+    const float l1 =
+        pair_fwd_out<NT, NP>(fs, vt, v, x, y, in, target != nullptr, s_tgt, color, Tout, ncontrib, dLdC, gv);
     // tile partial sum of |C - target|, reduced in a fixed order
     if (target) tile_l1_partial<NW>(l1, s_l1, l1_partial + g);
   }
   leave<PERSIST>(ctr);
 }
 
-// The lane's two pixels' terms (bwd_terms with ZERO) of a staged record, summed
-// over the two into G; T2 and NG2 (the suffix colour term g . S, negated) move
-// on at the pixels where `pos` holds and the record covers the pixel.  There
-// alpha takes its value, elsewhere zero, so that 1 / (1 - alpha) = 1 leaves T
-// and a zero weight leaves NG2 and the colour terms (with a non-finite colour,
-// `odd`, g . c is dropped there).  Returns whether either pixel is covered.
-__device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x2 x2, float yf, float amax, bool odd,
-                                           bool pos0, bool pos1, f32x2 gx, f32x2 gy, f32x2 gz, f32x2& T2, f32x2& NG2,
-                                           float G[kGrad2d]) {
-  f32x2 u, v;
-  const f32x2 om = rec_om_pair(f0, f1, x2, yf, u, v);
-  float b0, b1, e0, e1, d0, d1, t0, t1;
-  unpack2(om, b0, b1);
-  const bool act0 = pos0 && b0 > 0.0f, act1 = pos1 && b1 > 0.0f;
-  b0 = fmaxf(b0, 5.9604645e-8f);   // 1 - r^2 >= 2^-24 wherever r^2 < 1
-  b1 = fmaxf(b1, 5.9604645e-8f);
-  const f32x2 lb = pack2(lg2_approx(b0), lg2_approx(b1));
-  unpack2(fma2(both2(f1.w), lb, both2(f2.x)), e0, e1);
-  const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);   // the forward's alpha
-  const f32x2 a2 = pack2(act0 ? fminf(p0, amax) : 0.0f, act1 ? fminf(p1, amax) : 0.0f);
-  unpack2(fma2(a2, both2(-1.0f), both2(1.0f)), d0, d1);
-  const f32x2 inv = pack2(rcp_approx(d0), rcp_approx(d1));
-  f32x2 gc = fma2(gx, both2(f2.y), fma2(gy, both2(f2.z), mul2(gz, both2(f2.w))));
-  if (odd) {
-    float c0, c1;
-    unpack2(gc, c0, c1);
-    gc = pack2(act0 ? c0 : 0.0f, act1 ? c1 : 0.0f);
-  }
-  const f32x2 dLa = mul2(fma2(T2, gc, NG2), inv);
-  T2 = mul2(T2, inv);
-  const f32x2 wgt = mul2(a2, T2);
-  unpack2(mul2(dLa, pack2(p0, p1)), t0, t1);
-  const f32x2 t = pack2(act0 && p0 < amax ? t0 : 0.0f,    // clamped alpha: no o/beta/r^2 gradient
-                        act1 && p1 < amax ? t1 : 0.0f);
-  const f32x2 kk = mul2(t, pack2(rcp_approx(b0), rcp_approx(b1)));
-  const f32x2 h0 = mul2(kk, u), h1 = mul2(kk, v);
-  G[0] = sum2(h0);
-  G[1] = sum2(h1);
-  G[2] = sum2(mul2(h0, u));
-  G[3] = sum2(mul2(h0, v));
-  G[4] = sum2(mul2(h1, v));
-  G[5] = sum2(t);
-  G[6] = sum2(mul2(t, lb));
-  G[7] = sum2(mul2(wgt, gx));
-  G[8] = sum2(mul2(wgt, gy));
-  G[9] = sum2(mul2(wgt, gz));
-  NG2 = fma2(mul2(wgt, both2(-1.0f)), gc, NG2);
-  return act0 || act1;
-}
-
-// Per-lane state the pixel-pair backward starts from: final transmittance,
-// the suffix colour term g . S (the background's, T bg . g), dL/dC and the
-// last-contributor position of the lane's two pixels (zeros off the image).
+// Per-lane state of the pixel-pair backward: transmittance, the suffix colour
+// term g . S, negated (at the start the background's, -T bg . g), dL/dC and the
+// last-contributor positions of the lane's pixels (zeros off the image).
+template <int NP>
 struct PairBwdState {
-  float T0, T1, GS0, GS1, g0x, g0y, g0z, g1x, g1y, g1z;
-  uint32_t nl0, nl1;
+  f32x2 T2[NP], NG2[NP], gx[NP], gy[NP], gz[NP];
+  uint32_t nl[2 * NP];
   int odd_colours;   // 1 / 0: some / none of the records has a non-finite colour; -1: not known
 };
 
-// Reverse walk of one tile's list lst at the lane's pixel pair, from the CTA's
+// The lane's pixels' terms (bwd_terms with ZERO) of a staged record, summed over
+// them into G; T2 and NG2 move on at the pixels where the record lies before the
+// last contributor (pos < nl, and `mine`) and covers the pixel.  There alpha
+// takes its value, elsewhere zero, so that 1 / (1 - alpha) = 1 leaves T and a
+// zero weight leaves NG2 and the colour terms (with a non-finite colour, `odd`,
+// g . c is dropped there).  Returns whether any pixel is covered.
+template <int NP>
+__device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x2 x2, float yf, float amax, bool odd,
+                                           bool mine, uint32_t pos, PairBwdState<NP>& st, float G[kGrad2d]) {
+  f32x2 dx, u, H[kGrad2d];
+  rec_cols(f0, f1, x2, dx, u);
+  bool any = false;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    f32x2 v;
+    const f32x2 om = rec_om(f0, f1, dx, u, i == 0 ? yf : yf + (float)i, v);
+    float b0, b1, e0, e1, d0, d1, t0, t1;
+    unpack2(om, b0, b1);
+    const bool act0 = mine && pos < st.nl[2 * i] && b0 > 0.0f, act1 = mine && pos < st.nl[2 * i + 1] && b1 > 0.0f;
+    any = any || act0 || act1;
+    b0 = fmaxf(b0, 5.9604645e-8f);   // 1 - r^2 >= 2^-24 wherever r^2 < 1
+    b1 = fmaxf(b1, 5.9604645e-8f);
+    const f32x2 lb = pack2(lg2_approx(b0), lg2_approx(b1));
+    unpack2(fma2(both2(f1.w), lb, both2(f2.x)), e0, e1);
+    const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);   // the forward's alpha
+    const f32x2 a2 = pack2(act0 ? fminf(p0, amax) : 0.0f, act1 ? fminf(p1, amax) : 0.0f);
+    unpack2(fma2(a2, both2(-1.0f), both2(1.0f)), d0, d1);
+    const f32x2 inv = pack2(rcp_approx(d0), rcp_approx(d1));
+    f32x2 gc = fma2(st.gx[i], both2(f2.y), fma2(st.gy[i], both2(f2.z), mul2(st.gz[i], both2(f2.w))));
+    if (odd) {
+      float c0, c1;
+      unpack2(gc, c0, c1);
+      gc = pack2(act0 ? c0 : 0.0f, act1 ? c1 : 0.0f);
+    }
+    const f32x2 dLa = mul2(fma2(st.T2[i], gc, st.NG2[i]), inv);
+    st.T2[i] = mul2(st.T2[i], inv);
+    const f32x2 wgt = mul2(a2, st.T2[i]);
+    unpack2(mul2(dLa, pack2(p0, p1)), t0, t1);
+    const f32x2 t = pack2(act0 && p0 < amax ? t0 : 0.0f,    // clamped alpha: no o/beta/r^2 gradient
+                          act1 && p1 < amax ? t1 : 0.0f);
+    const f32x2 kk = mul2(t, pack2(rcp_approx(b0), rcp_approx(b1)));
+    const f32x2 h0 = mul2(kk, u), h1 = mul2(kk, v);
+    auto acc = [&](int q, f32x2 a, f32x2 b) { H[q] = i == 0 ? mul2(a, b) : fma2(a, b, H[q]); };
+    H[0] = i == 0 ? h0 : add2(H[0], h0);
+    H[1] = i == 0 ? h1 : add2(H[1], h1);
+    acc(2, h0, u);
+    acc(3, h0, v);
+    acc(4, h1, v);
+    H[5] = i == 0 ? t : add2(H[5], t);
+    acc(6, t, lb);
+    acc(7, wgt, st.gx[i]);
+    acc(8, wgt, st.gy[i]);
+    acc(9, wgt, st.gz[i]);
+    st.NG2[i] = fma2(mul2(wgt, both2(-1.0f)), gc, st.NG2[i]);
+  }
+#pragma unroll
+  for (int q = 0; q < kGrad2d; ++q) G[q] = sum2(H[q]);
+  return any;
+}
+
+// Reverse walk of one tile's list lst at the lane's pixel pairs, from the CTA's
 // largest last-contributor position down: batches of S records staged as the
 // forward staged them (so chunks start at multiples of 32), the list entries
 // of the next batch down loaded one batch ahead; per chunk the cover masks
 // (the forward's from hslot for the list's first hm_chunks chunks, else the
 // cover pass again), then every lane's
-// walk of its records in reverse list order at both pixels with three vector
+// walk of its records in reverse list order at its pixels with three vector
 // atomics per record, and records covering more than kLaneAtomics of the
-// warp's pairs by the whole warp (reduce-scatter, one atomic per value).
+// warp's lanes by the whole warp (reduce-scatter, one atomic per value).
 // When the first batch it needs is reuse_batch, which a forward walk left
 // complete in s_rec[reuse_buf] with its indices in s_ridx[reuse_buf], it
 // starts from there instead of staging it again (reuse_batch = -1: never).
 // Returns with every copy landed and the CTA synchronised.
-template <int TW, int TH, int S>
+template <int TW, int TH, int S, int NP>
 __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], uint32_t (&s_ridx)[2][S],
-                                              uint32_t (&s_wmax)[TW * TH / 64], const float4* __restrict__ rec,
-                                              const uint32_t* __restrict__ lst, const uint32_t* hslot,
-                                              int hm_chunks, float* __restrict__ grad2d, float xf, float yf,
-                                              float bxf, float byf, float amax, int my_field,
-                                              const PairBwdState& st, int reuse_batch, int reuse_buf) {
-  using PB = PairBlock<TW>;
-  constexpr int NT = TW * TH / 2, NW = NT / 32, RPT = (S + NT - 1) / NT;
+                                              uint32_t (&s_wmax)[PairBlock<TW, TH, NP>::NW],
+                                              const float4* __restrict__ rec, const uint32_t* __restrict__ lst,
+                                              const uint32_t* hslot, int hm_chunks, float* __restrict__ grad2d,
+                                              float xf, float yf, float bxf, float byf, float amax, int my_field,
+                                              PairBwdState<NP>& st, int reuse_batch, int reuse_buf) {
+  using PB = PairBlock<TW, TH, NP>;
+  constexpr int NT = PB::NT, NW = PB::NW, RPT = (S + NT - 1) / NT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  f32x2 T2 = pack2(st.T0, st.T1), NG2 = pack2(-st.GS0, -st.GS1);
-  const f32x2 gx = pack2(st.g0x, st.g1x), gy = pack2(st.g0y, st.g1y), gz = pack2(st.g0z, st.g1z);
   const f32x2 x2 = pack2(xf, xf + 1.0f);
-  const uint32_t nl0 = st.nl0, nl1 = st.nl1;
-  const uint32_t nlm = max(nl0, nl1);
+  uint32_t nlm = 0;
+#pragma unroll
+  for (int q = 0; q < 2 * NP; ++q) nlm = max(nlm, st.nl[q]);
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, nlm);
   if (lane == 0) s_wmax[warp] = wmax;
   __syncthreads();
@@ -1263,8 +1340,8 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
       } else {
         const int idx = c + lane;
         const uint32_t cov = (idx < cnt && (uint32_t)(lo + idx) < wmax)
-                                 ? pair_cover<PB::BW>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf) : 0u;
-        wide = __ballot_sync(0xffffffffu, __popc(cov) > kLaneAtomics);
+                                 ? pair_cover<PB::BW, NP>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf) : 0u;
+        wide = __ballot_sync(0xffffffffu, __popc(cov) > PB::kWide);
         mine = transpose32(cov, lane);
       }
       if (hslot && j >= 1 && j - 1 < hm_chunks) {     // the next chunk's stored masks, one chunk ahead
@@ -1292,8 +1369,7 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
           const int s = c + k;
           const uint32_t pos = (uint32_t)(lo + s);
           float G[kGrad2d];
-          if (!pair_terms(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, pos < nl0, pos < nl1,
-                          gx, gy, gz, T2, NG2, G))
+          if (!pair_terms<NP>(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, true, pos, st, G))
             continue;                                 // outside the support (the cover is conservative)
           float* gdst = grad2d + (size_t)s_ridx[buf][s] * kGrad2dStride;
           red_add_v4(gdst + 0, G[0], G[1], G[2], G[3]);
@@ -1307,8 +1383,7 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         const int s = c + kb;
         const uint32_t pos = (uint32_t)(lo + s);
         float G[kGrad2d];                              // zero where a pixel is not covered
-        pair_terms(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, mine_kb && pos < nl0,
-                   mine_kb && pos < nl1, gx, gy, gz, T2, NG2, G);
+        pair_terms<NP>(s_rec[buf][s][0], s_rec[buf][s][1], s_rec[buf][s][2], x2, yf, amax, odd, mine_kb, pos, st, G);
         const float tot = warp_sum10(G, lane);
         float* gdst = grad2d + (size_t)s_ridx[buf][s] * kGrad2dStride;
         if (my_field >= 0 && tot != 0.0f) atomicAdd(gdst + my_field, tot);
@@ -1320,60 +1395,64 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
   __syncthreads();
 }
 
-template <int TW, int TH, int S, bool PERSIST>
-__global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_threads_per_sm(S))) k_raster_bwd2(
+template <int TW, int TH, int S, int NP, bool PERSIST>
+__global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_bwd2(
     ViewTable vt, RenderOpts ro, const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
     const uint32_t* __restrict__ ranges, const float* __restrict__ Tfin, const uint32_t* __restrict__ ncontrib,
     const float* __restrict__ dLdC, float* __restrict__ grad2d, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const uint32_t* __restrict__ hm, size_t hm_words) {
-  using PB = PairBlock<TW>;
-  constexpr int NT = TW * TH / 2, NW = NT / 32;
+  using PB = PairBlock<TW, TH, NP>;
+  constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ uint32_t s_ridx[2][S];
   __shared__ uint32_t s_wmax[NW];
   __shared__ int s_item;
   if (*status != 0) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x & 31;
   const float amax = ro.alpha_max;
   const int my_field = warp_sum10_field(lane);
   for (int iter = 0;; ++iter) {
     const int g = next_tile<PERSIST>(iter, vt.total_tiles, ctr, order, &s_item);
     if (g < 0) break;
     const int v = view_of_tile(vt, g);
-    const int W = vt.v[v].width, H = vt.v[v].height;
-    int tx, ty;
+    int tx, ty, bx, by, x, y;
+    bool in[2 * NP];
     tile_xy(vt.v[v], g, tx, ty);
-    const int bx = tx * TW + (warp % PB::WX) * PB::BW, by = ty * TH + (warp / PB::WX) * PB::BH;
-    const int x = bx + 2 * (lane % PB::PC), y = by + lane / PB::PC;   // pixels (x, y), (x + 1, y)
-    const bool in0 = x < W && y < H, in1 = x + 1 < W && y < H;
+    lane_pixels<TW, TH, NP>(vt.v[v], tx, ty, bx, by, x, y, in);
     const uint32_t range0 = ranges[g];
     const uint32_t* const hslot = hit_tile<NT>(const_cast<uint32_t*>(hm), hm_words, range0, ranges[g + 1], g);
 
-    PairBwdState bs{1.0f, 1.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0u, 0u, -1};
+    PairBwdState<NP> bs;
+    bs.odd_colours = -1;
     {
-      const int64_t HW = (int64_t)W * H;
+      const int W = vt.v[v].width;
+      const int64_t HW = (int64_t)W * vt.v[v].height;
       const int64_t pix = vt.v[v].pix_off + (int64_t)y * W + x;
       const float* gb = dLdC + 3 * vt.v[v].pix_off + (int64_t)y * W + x;
       const float* bg = vt.v[v].bg;
-      if (in0) {
-        bs.g0x = gb[0];
-        bs.g0y = gb[HW];
-        bs.g0z = gb[2 * HW];
-        bs.T0 = Tfin[pix];
-        bs.nl0 = ncontrib[pix];
-        bs.GS0 = bs.T0 * (bs.g0x * bg[0] + bs.g0y * bg[1] + bs.g0z * bg[2]);
-      }
-      if (in1) {
-        bs.g1x = gb[1];
-        bs.g1y = gb[HW + 1];
-        bs.g1z = gb[2 * HW + 1];
-        bs.T1 = Tfin[pix + 1];
-        bs.nl1 = ncontrib[pix + 1];
-        bs.GS1 = bs.T1 * (bs.g1x * bg[0] + bs.g1y * bg[1] + bs.g1z * bg[2]);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        float T[2], gx[2], gy[2], gz[2], ng[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int64_t at = (int64_t)i * W + h;
+          const bool inside = in[2 * i + h];
+          T[h] = inside ? Tfin[pix + at] : 1.0f;
+          gx[h] = inside ? gb[at] : 0.0f;
+          gy[h] = inside ? gb[HW + at] : 0.0f;
+          gz[h] = inside ? gb[2 * HW + at] : 0.0f;
+          bs.nl[2 * i + h] = inside ? ncontrib[pix + at] : 0u;
+          ng[h] = inside ? -(T[h] * (gx[h] * bg[0] + gy[h] * bg[1] + gz[h] * bg[2])) : 0.0f;
+        }
+        bs.T2[i] = pack2(T[0], T[1]);
+        bs.NG2[i] = pack2(ng[0], ng[1]);
+        bs.gx[i] = pack2(gx[0], gx[1]);
+        bs.gy[i] = pack2(gy[0], gy[1]);
+        bs.gz[i] = pack2(gz[0], gz[1]);
       }
     }
-    pair_bwd_walk<TW, TH, S>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX, grad2d, (float)x, (float)y,
+    pair_bwd_walk<TW, TH, S, NP>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX, grad2d, (float)x, (float)y,
                              (float)bx, (float)by, amax, my_field, bs, -1, 0);
   }
   leave<PERSIST>(ctr);
@@ -1392,75 +1471,68 @@ __global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_thre
 // equal k_raster_fwd2's bit for bit, and every per-record term the backward
 // adds equals k_raster_bwd2's (the sums differ only by the order of the
 // floating-point atomics).
-constexpr int kStepMaskChunks(int nt) { return nt >= 384 ? 1 : 384 / nt; }
+constexpr int kStepMaskChunks(int nt) { return nt >= 384 ? 1 : 384 / nt < 6 ? 384 / nt : 6; }
 
-template <int TW, int TH, int S, bool PERSIST>
-__global__ void __launch_bounds__(TW * TH / 2, min_blocks(TW * TH / 2, pair_threads_per_sm(S))) k_raster_step2(
+template <int TW, int TH, int S, int NP, bool PERSIST>
+__global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_step2(
     ViewTable vt, RenderOpts ro, const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
     const uint32_t* __restrict__ ranges, float* __restrict__ color, float* __restrict__ Tout,
     uint32_t* __restrict__ ncontrib, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const float* __restrict__ target, float* __restrict__ dLdC,
     float* __restrict__ l1_partial, float* __restrict__ grad2d) {
-  using PB = PairBlock<TW>;
-  constexpr int NT = TW * TH / 2, NW = NT / 32;
+  using PB = PairBlock<TW, TH, NP>;
+  constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ uint32_t s_ridx[2][S];
   __shared__ float s_l1[NW];
-  __shared__ float s_tgt[3][2 * NT];   // the pixels' targets, copied in while the tile composites
+  __shared__ float s_tgt[3][2 * NP * NT];   // the pixels' targets, copied in while the tile composites
   __shared__ uint32_t s_wmax[NW];
   __shared__ uint32_t s_hm[kStepMaskChunks(NT) * (NT + NW)];   // cover masks, hit-mask slot layout
   __shared__ int s_item;
   if (*status != 0) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x & 31;
   const float t_eps = ro.t_eps, amax = ro.alpha_max;
   const int my_field = warp_sum10_field(lane);
   for (int iter = 0;; ++iter) {
     const int g = next_tile<PERSIST>(iter, vt.total_tiles, ctr, order, &s_item);
     if (g < 0) break;
     const int v = view_of_tile(vt, g);
-    const int W = vt.v[v].width, H = vt.v[v].height;
-    int tx, ty;
+    int tx, ty, bx, by, x, y;
+    bool in[2 * NP];
     tile_xy(vt.v[v], g, tx, ty);
-    const int bx = tx * TW + (warp % PB::WX) * PB::BW, by = ty * TH + (warp / PB::WX) * PB::BH;
-    const int x = bx + 2 * (lane % PB::PC), y = by + lane / PB::PC;   // pixels (x, y), (x + 1, y)
-    const bool in0 = x < W && y < H, in1 = x + 1 < W && y < H;
+    lane_pixels<TW, TH, NP>(vt.v[v], tx, ty, bx, by, x, y, in);
     const float xf = (float)x, yf = (float)y, bxf = (float)bx, byf = (float)by;
     const uint32_t start = ranges[g], end = ranges[g + 1];
-    {
-      const int64_t HW = (int64_t)W * H;
-      const int64_t o = 3 * vt.v[v].pix_off + (int64_t)y * W + x;
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        if (in0) cp_async4(&s_tgt[ch][2 * tid], target + o + ch * HW);
-        if (in1) cp_async4(&s_tgt[ch][2 * tid + 1], target + o + 1 + ch * HW);
-      }
-    }
-    PairFwdState fs;
-    pair_fwd_walk<TW, TH, S>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
-                             byf, in0, in1, t_eps, amax, fs);
-    float gv[6];
-    const float l1 = pair_fwd_out<NT>(fs, vt, v, x, y, in0, in1, true, s_tgt, color, Tout, ncontrib, dLdC, gv);
+    copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
+    PairFwdState<NP> fs;
+    pair_fwd_walk<TW, TH, S, NP>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
+                             byf, in, t_eps, amax, fs);
+    float gv[6 * NP];
+    const float l1 = pair_fwd_out<NT, NP>(fs, vt, v, x, y, in, true, s_tgt, color, Tout, ncontrib, dLdC, gv);
     // also the barrier after which no warp still reads the forward's s_rec
     // and every cover mask in s_hm is visible to the whole CTA
     tile_l1_partial<NW>(l1, s_l1, l1_partial + g);
 
     const float* bg = vt.v[v].bg;
-    PairBwdState bs;
-    bs.T0 = fs.T0;
-    bs.T1 = fs.T1;
-    bs.g0x = gv[0];
-    bs.g0y = gv[1];
-    bs.g0z = gv[2];
-    bs.g1x = gv[3];
-    bs.g1y = gv[4];
-    bs.g1z = gv[5];
-    bs.nl0 = fs.last0;
-    bs.nl1 = fs.last1;
+    PairBwdState<NP> bs;
     bs.odd_colours = fs.odd_colours ? 1 : 0;
-    bs.GS0 = in0 ? bs.T0 * (bs.g0x * bg[0] + bs.g0y * bg[1] + bs.g0z * bg[2]) : 0.0f;
-    bs.GS1 = in1 ? bs.T1 * (bs.g1x * bg[0] + bs.g1y * bg[1] + bs.g1z * bg[2]) : 0.0f;
-    pair_bwd_walk<TW, TH, S>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      float ng[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float* gp = gv + 3 * (2 * i + h);
+        ng[h] = in[2 * i + h] ? -(fs.T[2 * i + h] * (gp[0] * bg[0] + gp[1] * bg[1] + gp[2] * bg[2])) : 0.0f;
+        bs.nl[2 * i + h] = fs.last[2 * i + h];
+      }
+      bs.T2[i] = pack2(fs.T[2 * i], fs.T[2 * i + 1]);
+      bs.NG2[i] = pack2(ng[0], ng[1]);
+      bs.gx[i] = pack2(gv[6 * i], gv[6 * i + 3]);
+      bs.gy[i] = pack2(gv[6 * i + 1], gv[6 * i + 4]);
+      bs.gz[i] = pack2(gv[6 * i + 2], gv[6 * i + 5]);
+    }
+    pair_bwd_walk<TW, TH, S, NP>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,
                              bxf, byf, amax, my_field, bs, fs.walked_batch, fs.walked_buf);
   }
   leave<PERSIST>(ctr);
@@ -1615,23 +1687,34 @@ int persistent_grid(K kernel, int threads, int total_tiles) {
   return std::max(1, std::min(total_tiles, per_sm * device_sm_count()));
 }
 
+template <int TW, int TH, int S, int NP>
+cudaError_t fwd_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* rec,
+                      const uint32_t* vals, const uint32_t* ranges, float* color, float* T_final,
+                      uint32_t* n_contrib, const int32_t* status, uint32_t* sched, const float* target,
+                      float* dL_dcolor, float* l1_partial, HitMasks hm, cudaStream_t s) {
+  constexpr int NT = PairBlock<TW, TH, NP>::NT;
+  if (sched) {
+    auto k = k_raster_fwd2<TW, TH, S, NP, true>;
+    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
+        target, dL_dcolor, l1_partial, hm.words, hm.n_words);
+  } else {
+    k_raster_fwd2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
+        l1_partial, hm.words, hm.n_words);
+  }
+  return cudaGetLastError();
+}
+
 template <int TW, int TH, int S>
 cudaError_t fwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* rec,
                       const uint32_t* vals, const uint32_t* ranges, float* color, float* T_final,
                       uint32_t* n_contrib, const int32_t* status, uint32_t* sched, const float* target,
                       float* dL_dcolor, float* l1_partial, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    constexpr int NT = TW * TH / 2;
-    if (sched) {
-      auto k = k_raster_fwd2<TW, TH, S, true>;
-      k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
-          target, dL_dcolor, l1_partial, hm.words, hm.n_words);
-    } else {
-      k_raster_fwd2<TW, TH, S, false><<<vt.total_tiles, NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
-          l1_partial, hm.words, hm.n_words);
-    }
+    if constexpr (quad_shape(TW, TH, S))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return fwd_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
+    return fwd_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
   } else {
     if (sched) {
       auto k = k_raster_fwd<TW, TH, S, true>;
@@ -1647,23 +1730,34 @@ cudaError_t fwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
   return cudaGetLastError();
 }
 
+template <int TW, int TH, int S, int NP>
+cudaError_t bwd_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* rec,
+                      const uint32_t* vals, const uint32_t* ranges, const float* T_final,
+                      const uint32_t* n_contrib, const float* dL_dcolor, float* grad2d,
+                      const int32_t* status, uint32_t* sched, HitMasks hm, cudaStream_t s) {
+  constexpr int NT = PairBlock<TW, TH, NP>::NT;
+  if (sched) {
+    auto k = k_raster_bwd2<TW, TH, S, NP, true>;
+    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
+        sched + kSchedOrder, hm.words, hm.n_words);
+  } else {
+    k_raster_bwd2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
+        hm.words, hm.n_words);
+  }
+  return cudaGetLastError();
+}
+
 template <int TW, int TH, int S>
 cudaError_t bwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* rec,
                       const uint32_t* vals, const uint32_t* ranges, const float* T_final,
                       const uint32_t* n_contrib, const float* dL_dcolor, float* grad2d,
                       const int32_t* status, uint32_t* sched, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    constexpr int NT = TW * TH / 2;
-    if (sched) {
-      auto k = k_raster_bwd2<TW, TH, S, true>;
-      k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
-          sched + kSchedOrder, hm.words, hm.n_words);
-    } else {
-      k_raster_bwd2<TW, TH, S, false><<<vt.total_tiles, NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
-          hm.words, hm.n_words);
-    }
+    if constexpr (quad_shape(TW, TH, S))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return bwd_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
+    return bwd_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
   } else {
     if (sched) {
       auto k = k_raster_bwd<TW, TH, S, true>;
@@ -1680,24 +1774,34 @@ cudaError_t bwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
 }
 
 // Forward + L1 + backward in one launch (pixel-pair tilings only).
+template <int TW, int TH, int S, int NP>
+cudaError_t step_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* rec, const uint32_t* vals,
+                       const uint32_t* ranges, float* color, float* T_final, uint32_t* n_contrib,
+                       const int32_t* status, uint32_t* sched, const float* target, float* dL_dcolor,
+                       float* l1_partial, float* grad2d, cudaStream_t s) {
+  constexpr int NT = PairBlock<TW, TH, NP>::NT;
+  if (sched) {
+    auto k = k_raster_step2<TW, TH, S, NP, true>;
+    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder, target,
+        dL_dcolor, l1_partial, grad2d);
+  } else {
+    k_raster_step2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
+        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
+        l1_partial, grad2d);
+  }
+  return cudaGetLastError();
+}
+
 template <int TW, int TH, int S>
 cudaError_t step_shape(const ViewTable& vt, const RenderOpts& ro, const float4* rec, const uint32_t* vals,
                        const uint32_t* ranges, float* color, float* T_final, uint32_t* n_contrib,
                        const int32_t* status, uint32_t* sched, const float* target, float* dL_dcolor,
                        float* l1_partial, float* grad2d, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    constexpr int NT = TW * TH / 2;
-    if (sched) {
-      auto k = k_raster_step2<TW, TH, S, true>;
-      k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder, target,
-          dL_dcolor, l1_partial, grad2d);
-    } else {
-      k_raster_step2<TW, TH, S, false><<<vt.total_tiles, NT, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
-          l1_partial, grad2d);
-    }
-    return cudaGetLastError();
+    if constexpr (quad_shape(TW, TH, S))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return step_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
+    return step_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
   } else {
     return cudaErrorInvalidValue;   // 8 x 4 tiles have no pixel-pair kernels
   }
@@ -1746,7 +1850,7 @@ cudaError_t launch_raster_fwd(const ViewTable& vt, const RenderOpts& ro, const f
 size_t hit_mask_bytes(const ViewTable& vt, const RenderOpts& ro, int64_t cap) {
   // one word per lane (per pixel pair in the pixel-pair kernels) and one per warp
   const bool pairs = pair_tiles(ro.tile_w, ro.tile_h);
-  const int64_t nt = (int64_t)ro.tile_w * ro.tile_h / (pairs ? 2 : 1);
+  const int64_t nt = (int64_t)ro.tile_w * ro.tile_h / (pairs ? 2 * lane_pairs(ro, vt.total_tiles) : 1);
   const int64_t slots = (std::max<int64_t>(cap, 0) >> 5) + vt.total_tiles + 1;
   return (size_t)slots * (size_t)(nt + nt / 32) * sizeof(uint32_t);
 }

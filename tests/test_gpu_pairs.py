@@ -26,6 +26,10 @@ def _scene(odd):
     return planes
 
 
+def _odd_index():
+    return int(np.argsort(_scene(False)[2, :60])[20])
+
+
 def _run(planes_np, cam, tile, s, fused):
     gc.ensure_built()
     planes = torch.from_numpy(planes_np).cuda()
@@ -61,3 +65,57 @@ def test_pair_kernels_equal_one_pixel_kernels(odd, tile, s, fused, w, h):
     # each sum off by at most ~sqrt(terms) roundings of its largest partial sums
     scale = np.max(np.abs(np.where(fin, g0, 0.0)), axis=1, keepdims=True) + 1e-30
     assert np.max(np.abs(np.where(fin, g1 - g0, 0.0)) / scale) < 1e-4
+
+
+@pytest.mark.parametrize("odd", [False, True])
+@pytest.mark.parametrize("tile,s,fused,persistent", [((16, 8), 64, True, False), ((16, 8), 64, False, True),
+                                                     ((16, 16), 64, True, True), ((16, 16), 128, False, False),
+                                                     ((32, 16), 64, False, False), ((32, 16), 128, True, False),
+                                                     ((32, 16), 256, True, True)])
+def test_quad_kernels_equal_one_pixel_kernels(odd, tile, s, fused, persistent):
+    """The same at an odd-sized view large enough for two pairs a lane; the split
+    path with hit masks."""
+    cam = scenes.pinhole(*scenes.look_at((0.0, 0.0, -3.0)), 2049, 1001)
+    assert -(-2049 // 16) * -(-1001 // 8) >= 16000
+    planes = _scene(odd)
+    c0, g0 = _run(planes, cam, (8, 4), 64, False)
+    gc.ensure_built()
+    p = torch.from_numpy(planes).cuda()
+    r = render.Rasterizer(60, p.shape[1], 1, [cam], _lib.default_opts(tile_w=tile[0], tile_h=tile[1], batch_s=s),
+                          persistent=persistent, hit_masks=True)
+    target = torch.from_numpy(scenes.target_images([cam], seed=3)[0].reshape(-1)).cuda()
+    r.forward(p)
+    grad = torch.zeros_like(p)
+    if fused:
+        r.raster_fwd_bwd_l1(p, target)
+    else:
+        r.raster_fwd_l1(p, target)
+        r.raster_bwd(p, r.dL_dcolor)
+    r.project_bwd(p, grad)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(r.color.cpu().numpy(), c0)
+    g1 = grad.cpu().numpy()
+    fin = np.isfinite(g0)
+    assert (np.isfinite(g1) == fin).all() and fin.any()
+    if odd:
+        # the infinite record's own lobe-direction gradients are 3e38 times sums that
+        # cancel (they differ between any two tilings): compared for finiteness only
+        g0[:, _odd_index()] = g1[:, _odd_index()] = 0.0
+    scale = np.max(np.abs(np.where(fin, g0, 0.0)), axis=1, keepdims=True) + 1e-30
+    with np.errstate(invalid="ignore"):
+        assert np.max(np.abs(np.where(fin, g1 - g0, 0.0)) / scale) < 1e-4
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_forward_grows_the_pair_buffers_behind_launched_rasters(persistent):
+    """An overflow found after the raster kernels were launched: they wrote
+    nothing, and the image after growing is that of large buffers."""
+    gc.ensure_built()
+    sc = scenes.config_scene(1)
+    planes = torch.from_numpy(sc.planes).cuda()
+    r0 = render.Rasterizer(sc.n, sc.pitch, sc.n_lobes, sc.cameras, persistent=persistent)
+    r1 = render.Rasterizer(sc.n, sc.pitch, sc.n_lobes, sc.cameras, persistent=persistent, pair_capacity=100)
+    want = r0.forward(planes).clone()
+    for _ in range(2):
+        assert torch.equal(r1.forward(planes), want)
+    assert r1.cap > 100 and r1.device_status() == (0, int(r0.count.item()))
