@@ -106,6 +106,27 @@ def test_quad_kernels_equal_one_pixel_kernels(odd, tile, s, fused, persistent):
         assert np.max(np.abs(np.where(fin, g1 - g0, 0.0)) / scale) < 1e-4
 
 
+@pytest.mark.parametrize("w,h,tile", [(1, 1, (8, 4)), (257, 129, (16, 16)), (1024, 512, (8, 4)), (1032, 512, (8, 4))])
+def test_schedule_orders_every_tile_longest_first(w, h, tile):
+    """One CTA up to 16384 tiles, three launches above: a permutation of the tiles
+    by descending bit length of their list."""
+    gc.ensure_built()
+    sc = scenes.config_scene(3, n=4000)
+    planes = torch.from_numpy(sc.planes).cuda()
+    r = render.Rasterizer(sc.n, sc.pitch, sc.n_lobes, [scenes.ring_camera(4.0, 15.0, 0.3, w, h)],
+                          _lib.default_opts(tile_w=tile[0], tile_h=tile[1], batch_s=64), persistent=True)
+    r.project(planes)
+    r.bin_sort(planes)
+    r.sched.fill_(-1)
+    r.schedule()
+    torch.cuda.synchronize()
+    sched, ranges = r.sched.cpu().numpy(), r.ranges.cpu().numpy().astype(np.int64)
+    order = sched[144:144 + r.total_tiles]
+    assert (sched[:4] == 0).all() and np.array_equal(np.sort(order), np.arange(r.total_tiles))
+    bits = np.array([int(n).bit_length() for n in np.diff(ranges)])[order]
+    assert (np.diff(bits) <= 0).all()
+
+
 @pytest.mark.parametrize("persistent", [False, True])
 def test_forward_grows_the_pair_buffers_behind_launched_rasters(persistent):
     """An overflow found after the raster kernels were launched: they wrote
