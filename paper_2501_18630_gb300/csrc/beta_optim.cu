@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(256, 4) k_adam(float* __restrict__ planes, con
                                               float* __restrict__ adam_m, float* __restrict__ adam_v,
                                               const float* __restrict__ eta, int n, int pitch, AdamDev a,
                                               double* __restrict__ reg) {
+  chain_begin();
   constexpr int NP = 15 + 6 * M;
   __shared__ double s_red[2][8];
   const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -192,7 +193,7 @@ cudaError_t launch_m(float* planes, const float* grad, float* m, float* v, const
                      int pitch, const AdamDev& a, double* reg, cudaStream_t s) {
   const int grid = ((n + 3) / 4 + 255) / 256;
   if (grid < 1) return cudaSuccess;
-  k_adam<M><<<grid, 256, 0, s>>>(planes, grad, m, v, eta, n, pitch, a, reg);
+  launch_chained(k_adam<M>, grid, 256, 0, s, planes, grad, m, v, eta, n, pitch, a, reg);
   return cudaGetLastError();
 }
 
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(kRelocBlock) k_reloc_weights(const float* __re
                                                                float* __restrict__ logit,
                                                                unsigned long long* __restrict__ bsum,
                                                                uint32_t* __restrict__ bdead) {
+  chain_begin();
   __shared__ unsigned long long s_w[8];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t wi = 0;
@@ -293,6 +295,7 @@ __global__ void __launch_bounds__(1024) k_reloc_scan(unsigned long long* __restr
                                                      const uint32_t* __restrict__ bdead, int nb,
                                                      unsigned long long* __restrict__ total,
                                                      int32_t* __restrict__ d_count) {
+  chain_begin();
   constexpr int kPer = 4;
   __shared__ unsigned long long s_w[32];
   __shared__ unsigned int s_d[32];
@@ -348,6 +351,7 @@ __global__ void __launch_bounds__(kRelocBlock) k_reloc_sample(const uint32_t* __
                                                               const uint32_t* __restrict__ rnd,
                                                               int32_t* __restrict__ src,
                                                               uint32_t* __restrict__ copies) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned long long T = *total;
@@ -409,6 +413,7 @@ __global__ void __launch_bounds__(256) k_reloc_copy(float* __restrict__ planes, 
                                                     const int32_t* __restrict__ src,
                                                     const uint32_t* __restrict__ copies,
                                                     const float* __restrict__ logit) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int32_t s = src[i];
@@ -470,11 +475,11 @@ cudaError_t launch_relocate(int n, int pitch, int n_planes, float* planes, float
   unsigned long long* total = (unsigned long long*)p; p += al256(8);
   uint32_t* copies = (uint32_t*)p;              p += al256((size_t)n * 4);
   int32_t* src = src_out ? src_out : (int32_t*)p;
-  k_reloc_weights<<<nb, kRelocBlock, 0, s>>>(planes, n, pitch, min_opacity, w, copies, logit, bsum, bdead);
-  k_reloc_scan<<<1, 1024, 0, s>>>(bsum, bdead, nb, total, d_count);
-  k_reloc_sample<<<nb, kRelocBlock, 0, s>>>(w, n, bsum, nb, total, rnd, src, copies);
+  launch_chained(k_reloc_weights, nb, kRelocBlock, 0, s, planes, n, pitch, min_opacity, w, copies, logit, bsum, bdead);
+  launch_chained(k_reloc_scan, 1, 1024, 0, s, bsum, bdead, nb, total, d_count);
+  launch_chained(k_reloc_sample, nb, kRelocBlock, 0, s, w, n, bsum, nb, total, rnd, src, copies);
   const dim3 grid((n + 255) / 256, (n_planes + kCopyPlanes - 1) / kCopyPlanes + 1);
-  k_reloc_copy<<<grid, 256, 0, s>>>(planes, m, v, n, pitch, n_planes, src, copies, logit);
+  launch_chained(k_reloc_copy, grid, 256, 0, s, planes, m, v, n, pitch, n_planes, src, copies, logit);
   return cudaGetLastError();
 }
 

@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_blocks_per_sm(M)) k_project(c
                                                  float4* __restrict__ rec, uint2* __restrict__ rect,
                                                  uint32_t* __restrict__ key, uint32_t* tiles,
                                                  uint32_t* work, uint32_t* __restrict__ n_work) {
+  chain_begin();
   __shared__ uint32_t s_nw;
   if (threadIdx.x == 0) s_nw = 0u;
   __syncthreads();
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
                                                      float* __restrict__ grad2d,
                                                      float* __restrict__ gout,
                                                      const int32_t* __restrict__ status) {
+  chain_begin();
   // 2D gradients of view v+1 in flight while view v is processed (one view
   // ahead measured faster than two or three):
   // [buffer][float4][thread], each thread reads only its own slots
@@ -522,7 +524,7 @@ static cudaError_t launch_project_m(const float* planes, int n, int pitch, const
   int grid = (pitch + kFwdThreads - 1) / kFwdThreads;
   if (grid < 1) return cudaSuccess;
   static_assert(kFwdThreads == kProjRegion, "a projection block owns one worklist region");
-  k_project<M><<<grid, kFwdThreads, 0, s>>>(planes, n, pitch, vt, ro, pb.rec, pb.rect, pb.key, pb.tiles,
+  launch_chained(k_project<M>, grid, kFwdThreads, 0, s, planes, n, pitch, vt, ro, pb.rec, pb.rect, pb.key, pb.tiles,
                                             pb.work, pb.n_work);
   return cudaGetLastError();
 }
@@ -533,7 +535,7 @@ static cudaError_t launch_project_bwd_m(const float* planes, int n, int pitch, c
                                         const int32_t* status, cudaStream_t s) {
   int grid = (n + kBwdThreads - 1) / kBwdThreads;
   if (grid < 1) return cudaSuccess;
-  k_project_bwd<M><<<grid, kBwdThreads, 0, s>>>(planes, n, pitch, vt, ro, grad2d, gout, status);
+  launch_chained(k_project_bwd<M>, grid, kBwdThreads, 0, s, planes, n, pitch, vt, ro, grad2d, gout, status);
   return cudaGetLastError();
 }
 

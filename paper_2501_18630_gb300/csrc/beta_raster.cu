@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1536)) k_raster_f
                                                        float* __restrict__ dLdC,
                                                        float* __restrict__ l1_partial,
                                                        uint32_t* __restrict__ hm, size_t hm_words) {
+  chain_begin();
   constexpr int NT = TW * TH, BXW = TW / 8, RPT = (S + NT - 1) / NT;
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ float s_l1[NT / 32];
@@ -490,6 +491,7 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
                                                        const int32_t* __restrict__ status,
                                                        uint32_t* ctr, const uint32_t* __restrict__ order,
                                                        const uint32_t* __restrict__ hm, size_t hm_words) {
+  chain_begin();
   constexpr int NT = TW * TH, NW = NT / 32, BXW = TW / 8, RPT = (S + NT - 1) / NT;
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ uint32_t s_ridx[2][S];
@@ -1140,6 +1142,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     uint32_t* __restrict__ ncontrib, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const float* __restrict__ target, float* __restrict__ dLdC,
     float* __restrict__ l1_partial, uint32_t* __restrict__ hm, size_t hm_words) {
+  chain_begin();
   using PB = PairBlock<TW, TH, NP>;
   constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
@@ -1401,6 +1404,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     const uint32_t* __restrict__ ranges, const float* __restrict__ Tfin, const uint32_t* __restrict__ ncontrib,
     const float* __restrict__ dLdC, float* __restrict__ grad2d, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const uint32_t* __restrict__ hm, size_t hm_words) {
+  chain_begin();
   using PB = PairBlock<TW, TH, NP>;
   constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
@@ -1480,6 +1484,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     uint32_t* __restrict__ ncontrib, const int32_t* __restrict__ status, uint32_t* ctr,
     const uint32_t* __restrict__ order, const float* __restrict__ target, float* __restrict__ dLdC,
     float* __restrict__ l1_partial, float* __restrict__ grad2d) {
+  chain_begin();
   using PB = PairBlock<TW, TH, NP>;
   constexpr int NT = PB::NT, NW = PB::NW;
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
@@ -1552,11 +1557,13 @@ __device__ __forceinline__ int tile_bucket(uint32_t count) {
 }
 
 __global__ void k_sched_prep(uint32_t* sched) {
+  chain_begin();
   for (int i = threadIdx.x; i < kSchedOrder; i += blockDim.x) sched[i] = 0u;
 }
 
 __global__ void k_sched_hist(const uint32_t* __restrict__ ranges, int total_tiles, uint32_t* sched,
                              const int32_t* __restrict__ status) {
+  chain_begin();
   __shared__ uint32_t h[kBuckets];
   if (*status != 0) return;
   for (int i = threadIdx.x; i < kBuckets; i += blockDim.x) h[i] = 0u;
@@ -1570,6 +1577,7 @@ __global__ void k_sched_hist(const uint32_t* __restrict__ ranges, int total_tile
 
 __global__ void k_sched_scatter(const uint32_t* __restrict__ ranges, int total_tiles,
                                 uint32_t* sched, const int32_t* __restrict__ status) {
+  chain_begin();
   __shared__ uint32_t base[kBuckets];
   if (*status != 0) return;
   if (threadIdx.x == 0) {
@@ -1593,6 +1601,7 @@ __global__ void k_sched_scatter(const uint32_t* __restrict__ ranges, int total_t
 constexpr int kSchedOneTiles = 16384, kSchedThreads = 1024;
 __global__ void __launch_bounds__(kSchedThreads) k_sched_one(const uint32_t* __restrict__ ranges, int total_tiles,
                                                              uint32_t* sched, const int32_t* __restrict__ status) {
+  chain_begin();
   __shared__ uint32_t s_n[kBuckets], s_at[kBuckets];
   const int lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < kSchedHist; i += kSchedThreads) sched[i] = 0u;   // the raster kernels' counters
@@ -1636,6 +1645,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_one(const uint32_t* __r
 __global__ void __launch_bounds__(256) k_l1(ViewTable vt, const float* __restrict__ color,
                                             const float* __restrict__ target, float* __restrict__ dLdC,
                                             float* __restrict__ partial) {
+  chain_begin();
   __shared__ float s_w[8];
   const int b = blockIdx.x;
   int lo = 0, hi = vt.n_views - 1;
@@ -1675,6 +1685,7 @@ __global__ void __launch_bounds__(256) k_l1(ViewTable vt, const float* __restric
 constexpr int kReduceThreads = 512, kReduceLoads = 8;
 __global__ void __launch_bounds__(kReduceThreads) k_l1_reduce(ViewTable vt, const float* __restrict__ partial,
                                                               int total_blocks, float* __restrict__ loss) {
+  chain_begin();
   __shared__ double s_w[32];
   const int v = blockIdx.x;
   const int b0 = vt.v[v].pad0;
@@ -1711,13 +1722,13 @@ cudaError_t launch_schedule(const ViewTable& vt, const uint32_t* ranges, uint32_
                             const int32_t* status, cudaStream_t s) {
   const int T = vt.total_tiles;
   if (T <= kSchedOneTiles) {
-    k_sched_one<<<1, kSchedThreads, 0, s>>>(ranges, T, sched, status);
+    launch_chained(k_sched_one, 1, kSchedThreads, 0, s, ranges, T, sched, status);
     return cudaGetLastError();
   }
   const int grid = std::max(1, std::min((T + 255) / 256, device_sm_count() * 4));
-  k_sched_prep<<<1, 160, 0, s>>>(sched);
-  k_sched_hist<<<grid, 256, 0, s>>>(ranges, T, sched, status);
-  k_sched_scatter<<<grid, 256, 0, s>>>(ranges, T, sched, status);
+  launch_chained(k_sched_prep, 1, 160, 0, s, sched);
+  launch_chained(k_sched_hist, grid, 256, 0, s, ranges, T, sched, status);
+  launch_chained(k_sched_scatter, grid, 256, 0, s, ranges, T, sched, status);
   return cudaGetLastError();
 }
 
@@ -1743,12 +1754,10 @@ cudaError_t fwd_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* r
   constexpr int NT = PairBlock<TW, TH, NP>::NT;
   if (sched) {
     auto k = k_raster_fwd2<TW, TH, S, NP, true>;
-    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
+    launch_chained(k, persistent_grid(k, NT, vt.total_tiles), NT, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
         target, dL_dcolor, l1_partial, hm.words, hm.n_words);
   } else {
-    k_raster_fwd2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
+    launch_chained(k_raster_fwd2<TW, TH, S, NP, false>, vt.total_tiles, NT, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
         l1_partial, hm.words, hm.n_words);
   }
   return cudaGetLastError();
@@ -1766,12 +1775,10 @@ cudaError_t fwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
   } else {
     if (sched) {
       auto k = k_raster_fwd<TW, TH, S, true>;
-      k<<<persistent_grid(k, TW * TH, vt.total_tiles), TW * TH, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
+      launch_chained(k, persistent_grid(k, TW * TH, vt.total_tiles), TW * TH, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder,
           target, dL_dcolor, l1_partial, hm.words, hm.n_words);
     } else {
-      k_raster_fwd<TW, TH, S, false><<<vt.total_tiles, TW * TH, 0, s>>>(
-          vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
+      launch_chained(k_raster_fwd<TW, TH, S, false>, vt.total_tiles, TW * TH, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
           l1_partial, hm.words, hm.n_words);
     }
   }
@@ -1786,12 +1793,10 @@ cudaError_t bwd_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* r
   constexpr int NT = PairBlock<TW, TH, NP>::NT;
   if (sched) {
     auto k = k_raster_bwd2<TW, TH, S, NP, true>;
-    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
+    launch_chained(k, persistent_grid(k, NT, vt.total_tiles), NT, 0, s, vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
         sched + kSchedOrder, hm.words, hm.n_words);
   } else {
-    k_raster_bwd2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
+    launch_chained(k_raster_bwd2<TW, TH, S, NP, false>, vt.total_tiles, NT, 0, s, vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
         hm.words, hm.n_words);
   }
   return cudaGetLastError();
@@ -1809,12 +1814,10 @@ cudaError_t bwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
   } else {
     if (sched) {
       auto k = k_raster_bwd<TW, TH, S, true>;
-      k<<<persistent_grid(k, TW * TH, vt.total_tiles), TW * TH, 0, s>>>(
-          vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
+      launch_chained(k, persistent_grid(k, TW * TH, vt.total_tiles), TW * TH, 0, s, vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched + 2,
           sched + kSchedOrder, hm.words, hm.n_words);
     } else {
-      k_raster_bwd<TW, TH, S, false><<<vt.total_tiles, TW * TH, 0, s>>>(
-          vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
+      launch_chained(k_raster_bwd<TW, TH, S, false>, vt.total_tiles, TW * TH, 0, s, vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, nullptr, nullptr,
           hm.words, hm.n_words);
     }
   }
@@ -1830,12 +1833,10 @@ cudaError_t step_pairs(const ViewTable& vt, const RenderOpts& ro, const float4* 
   constexpr int NT = PairBlock<TW, TH, NP>::NT;
   if (sched) {
     auto k = k_raster_step2<TW, TH, S, NP, true>;
-    k<<<persistent_grid(k, NT, vt.total_tiles), NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder, target,
+    launch_chained(k, persistent_grid(k, NT, vt.total_tiles), NT, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched + 0, sched + kSchedOrder, target,
         dL_dcolor, l1_partial, grad2d);
   } else {
-    k_raster_step2<TW, TH, S, NP, false><<<vt.total_tiles, NT, 0, s>>>(
-        vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
+    launch_chained(k_raster_step2<TW, TH, S, NP, false>, vt.total_tiles, NT, 0, s, vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, nullptr, nullptr, target, dL_dcolor,
         l1_partial, grad2d);
   }
   return cudaGetLastError();
@@ -1921,7 +1922,7 @@ cudaError_t launch_raster_fwd_l1(const ViewTable& vt_in, const RenderOpts& ro, c
   if (e != cudaSuccess) return e;
   ViewTable vt = vt_in;   // the reduce finds view v's partials from tile_off[v]
   for (int v = 0; v < vt.n_views; ++v) vt.v[v].pad0 = vt.v[v].tile_off;
-  k_l1_reduce<<<vt.n_views, kReduceThreads, 0, s>>>(vt, ws, vt.total_tiles, loss);
+  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, vt.total_tiles, loss);
   return cudaGetLastError();
 }
 
@@ -1943,7 +1944,7 @@ cudaError_t launch_raster_step_l1(const ViewTable& vt_in, const RenderOpts& ro, 
   if (e != cudaSuccess) return e;
   ViewTable vt = vt_in;   // the reduce finds view v's partials from tile_off[v]
   for (int v = 0; v < vt.n_views; ++v) vt.v[v].pad0 = vt.v[v].tile_off;
-  k_l1_reduce<<<vt.n_views, kReduceThreads, 0, s>>>(vt, ws, vt.total_tiles, loss);
+  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, vt.total_tiles, loss);
   return cudaGetLastError();
 }
 
@@ -1977,8 +1978,8 @@ cudaError_t launch_l1(const ViewTable& vt_in, const float* color, const float* t
   ViewTable vt = vt_in;
   int nb = l1_blocks(vt);
   if (nb <= 0) return cudaSuccess;
-  k_l1<<<nb, 256, 0, s>>>(vt, color, target, dL_dcolor, ws);
-  k_l1_reduce<<<vt.n_views, kReduceThreads, 0, s>>>(vt, ws, nb, loss);
+  launch_chained(k_l1, nb, 256, 0, s, vt, color, target, dL_dcolor, ws);
+  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, nb, loss);
   return cudaGetLastError();
 }
 

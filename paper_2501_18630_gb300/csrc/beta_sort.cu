@@ -114,6 +114,7 @@ size_t binsort_ws_bytes(int64_t n_items, int64_t cap, int total_tiles) {
 
 __global__ void k_sort_prep(uint32_t* cnt, int total_tiles, u64* look, int64_t nb_scan,
                             uint32_t* counters, int64_t* d_count, int32_t* status) {
+  chain_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (int64_t i = t; i < (int64_t)kSub * crow(total_tiles); i += stride) cnt[i] = 0u;
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_count(const uint2* __rest
                                                          const uint32_t* __restrict__ tiles, int64_t n_items,
                                                          int pitch, ViewTable vt, int total_tiles,
                                                          uint32_t* cnt) {
+  chain_begin();
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_items;
        r += (int64_t)gridDim.x * blockDim.x) {
     const Rect q = rect_of(rects[r], tiles[r]);
@@ -259,6 +261,7 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scan(const uint32_t* __re
                                                         uint32_t* __restrict__ longl, int64_t cap,
                                                         int64_t* d_count, int32_t* status,
                                                         int spin_limit, int64_t withhold) {
+  chain_begin();
   constexpr int kTile = kSortThreads * ITEMS;
   __shared__ u64 s_w[kSortThreads / 32];
   __shared__ u64 s_base;
@@ -380,6 +383,7 @@ __global__ void __launch_bounds__(kSortThreads) k_tile_scatter(const uint2* __re
                                                            int total_tiles, uint32_t* cursor,
                                                            u64* __restrict__ items,
                                                            int64_t cap, const int32_t* __restrict__ status) {
+  chain_begin();
   if (*status != 0) return;   // capacity overflow (or a failed scan): no list is written
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_items;
        r += (int64_t)gridDim.x * blockDim.x) {
@@ -713,6 +717,7 @@ __global__ void __launch_bounds__(kSortThreads, kSortCtasPerSM) k_tile_sort(cons
                                                            uint32_t* __restrict__ vals,
                                                            const int32_t* __restrict__ status,
                                                            int ticket_lists) {
+  chain_begin();
   constexpr int kWarpSm = kWarpMax + kWarpMax / 16;
   __shared__ u64 sm[kCtaMax + kCtaMax / 16];
   __shared__ uint32_t s_t;
@@ -785,26 +790,25 @@ cudaError_t launch_bin_sort(const ViewTable& vt, int pitch, ProjBuffers pb, uint
   const int64_t grid_p = std::min<int64_t>(cdiv(std::max<int64_t>((int64_t)kSub * crow(total_tiles), nb_scan), kSortThreads), 1024);
   const int64_t grid_r = std::max<int64_t>(1, std::min<int64_t>(cdiv(n_items, kSortThreads), 1 << 20));
 
-  k_sort_prep<<<(unsigned)std::max<int64_t>(grid_p, 1), kSortThreads, 0, s>>>(w.cnt, total_tiles, w.look,
+  launch_chained(k_sort_prep, (unsigned)std::max<int64_t>(grid_p, 1), kSortThreads, 0, s, w.cnt, total_tiles, w.look,
                                                                           (int64_t)(align256((size_t)nb_scan * 8) / 8),
                                                                           w.counters, d_count, d_status);
-  k_tile_count<<<(unsigned)grid_r, kSortThreads, 0, s>>>(pb.rect, pb.tiles, n_items, pitch, vt, total_tiles, w.cnt);
+  launch_chained(k_tile_count, (unsigned)grid_r, kSortThreads, 0, s, pb.rect, pb.tiles, n_items, pitch, vt, total_tiles, w.cnt);
   // look-back entries the workspace holds (its pieces are 256-byte aligned)
   const int64_t entries = (int64_t)(align256((size_t)nb_scan * 8) / 8);
   auto scan = [&](auto kernel, int items) {
-    kernel<<<(unsigned)cdiv(total_tiles, kSortThreads * items), kSortThreads, 0, s>>>(
-        w.cnt, total_tiles, w.look, w.counters, ranges, w.cursor, w.longl, cap, d_count, d_status,
+    launch_chained(kernel, (unsigned)cdiv(total_tiles, kSortThreads * items), kSortThreads, 0, s, w.cnt, total_tiles, w.look, w.counters, ranges, w.cursor, w.longl, cap, d_count, d_status,
         g_spin_limit.load(), g_withhold.load());
   };
   if (cdiv(total_tiles, kSortThreads) <= entries) scan(k_tile_scan<1>, 1);
   else if (cdiv(total_tiles, kSortThreads * 2) <= entries) scan(k_tile_scan<2>, 2);
   else if (cdiv(total_tiles, kSortThreads * 4) <= entries) scan(k_tile_scan<4>, 4);
   else scan(k_tile_scan<kScanItems>, kScanItems);
-  k_tile_scatter<<<(unsigned)grid_r, kSortThreads, 0, s>>>(pb.rect, pb.tiles, pb.key, n_items, pitch, vt, total_tiles,
+  launch_chained(k_tile_scatter, (unsigned)grid_r, kSortThreads, 0, s, pb.rect, pb.tiles, pb.key, n_items, pitch, vt, total_tiles,
                                                        w.cursor, w.items, cap, d_status);
   const int sort_grid = device_sm_count() * kSortCtasPerSM;
   const int tickets = std::max(1, std::min(kTicketLists, total_tiles / (sort_grid * (kSortThreads / 32))));
-  k_tile_sort<<<(unsigned)sort_grid, kSortThreads, 0, s>>>(ranges, total_tiles, w.longl, w.counters, w.items, w.tmp,
+  launch_chained(k_tile_sort, (unsigned)sort_grid, kSortThreads, 0, s, ranges, total_tiles, w.longl, w.counters, w.items, w.tmp,
                                                            pair_vals, d_status, tickets);
   return cudaGetLastError();
 }

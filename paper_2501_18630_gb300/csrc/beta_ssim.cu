@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(kThreads2, 4) k_ssim_stats(ViewTable vt, SsimW
                                                              const float* __restrict__ target,
                                                              float2* __restrict__ ab, float* __restrict__ cc,
                                                              double* __restrict__ acc) {
+  chain_begin();
   // the staged (x, y), then the horizontal results (x, y, (x - y)^2, x y)
   __shared__ __align__(16) float4 s_buf[kRowsV * kSH];
   __shared__ double s_w[8];
@@ -331,6 +332,7 @@ __global__ void __launch_bounds__(kThreads2, 4) k_ssim_grad(ViewTable vt, SsimWi
                                                             const float2* __restrict__ ab, const float* __restrict__ cc,
                                                             float lambda, float* __restrict__ dLdC,
                                                             double* __restrict__ acc) {
+  chain_begin();
   // the staged (a, b) and c, then their horizontal pass
   __shared__ __align__(16) float2 s_ab[kHY * kSX];
   __shared__ float s_c[kHY * kSX];
@@ -429,6 +431,7 @@ __global__ void __launch_bounds__(kThreads2, 4) k_ssim_grad(ViewTable vt, SsimWi
 // per view: the sums of its blocks' partials (fixed order), then the loss
 __global__ void __launch_bounds__(512) k_ssim_loss(ViewTable vt, const double* __restrict__ acc, int nb,
                                                    float lambda, float* __restrict__ loss) {
+  chain_begin();
   const int v = blockIdx.x;
   const int b0 = vt.v[v].pad0, b1 = v + 1 < vt.n_views ? vt.v[v + 1].pad0 : nb;
   double ss = 0.0, sl = 0.0;
@@ -510,9 +513,9 @@ cudaError_t launch_ssim_loss(const ViewTable& vt_in, const float* color, const f
   float2* ab = (float2*)ws;                 // (a, b) of every value, then c
   float* cc = (float*)ws + 2 * plane;
   double* acc = (double*)((char*)ws + ((size_t)9 * vt.total_pixels * sizeof(float) + 255) / 256 * 256);
-  k_ssim_stats<<<nb, kThreads2, 0, s>>>(vt, win, color, target, ab, cc, acc);
-  k_ssim_grad<<<nb, kThreads2, 0, s>>>(vt, win, color, target, ab, cc, lambda, dL_dcolor, acc);
-  k_ssim_loss<<<vt.n_views, 512, 0, s>>>(vt, acc, nb, lambda, loss);
+  launch_chained(k_ssim_stats, nb, kThreads2, 0, s, vt, win, color, target, ab, cc, acc);
+  launch_chained(k_ssim_grad, nb, kThreads2, 0, s, vt, win, color, target, ab, cc, lambda, dL_dcolor, acc);
+  launch_chained(k_ssim_loss, vt.n_views, 512, 0, s, vt, acc, nb, lambda, loss);
   return cudaGetLastError();
 }
 
