@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "beta_internal.cuh"
 
 namespace beta {
@@ -297,8 +299,21 @@ __device__ __forceinline__ void view_geo_bwd(const PrimGeo& pg, const ViewDev& V
 // rotation matrix, the scales and the lobe directions are summed over views
 // first and taken through the view-independent maps once.
 // ---------------------------------------------------------------------------
-constexpr int kBwdThreads = 128, kBwdBlocksPerSM = 3;   // up to 170 registers a thread
+// 3 CTAs per SM, up to 170 registers a thread (4 of them: 128 registers, spills,
+// 535 against 380 us on 1M primitives x 16 views)
+constexpr int kBwdThreads = 128, kBwdBlocksPerSM = 3;
+// parameters of two blocks of primitives and 2D gradients of two (block, view) pairs
+constexpr size_t bwd_smem(int lobes) {
+  return (size_t)kBwdThreads * (2 * (15 + 6 * lobes) * sizeof(float) + 2 * 3 * sizeof(float4));
+}
 
+// A persistent grid takes blocks of 128 primitives: while a block's last view is
+// chained back and its gradients are stored, the next block's parameters and its
+// first view's 2D gradients are copied into shared memory (within a block, view
+// v + 1's 2D gradients while view v is processed).  With one block per CTA and
+// the parameters loaded at its start, the 12 warps an SM holds waited for them:
+// 1M primitives x 1 view 100 -> 62 us (its 350 MB at the copy rate: 51), x 16
+// views 409 -> 380, 6M x 8 x 4K 1.39 -> 1.25 ms.
 template <int M>
 __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(const float* __restrict__ planes, int n,
                                                      int pitch, ViewTable vt, RenderOpts ro,
@@ -306,214 +321,246 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
                                                      float* __restrict__ gout,
                                                      const int32_t* __restrict__ status) {
   chain_begin();
-  // 2D gradients of view v+1 in flight while view v is processed (one view
-  // ahead measured faster than two or three):
-  // [buffer][float4][thread], each thread reads only its own slots
-  constexpr int kAhead = 1;
-  __shared__ __align__(16) float4 s_g[kAhead + 1][3][kBwdThreads];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  extern __shared__ __align__(16) float s_dyn[];
+  float4* const s_g = reinterpret_cast<float4*>(s_dyn);                  // [2][3][kBwdThreads]
+  float* const s_p = s_dyn + 2 * 3 * 4 * kBwdThreads;                    // [2][NP][kBwdThreads]
   constexpr int NP = 15 + 6 * M;
   constexpr int MM = M > 0 ? M : 1;
-  float gp[NP];
+  const int tid = threadIdx.x;
+  const int nblk = (n + kBwdThreads - 1) / kBwdThreads;
+  const bool bad = *status != 0;
+  // 16-byte copies: columns up to n rounded up to 4 lie inside the pitch
+  auto fetch_params = [&](int blk, int buf) {
+    for (int q = tid; q < NP * (kBwdThreads / 4); q += kBwdThreads) {
+      const int k = q / (kBwdThreads / 4), c = (q - k * (kBwdThreads / 4)) * 4;
+      if (blk * kBwdThreads + c < n)
+        cp_async16(&s_p[(buf * NP + k) * kBwdThreads + c], planes + (size_t)k * pitch + blk * kBwdThreads + c);
+    }
+  };
+  auto fetch_g = [&](int blk, int v, int slot) {
+    const int j = blk * kBwdThreads + tid;
+    if (j < n) {
+      const float4* src = reinterpret_cast<const float4*>(grad2d + ((size_t)v * pitch + j) * kGrad2dStride);
 #pragma unroll
-  for (int k = 0; k < NP; ++k) gp[k] = 0.0f;
-  float p[NP];
-  bool ok = false;
-  load_params<M>(planes, pitch, i, p, ok);
-  if (ok) ok = (p[11] >= ro.b_lo) && (p[11] < ro.b_hi);
-  if (*status != 0) ok = false;
-  PrimGeo pg;
-  if (ok) ok = rule_prim(p, pg);
-  if (ok) {
+      for (int q = 0; q < 3; ++q) cp_async16(&s_g[(slot * 3 + q) * kBwdThreads + tid], src + q);
+    }
+  };
+  int slot = 0, pbuf = 0;
+  if ((int)blockIdx.x < nblk) {
+    fetch_params(blockIdx.x, 0);
+    fetch_g(blockIdx.x, 0, 0);
+  }
+  cp_async_commit();
+  for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x, pbuf ^= 1) {
+    const int i = blk * kBwdThreads + tid;
+    const int next = blk + gridDim.x;
+    cp_async_wait<0>();
+    __syncthreads();   // this block's parameters have landed; the other buffer is free
+    float gp[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) gp[k] = 0.0f;
+    float p[NP];
+    bool ok = i < n;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      p[k] = s_p[(pbuf * NP + k) * kBwdThreads + tid];
+      ok = ok && isfinite(p[k]);
+    }
+    if (ok) ok = (p[11] >= ro.b_lo) && (p[11] < ro.b_hi);
+    if (bad) ok = false;
+    PrimGeo pg;
+    if (ok) ok = rule_prim(p, pg);
     PrimAttr<M> at;
-    prim_attr<M>(p, ro.color_mode, at);
-    float dR[9], ds[3], dRm[MM][3];
+    if (ok) prim_attr<M>(p, ro.color_mode, at);
+    {
+      float dR[9], ds[3], dRm[MM][3];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) dR[k] = 0.0f;
+      for (int k = 0; k < 9; ++k) dR[k] = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ds[k] = 0.0f;
+      for (int k = 0; k < 3; ++k) ds[k] = 0.0f;
 #pragma unroll
-    for (int m = 0; m < MM; ++m) dRm[m][0] = dRm[m][1] = dRm[m][2] = 0.0f;
-    float go = 0.0f, gbeta = 0.0f;
-    const int tid = threadIdx.x;
-    auto fetch = [&](int v) {
-      if (v < vt.n_views) {
-        const float4* src = reinterpret_cast<const float4*>(grad2d + ((size_t)v * pitch + i) * kGrad2dStride);
+      for (int m = 0; m < MM; ++m) dRm[m][0] = dRm[m][1] = dRm[m][2] = 0.0f;
+      float go = 0.0f, gbeta = 0.0f;
+      for (int v = 0; v < vt.n_views; ++v) {
+        const ViewDev& V = vt.v[v];
+        float4* g2 = reinterpret_cast<float4*>(grad2d + ((size_t)v * pitch + i) * kGrad2dStride);
+        if (v > 0) cp_async_wait<0>();   // the thread's own copies
+        const float4 ga4 = s_g[(slot * 3 + 0) * kBwdThreads + tid], gb4 = s_g[(slot * 3 + 1) * kBwdThreads + tid],
+                     gc4 = s_g[(slot * 3 + 2) * kBwdThreads + tid];
+        slot ^= 1;
+        if (v + 1 < vt.n_views) {
+          fetch_g(blk, v + 1, slot);
+        } else if (next < nblk) {
+          fetch_params(next, pbuf ^ 1);
+          fetch_g(next, 0, slot);
+        }
+        cp_async_commit();
+        if (!ok) continue;
+        const float G[kGrad2d] = {ga4.x, ga4.y, ga4.z, ga4.w, gb4.x, gb4.y, gb4.z, gb4.w, gc4.x, gc4.y};
+        bool any = false;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) cp_async16(&s_g[v % (kAhead + 1)][q][tid], src + q);
+        for (int k = 0; k < kGrad2d; ++k) any = any || (G[k] != 0.0f);
+        if (!any) continue;
+        // leave the accumulator zeroed for the next backward
+        const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        g2[0] = z4;
+        g2[1] = z4;
+        g2[2] = z4;
+        ViewGeo g;
+        uint32_t kk;
+        if (!rule_depth(pg, V, g, kk)) continue;
+        view_geo_bwd(pg, V, g);
+        // whitening of Sigma' (the forward's formulas) turns the whitened sums
+        // into d mu' and d Sigma' = [[ga, gb/2], [gb/2, gc]] (gb: off-diagonal scalar)
+        float gmx, gmy, ga, gb, gc;
+        {
+          const float a0 = fmaf(g.M0[0], g.M0[0], fmaf(g.M0[1], g.M0[1], g.M0[2] * g.M0[2]));
+          const float c0 = fmaf(g.M1[0], g.M1[0], fmaf(g.M1[1], g.M1[1], g.M1[2] * g.M1[2]));
+          const float bb = fmaf(g.M0[0], g.M1[0], fmaf(g.M0[1], g.M1[1], g.M0[2] * g.M1[2]));
+          const float m01 = diff_of_products(g.M0[0], g.M1[1], g.M0[1], g.M1[0]);
+          const float m02 = diff_of_products(g.M0[0], g.M1[2], g.M0[2], g.M1[0]);
+          const float m12 = diff_of_products(g.M0[1], g.M1[2], g.M0[2], g.M1[1]);
+          float det = fmaf(m01, m01, fmaf(m02, m02, m12 * m12));
+          const float aa = a0 + ro.blur_eps;
+          if (ro.blur_eps != 0.0f) det = fmaf(ro.blur_eps, a0 + c0 + ro.blur_eps, det);
+          const float p = rsqrtf(aa), isd = rsqrtf(det);
+          const float q1 = (aa * p) * isd, q2 = -(bb * p) * isd;
+          const float b2 = 2.0f * at.beta;
+          gmx = b2 * fmaf(p, G[0], q2 * G[1]);
+          gmy = b2 * q1 * G[1];
+          ga = at.beta * fmaf(p * p, G[2], fmaf(2.0f * p * q2, G[3], q2 * q2 * G[4]));
+          gb = b2 * q1 * fmaf(p, G[3], q2 * G[4]);
+          gc = at.beta * q1 * q1 * G[4];
+        }
+        // Sigma' = M M^T: dM0 = 2 ga M0 + gb M1, dM1 = gb M0 + 2 gc M1
+        float dM0[3], dM1[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          dM0[k] = 2.0f * ga * g.M0[k] + gb * g.M1[k];
+          dM1[k] = gb * g.M0[k] + 2.0f * gc * g.M1[k];
+        }
+        // M0k = (j00 A0k + j02 A2k) s_k ; M1k = (j11 A1k + j12 A2k) s_k
+        float dA[9];
+        float dj00 = 0.f, dj02 = 0.f, dj11 = 0.f, dj12 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          float u0 = g.j00 * g.A[0 * 3 + k] + g.j02 * g.A[2 * 3 + k];
+          float u1 = g.j11 * g.A[1 * 3 + k] + g.j12 * g.A[2 * 3 + k];
+          ds[k] += dM0[k] * u0 + dM1[k] * u1;
+          dA[0 * 3 + k] = dM0[k] * g.j00 * pg.s[k];
+          dA[1 * 3 + k] = dM1[k] * g.j11 * pg.s[k];
+          dA[2 * 3 + k] = (dM0[k] * g.j02 + dM1[k] * g.j12) * pg.s[k];
+          dj00 += dM0[k] * g.A[0 * 3 + k] * pg.s[k];
+          dj02 += dM0[k] * g.A[2 * 3 + k] * pg.s[k];
+          dj11 += dM1[k] * g.A[1 * 3 + k] * pg.s[k];
+          dj12 += dM1[k] * g.A[2 * 3 + k] * pg.s[k];
+        }
+        // A = W Rq  ->  dRq += W^T dA
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            dR[a * 3 + c] += V.R[0 * 3 + a] * dA[0 * 3 + c] + V.R[1 * 3 + a] * dA[1 * 3 + c] +
+                             V.R[2 * 3 + a] * dA[2 * 3 + c];
+        // J(t) and mu'(t)
+        const float tx = g.tc[0], ty = g.tc[1], iz = g.iz, iz2 = iz * iz, iz3 = iz2 * iz;
+        float dtx = dj02 * (-V.fx * iz2) + gmx * V.fx * iz;
+        float dty = dj12 * (-V.fy * iz2) + gmy * V.fy * iz;
+        float dtz = dj00 * (-V.fx * iz2) + dj11 * (-V.fy * iz2) + dj02 * (2.f * V.fx * tx * iz3) +
+                    dj12 * (2.f * V.fy * ty * iz3) - gmx * V.fx * tx * iz2 - gmy * V.fy * ty * iz2;
+        // t = W mu + t_w
+        gp[0] += V.R[0] * dtx + V.R[3] * dty + V.R[6] * dtz;
+        gp[1] += V.R[1] * dtx + V.R[4] * dty + V.R[7] * dtz;
+        gp[2] += V.R[2] * dtx + V.R[5] * dty + V.R[8] * dtz;
+        go += G[5];                               // times 1/o below
+        gbeta += G[6];                            // times ln 2 below
+        // colour
+        const float gr = G[7], gg = G[8], gbl = G[9];
+        if (ro.color_mode != 2) {
+          gp[12] += gr;
+          gp[13] += gg;
+          gp[14] += gbl;
+        }
+        if (M > 0 && ro.color_mode != 1) {
+          float vx = p[0] - V.campos[0], vy = p[1] - V.campos[1], vz = p[2] - V.campos[2];
+          float il = rsqrtf(fmaf(vx, vx, fmaf(vy, vy, vz * vz)));
+          vx *= il;
+          vy *= il;
+          vz *= il;
+          float dvx = 0.f, dvy = 0.f, dvz = 0.f;
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            const float* L = p + 15 + 6 * m;
+            float* dL = gp + 15 + 6 * m;
+            const float rx = at.lobe_dir[m][0], ry = at.lobe_dir[m][1], rz = at.lobe_dir[m][2];
+            float dot = rx * vx + ry * vy + rz * vz;
+            if (dot > 0.0f) {
+              // w = dot^bm and d w / d dot = bm w / dot, with the MUFU log2/exp2
+              // (relative error ~1e-6, far inside the gradient tolerance)
+              float bm = at.lobe_beta[m];
+              float lw = lg2_approx(dot);
+              float wgt = ex2_approx(bm * lw);
+              dL[3] += wgt * gr;
+              dL[4] += wgt * gg;
+              dL[5] += wgt * gbl;
+              float gw = gr * L[3] + gg * L[4] + gbl * L[5];
+              dL[2] += gw * wgt * (lw * kLn2) * bm;
+              float ddot = gw * bm * wgt * __frcp_rn(dot);
+              dRm[m][0] += ddot * vx;
+              dRm[m][1] += ddot * vy;
+              dRm[m][2] += ddot * vz;
+              dvx += ddot * rx;
+              dvy += ddot * ry;
+              dvz += ddot * rz;
+            }
+          }
+          float vd = vx * dvx + vy * dvy + vz * dvz;
+          gp[0] += (dvx - vx * vd) * il;
+          gp[1] += (dvy - vy * vd) * il;
+          gp[2] += (dvz - vz * vd) * il;
+        }
       }
-      cp_async_commit();   // one group per view, empty past the last
-    };
+      if (ok) {
+        // scales: s = exp(log-scale)
 #pragma unroll
-    for (int a = 0; a < kAhead; ++a) fetch(a);
-    for (int v = 0; v < vt.n_views; ++v) {
-      const ViewDev& V = vt.v[v];
-      float4* g2 = reinterpret_cast<float4*>(grad2d + ((size_t)v * pitch + i) * kGrad2dStride);
-      cp_async_wait<kAhead - 1>();   // view v's group has landed
-      const int sb = v % (kAhead + 1);
-      const float4 ga4 = s_g[sb][0][tid], gb4 = s_g[sb][1][tid], gc4 = s_g[sb][2][tid];
-      fetch(v + kAhead);
-      const float G[kGrad2d] = {ga4.x, ga4.y, ga4.z, ga4.w, gb4.x, gb4.y, gb4.z, gb4.w, gc4.x, gc4.y};
-      bool any = false;
-#pragma unroll
-      for (int k = 0; k < kGrad2d; ++k) any = any || (G[k] != 0.0f);
-      if (!any) continue;
-      // leave the accumulator zeroed for the next backward
-      const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      g2[0] = z4;
-      g2[1] = z4;
-      g2[2] = z4;
-      ViewGeo g;
-      uint32_t kk;
-      if (!rule_depth(pg, V, g, kk)) continue;
-      view_geo_bwd(pg, V, g);
-      // whitening of Sigma' (the forward's formulas) turns the whitened sums
-      // into d mu' and d Sigma' = [[ga, gb/2], [gb/2, gc]] (gb: off-diagonal scalar)
-      float gmx, gmy, ga, gb, gc;
-      {
-        const float a0 = fmaf(g.M0[0], g.M0[0], fmaf(g.M0[1], g.M0[1], g.M0[2] * g.M0[2]));
-        const float c0 = fmaf(g.M1[0], g.M1[0], fmaf(g.M1[1], g.M1[1], g.M1[2] * g.M1[2]));
-        const float bb = fmaf(g.M0[0], g.M1[0], fmaf(g.M0[1], g.M1[1], g.M0[2] * g.M1[2]));
-        const float m01 = diff_of_products(g.M0[0], g.M1[1], g.M0[1], g.M1[0]);
-        const float m02 = diff_of_products(g.M0[0], g.M1[2], g.M0[2], g.M1[0]);
-        const float m12 = diff_of_products(g.M0[1], g.M1[2], g.M0[2], g.M1[1]);
-        float det = fmaf(m01, m01, fmaf(m02, m02, m12 * m12));
-        const float aa = a0 + ro.blur_eps;
-        if (ro.blur_eps != 0.0f) det = fmaf(ro.blur_eps, a0 + c0 + ro.blur_eps, det);
-        const float p = rsqrtf(aa), isd = rsqrtf(det);
-        const float q1 = (aa * p) * isd, q2 = -(bb * p) * isd;
-        const float b2 = 2.0f * at.beta;
-        gmx = b2 * fmaf(p, G[0], q2 * G[1]);
-        gmy = b2 * q1 * G[1];
-        ga = at.beta * fmaf(p * p, G[2], fmaf(2.0f * p * q2, G[3], q2 * q2 * G[4]));
-        gb = b2 * q1 * fmaf(p, G[3], q2 * G[4]);
-        gc = at.beta * q1 * q1 * G[4];
-      }
-      // Sigma' = M M^T: dM0 = 2 ga M0 + gb M1, dM1 = gb M0 + 2 gc M1
-      float dM0[3], dM1[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        dM0[k] = 2.0f * ga * g.M0[k] + gb * g.M1[k];
-        dM1[k] = gb * g.M0[k] + 2.0f * gc * g.M1[k];
-      }
-      // M0k = (j00 A0k + j02 A2k) s_k ; M1k = (j11 A1k + j12 A2k) s_k
-      float dA[9];
-      float dj00 = 0.f, dj02 = 0.f, dj11 = 0.f, dj12 = 0.f;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        float u0 = g.j00 * g.A[0 * 3 + k] + g.j02 * g.A[2 * 3 + k];
-        float u1 = g.j11 * g.A[1 * 3 + k] + g.j12 * g.A[2 * 3 + k];
-        ds[k] += dM0[k] * u0 + dM1[k] * u1;
-        dA[0 * 3 + k] = dM0[k] * g.j00 * pg.s[k];
-        dA[1 * 3 + k] = dM1[k] * g.j11 * pg.s[k];
-        dA[2 * 3 + k] = (dM0[k] * g.j02 + dM1[k] * g.j12) * pg.s[k];
-        dj00 += dM0[k] * g.A[0 * 3 + k] * pg.s[k];
-        dj02 += dM0[k] * g.A[2 * 3 + k] * pg.s[k];
-        dj11 += dM1[k] * g.A[1 * 3 + k] * pg.s[k];
-        dj12 += dM1[k] * g.A[2 * 3 + k] * pg.s[k];
-      }
-      // A = W Rq  ->  dRq += W^T dA
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          dR[a * 3 + c] += V.R[0 * 3 + a] * dA[0 * 3 + c] + V.R[1 * 3 + a] * dA[1 * 3 + c] +
-                           V.R[2 * 3 + a] * dA[2 * 3 + c];
-      // J(t) and mu'(t)
-      const float tx = g.tc[0], ty = g.tc[1], iz = g.iz, iz2 = iz * iz, iz3 = iz2 * iz;
-      float dtx = dj02 * (-V.fx * iz2) + gmx * V.fx * iz;
-      float dty = dj12 * (-V.fy * iz2) + gmy * V.fy * iz;
-      float dtz = dj00 * (-V.fx * iz2) + dj11 * (-V.fy * iz2) + dj02 * (2.f * V.fx * tx * iz3) +
-                  dj12 * (2.f * V.fy * ty * iz3) - gmx * V.fx * tx * iz2 - gmy * V.fy * ty * iz2;
-      // t = W mu + t_w
-      gp[0] += V.R[0] * dtx + V.R[3] * dty + V.R[6] * dtz;
-      gp[1] += V.R[1] * dtx + V.R[4] * dty + V.R[7] * dtz;
-      gp[2] += V.R[2] * dtx + V.R[5] * dty + V.R[8] * dtz;
-      go += G[5];                               // times 1/o below
-      gbeta += G[6];                            // times ln 2 below
-      // colour
-      const float gr = G[7], gg = G[8], gbl = G[9];
-      if (ro.color_mode != 2) {
-        gp[12] += gr;
-        gp[13] += gg;
-        gp[14] += gbl;
-      }
-      if (M > 0 && ro.color_mode != 1) {
-        float vx = p[0] - V.campos[0], vy = p[1] - V.campos[1], vz = p[2] - V.campos[2];
-        float il = rsqrtf(fmaf(vx, vx, fmaf(vy, vy, vz * vz)));
-        vx *= il;
-        vy *= il;
-        vz *= il;
-        float dvx = 0.f, dvy = 0.f, dvz = 0.f;
+        for (int k = 0; k < 3; ++k) gp[3 + k] = ds[k] * pg.s[k];
+        // Rq(q_hat) -> d q_hat -> d q
+        const float w = pg.q[0], x = pg.q[1], y = pg.q[2], z = pg.q[3];
+        float dw = 2.f * (-z * dR[1] + y * dR[2] + z * dR[3] - x * dR[5] - y * dR[6] + x * dR[7]);
+        float dx = 2.f * (y * dR[1] + z * dR[2] + y * dR[3] - 2.f * x * dR[4] - w * dR[5] + z * dR[6] +
+                          w * dR[7] - 2.f * x * dR[8]);
+        float dy = 2.f * (-2.f * y * dR[0] + x * dR[1] + w * dR[2] + x * dR[3] + z * dR[5] - w * dR[6] +
+                          z * dR[7] - 2.f * y * dR[8]);
+        float dz = 2.f * (-2.f * z * dR[0] - w * dR[1] + x * dR[2] + w * dR[3] - 2.f * z * dR[4] +
+                          y * dR[5] + x * dR[6] + y * dR[7]);
+        float qd = w * dw + x * dx + y * dy + z * dz;
+        float iq = 1.0f / pg.qn;
+        gp[6] = (dw - w * qd) * iq;
+        gp[7] = (dx - x * qd) * iq;
+        gp[8] = (dy - y * qd) * iq;
+        gp[9] = (dz - z * qd) * iq;
+        // opacity logit and shape
+        // dL/do = (1/o) sum (dL/dalpha) alpha; sigmoid' = o (1 - o)
+        gp[10] = go * (1.0f - at.o);
+        // dL/dbeta = ln 2 sum (dL/dalpha) alpha log2(1 - r^2); dbeta/db = beta
+        gp[11] = gbeta * kLn2 * at.beta;
+        // lobe directions R = (sin t cos p, sin t sin p, cos t)
 #pragma unroll
         for (int m = 0; m < M; ++m) {
           const float* L = p + 15 + 6 * m;
-          float* dL = gp + 15 + 6 * m;
-          const float rx = at.lobe_dir[m][0], ry = at.lobe_dir[m][1], rz = at.lobe_dir[m][2];
-          float dot = rx * vx + ry * vy + rz * vz;
-          if (dot > 0.0f) {
-            // w = dot^bm and d w / d dot = bm w / dot, with the MUFU log2/exp2
-            // (relative error ~1e-6, far inside the gradient tolerance)
-            float bm = at.lobe_beta[m];
-            float lw = lg2_approx(dot);
-            float wgt = ex2_approx(bm * lw);
-            dL[3] += wgt * gr;
-            dL[4] += wgt * gg;
-            dL[5] += wgt * gbl;
-            float gw = gr * L[3] + gg * L[4] + gbl * L[5];
-            dL[2] += gw * wgt * (lw * kLn2) * bm;
-            float ddot = gw * bm * wgt * __frcp_rn(dot);
-            dRm[m][0] += ddot * vx;
-            dRm[m][1] += ddot * vy;
-            dRm[m][2] += ddot * vz;
-            dvx += ddot * rx;
-            dvy += ddot * ry;
-            dvz += ddot * rz;
-          }
+          float st, ct, sp, cp;
+          sincosf(L[0], &st, &ct);
+          sincosf(L[1], &sp, &cp);
+          gp[15 + 6 * m + 0] = dRm[m][0] * ct * cp + dRm[m][1] * ct * sp - dRm[m][2] * st;
+          gp[15 + 6 * m + 1] = -dRm[m][0] * st * sp + dRm[m][1] * st * cp;
         }
-        float vd = vx * dvx + vy * dvy + vz * dvz;
-        gp[0] += (dvx - vx * vd) * il;
-        gp[1] += (dvy - vy * vd) * il;
-        gp[2] += (dvz - vz * vd) * il;
       }
     }
-    // scales: s = exp(log-scale)
+    if (i < n) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) gp[3 + k] = ds[k] * pg.s[k];
-    // Rq(q_hat) -> d q_hat -> d q
-    const float w = pg.q[0], x = pg.q[1], y = pg.q[2], z = pg.q[3];
-    float dw = 2.f * (-z * dR[1] + y * dR[2] + z * dR[3] - x * dR[5] - y * dR[6] + x * dR[7]);
-    float dx = 2.f * (y * dR[1] + z * dR[2] + y * dR[3] - 2.f * x * dR[4] - w * dR[5] + z * dR[6] +
-                      w * dR[7] - 2.f * x * dR[8]);
-    float dy = 2.f * (-2.f * y * dR[0] + x * dR[1] + w * dR[2] + x * dR[3] + z * dR[5] - w * dR[6] +
-                      z * dR[7] - 2.f * y * dR[8]);
-    float dz = 2.f * (-2.f * z * dR[0] - w * dR[1] + x * dR[2] + w * dR[3] - 2.f * z * dR[4] +
-                      y * dR[5] + x * dR[6] + y * dR[7]);
-    float qd = w * dw + x * dx + y * dy + z * dz;
-    float iq = 1.0f / pg.qn;
-    gp[6] = (dw - w * qd) * iq;
-    gp[7] = (dx - x * qd) * iq;
-    gp[8] = (dy - y * qd) * iq;
-    gp[9] = (dz - z * qd) * iq;
-    // opacity logit and shape
-    // dL/do = (1/o) sum (dL/dalpha) alpha; sigmoid' = o (1 - o)
-    gp[10] = go * (1.0f - at.o);
-    // dL/dbeta = ln 2 sum (dL/dalpha) alpha log2(1 - r^2); dbeta/db = beta
-    gp[11] = gbeta * kLn2 * at.beta;
-    // lobe directions R = (sin t cos p, sin t sin p, cos t)
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const float* L = p + 15 + 6 * m;
-      float st, ct, sp, cp;
-      sincosf(L[0], &st, &ct);
-      sincosf(L[1], &sp, &cp);
-      gp[15 + 6 * m + 0] = dRm[m][0] * ct * cp + dRm[m][1] * ct * sp - dRm[m][2] * st;
-      gp[15 + 6 * m + 1] = -dRm[m][0] * st * sp + dRm[m][1] * st * cp;
+      for (int k = 0; k < NP; ++k) gout[(size_t)k * pitch + i] = gp[k];
     }
   }
-#pragma unroll
-  for (int k = 0; k < NP; ++k) gout[(size_t)k * pitch + i] = gp[k];
 }
 
 }  // namespace
@@ -533,9 +580,15 @@ template <int M>
 static cudaError_t launch_project_bwd_m(const float* planes, int n, int pitch, const ViewTable& vt,
                                         const RenderOpts& ro, float* grad2d, float* gout,
                                         const int32_t* status, cudaStream_t s) {
-  int grid = (n + kBwdThreads - 1) / kBwdThreads;
-  if (grid < 1) return cudaSuccess;
-  launch_chained(k_project_bwd<M>, grid, kBwdThreads, 0, s, planes, n, pitch, vt, ro, grad2d, gout, status);
+  const int nblk = (n + kBwdThreads - 1) / kBwdThreads;
+  if (nblk < 1) return cudaSuccess;
+  constexpr size_t smem = bwd_smem(M);
+  const cudaError_t e = cudaFuncSetAttribute(k_project_bwd<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // CTAs an SM's 227 KB of shared memory hold (8 lobes: two)
+  constexpr int per_sm = (int)std::min<size_t>(kBwdBlocksPerSM, 227 * 1024 / (smem + 1024));
+  const int grid = std::min(nblk, device_sm_count() * per_sm);
+  launch_chained(k_project_bwd<M>, grid, kBwdThreads, smem, s, planes, n, pitch, vt, ro, grad2d, gout, status);
   return cudaGetLastError();
 }
 
