@@ -221,7 +221,7 @@ int beta_schedule(const beta_camera* cams, int32_t n_views, const beta_opts* opt
  * one 32-bit word per thread of the tile's raster CTA (which of the 32
  * primitives may cover its pixels: a pair of horizontally adjacent pixels or a
  * 2 x 2 quad, or one pixel in 8x4 tiles) and one per warp (which cover more
- * than 12 of its threads' pixels, 24 with quads): ((pair_capacity >> 5) +
+ * than 12 of its threads' pixels, 16 with pairs, 24 with quads): ((pair_capacity >> 5) +
  * total_tiles + 1) x (L x 33/32) x 4 bytes, L = tile pixels / 2 (/ 4 with quads;
  * tile pixels for 8x4 tiles).  Quads are used for 16 x 8 and larger tiles with
  * batches of at most tile pixels / 2 records when the views hold at least 16000

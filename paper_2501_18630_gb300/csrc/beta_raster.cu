@@ -710,13 +710,19 @@ struct PairBlock {
   static constexpr int WX = TW / BW;                 // blocks per tile row
   static constexpr int NT = TW * TH / (2 * NP);      // threads of a tile's CTA
   static constexpr int NW = NT / 32;
-  // Records covering more lanes than this are reduced across the warp.  With
-  // quads a lane's atomics serve four pixels, so more lanes add their own: 12 /
-  // 16 / 20 / 24 / 28 took 3.17 / 2.96 / 2.87 / 2.84 / 2.82 ms (one launch, 1M
-  // Betas x 16 x 1080p) and 18.4 / 16.1 / 14.7 / 14.2 / 14.7 ms (backward, 6M x 8
-  // x 4K).
-  static constexpr int kWide = NP == 1 ? kLaneAtomics : 24;
 };
+
+// Records covering more of a warp's lanes than this are reduced across the warp
+// in the backward, the others add their terms lane by lane; the one launch and
+// the separate backward have their own best.  One pair, 12 / 16 / 20 / 24: one
+// launch of 3M Betas x 16 mixed views (8x8) 8.47 / 8.05 / 8.00 / 8.11 ms,
+// backward 6.32 / 6.16 / 6.50 / 6.90; 6M x 2 x 4K (16x16) 8.03 / 7.42 / 7.14 / 7.12
+// and 5.20 / 4.78 / 5.14 / 5.77.  Quads, 12 / 16 / 20 / 24 / 28: one launch of 1M x
+// 16 x 1080p (16x8) 3.17 / 2.96 / 2.87 / 2.84 / 2.82, backward of 6M x 8 x 4K 18.4 /
+// 16.1 / 14.7 / 14.2 / 14.7.
+constexpr int wide_lanes(int np, bool one_launch) {
+  return np == 1 ? (one_launch ? 20 : 16) : (one_launch ? 28 : 24);
+}
 
 // CTAs per SM asked of the register allocator.  One pair: 1152 threads (56
 // registers) where the record buffers of 64-record batches leave room for that
@@ -724,7 +730,7 @@ struct PairBlock {
 // threads: one launch 3.44 / 3.43 / 3.59 ms, backward of 6M x 8 x 4K 20.66 / 20.28
 // / 21.00 ms: packed pairs take aligned register pairs, and 48 registers spill).
 // Two pairs: 704 threads (80 registers; 1024 / 800 / 704 / 640: 3.93 / 3.34 /
-// 3.17 / 3.2 ms with kWide 12), 768 for larger batches.
+// 3.17 / 3.2 ms with 12 wide lanes), 768 for larger batches.
 constexpr int pair_ctas_per_sm(int tw, int th, int S, int np) {
   return min_blocks(tw * th / (2 * np), np == 1 ? (S <= 64 ? 1152 : 1024) : (S <= 64 ? 704 : 768));
 }
@@ -876,7 +882,7 @@ struct PairFwdState {
 // so that a backward can start from the last batch still in s_rec.  Returns
 // with every copy landed; the caller synchronises the CTA before s_rec is
 // staged again.
-template <int TW, int TH, int S, int NP>
+template <int TW, int TH, int S, int NP, int WIDE>
 __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], uint32_t* ridx,
                                               const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
                                               uint32_t start, uint32_t end, uint32_t* hslot, int hm_chunks,
@@ -955,7 +961,7 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
       const int jc = (int)((base - start + c) >> 5);
       if (hslot && jc < hm_chunks) {
         uint32_t* slot = hslot + (size_t)jc * (NT + NW);
-        const uint32_t wide = __ballot_sync(0xffffffffu, __popc(cov) > PB::kWide);
+        const uint32_t wide = __ballot_sync(0xffffffffu, __popc(cov) > WIDE);
         slot[tid] = mine;
         if (lane == 0) slot[NT + warp] = wide;
       }
@@ -1164,7 +1170,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     uint32_t* const hslot = hit_tile<NT>(hm, hm_words, start, end, g);
     if (target) copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
     PairFwdState<NP> fs;
-    pair_fwd_walk<TW, TH, S, NP>(s_rec, nullptr, rec, vals, start, end, hslot, INT_MAX, (float)x, (float)y, (float)bx,
+    pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, false)>(s_rec, nullptr, rec, vals, start, end, hslot, INT_MAX, (float)x, (float)y, (float)bx,
                              (float)by, in, t_eps, amax, fs);
     float gv[6 * NP];
     const float l1 =
@@ -1252,13 +1258,13 @@ __device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x
 // (the forward's from hslot for the list's first hm_chunks chunks, else the
 // cover pass again), then every lane's
 // walk of its records in reverse list order at its pixels with three vector
-// atomics per record, and records covering more than kLaneAtomics of the
-// warp's lanes by the whole warp (reduce-scatter, one atomic per value).
+// atomics per record, and records covering more than WIDE of the warp's lanes
+// by the whole warp (reduce-scatter, one atomic per value).
 // When the first batch it needs is reuse_batch, which a forward walk left
 // complete in s_rec[reuse_buf] with its indices in s_ridx[reuse_buf], it
 // starts from there instead of staging it again (reuse_batch = -1: never).
 // Returns with every copy landed and the CTA synchronised.
-template <int TW, int TH, int S, int NP>
+template <int TW, int TH, int S, int NP, int WIDE>
 __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], uint32_t (&s_ridx)[2][S],
                                               uint32_t (&s_wmax)[PairBlock<TW, TH, NP>::NW],
                                               const float4* __restrict__ rec, const uint32_t* __restrict__ lst,
@@ -1344,7 +1350,7 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         const int idx = c + lane;
         const uint32_t cov = (idx < cnt && (uint32_t)(lo + idx) < wmax)
                                  ? pair_cover<PB::BW, NP>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf) : 0u;
-        wide = __ballot_sync(0xffffffffu, __popc(cov) > PB::kWide);
+        wide = __ballot_sync(0xffffffffu, __popc(cov) > WIDE);
         mine = transpose32(cov, lane);
       }
       if (hslot && j >= 1 && j - 1 < hm_chunks) {     // the next chunk's stored masks, one chunk ahead
@@ -1456,7 +1462,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
         bs.gz[i] = pack2(gz[0], gz[1]);
       }
     }
-    pair_bwd_walk<TW, TH, S, NP>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX, grad2d, (float)x, (float)y,
+    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, false)>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX, grad2d, (float)x, (float)y,
                              (float)bx, (float)by, amax, my_field, bs, -1, 0);
   }
   leave<PERSIST>(ctr);
@@ -1511,7 +1517,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     const uint32_t start = ranges[g], end = ranges[g + 1];
     copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
     PairFwdState<NP> fs;
-    pair_fwd_walk<TW, TH, S, NP>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
+    pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
                              byf, in, t_eps, amax, fs);
     float gv[6 * NP];
     const float l1 = pair_fwd_out<NT, NP>(fs, vt, v, x, y, in, true, s_tgt, color, Tout, ncontrib, dLdC, gv);
@@ -1537,7 +1543,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
       bs.gy[i] = pack2(gv[6 * i + 1], gv[6 * i + 4]);
       bs.gz[i] = pack2(gv[6 * i + 2], gv[6 * i + 5]);
     }
-    pair_bwd_walk<TW, TH, S, NP>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,
+    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,
                              bxf, byf, amax, my_field, bs, fs.walked_batch, fs.walked_buf);
   }
   leave<PERSIST>(ctr);
