@@ -729,10 +729,13 @@ constexpr int wide_lanes(int np, bool one_launch) {
 // many CTAs, 1024 (64) for larger batches (at 16x8 / 64, 1280 / 1152 / 1024
 // threads: one launch 3.44 / 3.43 / 3.59 ms, backward of 6M x 8 x 4K 20.66 / 20.28
 // / 21.00 ms: packed pairs take aligned register pairs, and 48 registers spill).
-// Two pairs: 704 threads (80 registers; 1024 / 800 / 704 / 640: 3.93 / 3.34 /
-// 3.17 / 3.2 ms with 12 wide lanes), 768 for larger batches.
-constexpr int pair_ctas_per_sm(int tw, int th, int S, int np) {
-  return min_blocks(tw * th / (2 * np), np == 1 ? (S <= 64 ? 1152 : 1024) : (S <= 64 ? 704 : 768));
+// Two pairs: the backward and the one launch 704 threads (80 registers; 1024 /
+// 800 / 704 / 640: 3.93 / 3.34 / 3.17 / 3.2 ms with 12 wide lanes), 768 for larger
+// batches; the forward, which needs less, 800 (72 registers; 1M Betas x 16 x 1080p
+// 1.15 -> 1.09 ms, 6M x 8 x 4K 6.97 -> 6.69 ms).
+constexpr int pair_ctas_per_sm(int tw, int th, int S, int np, bool forward_only = false) {
+  return min_blocks(tw * th / (2 * np),
+                    np == 1 ? (S <= 64 ? 1152 : 1024) : (S > 64 ? 768 : forward_only ? 800 : 704));
 }
 
 // Two floats in one 64-bit register (the lane's two pixels: lo = pixel 0) and
@@ -1142,7 +1145,7 @@ __device__ __forceinline__ void tile_l1_partial(float l1, float (&s_l1)[NW], flo
 }
 
 template <int TW, int TH, int S, int NP, bool PERSIST>
-__global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_fwd2(
+__global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP, true)) k_raster_fwd2(
     ViewTable vt, RenderOpts ro, const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
     const uint32_t* __restrict__ ranges, float* __restrict__ color, float* __restrict__ Tout,
     uint32_t* __restrict__ ncontrib, const int32_t* __restrict__ status, uint32_t* ctr,
