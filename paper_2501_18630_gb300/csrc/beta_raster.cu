@@ -9,9 +9,9 @@
 //
 // Layout: one CTA per TW x TH tile.  In 8 x 4 tiles (k_raster_fwd /
 // k_raster_bwd) every thread owns one pixel and warp w an 8 x 4 block; in the
-// others (k_raster_fwd2 / k_raster_bwd2, below) every thread owns two
-// horizontally adjacent pixels and the warp a 16 x 4 or 8 x 8 block, "pixel"
-// reading "pixel pair" in what follows.  Records of the tile's list are
+// others (k_raster_fwd2 / k_raster_bwd2, below) every thread owns a pair of
+// horizontally adjacent pixels, or a 2 x 2 quad, and the warp a 16 x 4, 8 x 8 or
+// 16 x 8 block, "pixel" reading "lane's pixels" in what follows.  Records of the tile's list are
 // staged S at a time in shared memory (double-buffered cp.async, one batch
 // ahead).  Each warp walks the staged records 32 at a time in two passes.
 // First, lane k works out which
@@ -29,9 +29,9 @@
 // last-contributor position down, recovering T_k = T_{k+1} / (1 - alpha_k)
 // and the suffix colour S (as g . S), and produces per-record 2D gradients
 // (d mu', d Sigma', d o, d beta, d colour): every lane adds its ten values
-// with three 16-byte vector atomics, except for records covering more than
-// 12 of the block's lanes, which the warp processes together and sums with a
-// 12-shuffle reduce-scatter, one atomic per value.
+// with three vector atomics, except for records covering more than 12 to 28 of
+// the block's lanes (by kernel), which the warp processes together and sums
+// with a 12-shuffle reduce-scatter, one atomic per value.
 //
 // Scheduling: with a schedule buffer (beta_schedule) the raster kernels are
 // persistent -- a grid sized to the SMs takes tiles from a global counter in
@@ -171,14 +171,15 @@ __device__ __forceinline__ void stage_record(float4* dst, const float4* __restri
 
 // Records covering more than this many pixels of a warp's block are reduced
 // across the warp before their atomics in the backward; for the others every
-// lane adds its own terms.
+// lane adds its own terms (the one-pixel kernels; wide_lanes gives the others').
 constexpr int kLaneAtomics = 12;
 
 // Hit masks (optional, written by the forward, read by the backward): per
 // tile g, per chunk j of 32 list positions, NT words (word t: the records of
 // the chunk that may cover pixel t of the tile, bit k = position 32 j + k,
 // from block_cover and the transpose) and NW words (word w: the chunk's
-// records covering more than kLaneAtomics pixels of warp w's block).  Chunk j
+// records covering more lanes of warp w's block than that kernel lets add their
+// own terms, kLaneAtomics or wide_lanes).  Chunk j
 // of tile g is slot (ranges[g] >> 5) + g + j, so the slots of the tiles never
 // overlap and (pairs >> 5) + tiles + 1 slots hold every list.  A tile whose
 // slots do not all fit in the buffer uses none (the backward recomputes its
@@ -1051,24 +1052,32 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
 
 // Epilogue of the pixel-pair forward at the lane's pixels (x + h, y + i) of view
 // v: the colour C + T bg to color; T and the last contributor to Tout / ncontrib
-// when those are given; with a target (tgt[ch][2 NP tid + q]: pixel q, channel
-// ch, landed in shared memory) the L1 term, whose gradient
+// when those are given; with a target the L1 term, whose gradient
 // sign(C - target) / (3 H W) goes to dLdC when given and to gv (pixel q,
 // channel ch at gv[3 q + ch]; zero off the image or without a target).
-// Returns the lane's sum of |C - target|.
-template <int NT, int NP>
+// Returns the lane's sum of |C - target|.  The targets are loaded here, all at
+// once, rather than copied to shared memory while the tile composites: 1.5 KB
+// less per 16 x 8 CTA is worth more than the hidden latency (16 x 1080p of the
+// sheets: forward 1166 -> 1157 us, one launch 2816 -> 2801; prefetched to L2
+// at the tile's start 1167 / 2807).
+template <int NP>
 __device__ __forceinline__ float pair_fwd_out(const PairFwdState<NP>& st, const ViewTable& vt, int v, int x, int y,
-                                              const bool (&in)[2 * NP], bool with_target,
-                                              const float (&tgt)[3][2 * NP * NT], float* __restrict__ color,
+                                              const bool (&in)[2 * NP], const float* __restrict__ target,
+                                              float* __restrict__ color,
                                               float* __restrict__ Tout, uint32_t* __restrict__ ncontrib,
                                               float* __restrict__ dLdC, float (&gv)[6 * NP]) {
-  const int tid = threadIdx.x;
   const int W = vt.v[v].width, H = vt.v[v].height;
   const int64_t HW = (int64_t)W * H;
   const int64_t pix = vt.v[v].pix_off + (int64_t)y * W + x;
   const int64_t o = 3 * vt.v[v].pix_off + (int64_t)y * W + x;
   const float scale = vt.v[v].l1_scale;
   float l1 = 0.0f;
+  float tgt[2 * NP][3];
+#pragma unroll
+  for (int q = 0; q < 2 * NP; ++q)
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch)
+      tgt[q][ch] = target && in[q] ? target[o + (int64_t)(q / 2) * W + (q & 1) + ch * HW] : 0.0f;
 #pragma unroll
   for (int q = 0; q < 2 * NP; ++q) {
 #pragma unroll
@@ -1081,11 +1090,11 @@ __device__ __forceinline__ float pair_fwd_out(const PairFwdState<NP>& st, const 
     for (int ch = 0; ch < 3; ++ch) color[o + at + ch * HW] = c[ch];
     if (Tout) Tout[pix + at] = T;
     if (ncontrib) ncontrib[pix + at] = st.last[q];
-    if (with_target) {
+    if (target) {
       // the per-pixel L1 term and its gradient, as beta_l1_loss computes them
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
-        const float d = c[ch] - tgt[ch][2 * NP * tid + q];
+        const float d = c[ch] - tgt[q][ch];
         l1 += fabsf(d);
         const float gd = d > 0.0f ? scale : (d < 0.0f ? -scale : 0.0f);
         gv[3 * q + ch] = gd;
@@ -1109,20 +1118,6 @@ __device__ __forceinline__ void lane_pixels(const ViewDev& V, int tx, int ty, in
   y = by + NP * (lane / PB::PC);
 #pragma unroll
   for (int q = 0; q < 2 * NP; ++q) in[q] = x + (q & 1) < V.width && y + q / 2 < V.height;
-}
-
-// Starts the copies of the lane's target values into shared memory.
-template <int NT, int NP>
-__device__ __forceinline__ void copy_targets(const ViewDev& V, const float* __restrict__ target, int x, int y,
-                                             const bool (&in)[2 * NP], float (&tgt)[3][2 * NP * NT]) {
-  const int64_t HW = (int64_t)V.width * V.height;
-  const int64_t o = 3 * V.pix_off + (int64_t)y * V.width + x;
-#pragma unroll
-  for (int ch = 0; ch < 3; ++ch)
-#pragma unroll
-    for (int q = 0; q < 2 * NP; ++q)
-      if (in[q])
-        cp_async4(&tgt[ch][2 * NP * threadIdx.x + q], target + o + (int64_t)(q / 2) * V.width + (q & 1) + ch * HW);
 }
 
 // The CTA's sum of the lanes' l1 in a fixed order (warp shuffles, then the
@@ -1157,7 +1152,6 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
   static_assert(pair_tiles(TW, TH) && TH % PB::BH == 0 && NT % 32 == 0, "tile must hold whole pair blocks");
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ float s_l1[NW];
-  __shared__ float s_tgt[3][2 * NP * NT];   // the pixels' targets, copied in while the tile composites
   __shared__ int s_item;
   if (*status != 0) return;
   const float t_eps = ro.t_eps, amax = ro.alpha_max;
@@ -1171,13 +1165,12 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     lane_pixels<TW, TH, NP>(vt.v[v], tx, ty, bx, by, x, y, in);
     const uint32_t start = ranges[g], end = ranges[g + 1];
     uint32_t* const hslot = hit_tile<NT>(hm, hm_words, start, end, g);
-    if (target) copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
     PairFwdState<NP> fs;
     pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, false)>(s_rec, nullptr, rec, vals, start, end, hslot, INT_MAX, (float)x, (float)y, (float)bx,
                              (float)by, in, t_eps, amax, fs);
     float gv[6 * NP];
     const float l1 =
-        pair_fwd_out<NT, NP>(fs, vt, v, x, y, in, target != nullptr, s_tgt, color, Tout, ncontrib, dLdC, gv);
+        pair_fwd_out<NP>(fs, vt, v, x, y, in, target, color, Tout, ncontrib, dLdC, gv);
     // tile partial sum of |C - target|, reduced in a fixed order
     if (target) tile_l1_partial<NW>(l1, s_l1, l1_partial + g);
   }
@@ -1478,8 +1471,8 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
 // memory between the two and the backward's record gathers find the records
 // the forward just staged in L2.  T, the last contributors and dL/dC are
 // stored only when their buffers are given.  The forward's cover masks of
-// each list's first kStepMaskChunks(NT) chunks of 32 records (192 records at
-// 64 threads, 1.5 KB) are kept in shared memory; the backward repeats the
+// each list's first kStepMaskChunks(NT) chunks of 32 records (192 records up to
+// 64 threads: 0.8 KB at 32) are kept in shared memory; the backward repeats the
 // cover passes of later chunks.  Colour, L1 partials, T, last contributors and dL/dC
 // equal k_raster_fwd2's bit for bit, and every per-record term the backward
 // adds equals k_raster_bwd2's (the sums differ only by the order of the
@@ -1500,7 +1493,6 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ uint32_t s_ridx[2][S];
   __shared__ float s_l1[NW];
-  __shared__ float s_tgt[3][2 * NP * NT];   // the pixels' targets, copied in while the tile composites
   __shared__ uint32_t s_wmax[NW];
   __shared__ uint32_t s_hm[kStepMaskChunks(NT) * (NT + NW)];   // cover masks, hit-mask slot layout
   __shared__ int s_item;
@@ -1518,12 +1510,11 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     lane_pixels<TW, TH, NP>(vt.v[v], tx, ty, bx, by, x, y, in);
     const float xf = (float)x, yf = (float)y, bxf = (float)bx, byf = (float)by;
     const uint32_t start = ranges[g], end = ranges[g + 1];
-    copy_targets<NT, NP>(vt.v[v], target, x, y, in, s_tgt);
     PairFwdState<NP> fs;
     pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
                              byf, in, t_eps, amax, fs);
     float gv[6 * NP];
-    const float l1 = pair_fwd_out<NT, NP>(fs, vt, v, x, y, in, true, s_tgt, color, Tout, ncontrib, dLdC, gv);
+    const float l1 = pair_fwd_out<NP>(fs, vt, v, x, y, in, target, color, Tout, ncontrib, dLdC, gv);
     // also the barrier after which no warp still reads the forward's s_rec
     // and every cover mask in s_hm is visible to the whole CTA
     tile_l1_partial<NW>(l1, s_l1, l1_partial + g);
