@@ -1471,13 +1471,22 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
 // memory between the two and the backward's record gathers find the records
 // the forward just staged in L2.  T, the last contributors and dL/dC are
 // stored only when their buffers are given.  The forward's cover masks of
-// each list's first kStepMaskChunks(NT) chunks of 32 records (192 records up to
-// 64 threads: 0.8 KB at 32) are kept in shared memory; the backward repeats the
-// cover passes of later chunks.  Colour, L1 partials, T, last contributors and dL/dC
+// each list's first kStepMaskChunks(NT, NP) chunks of 32 records are kept in
+// shared memory (12 chunks, 1.6 KB, for a quad tile of one warp); the backward
+// repeats the cover passes of later chunks.  Colour, L1 partials, T, last contributors and dL/dC
 // equal k_raster_fwd2's bit for bit, and every per-record term the backward
 // adds equals k_raster_bwd2's (the sums differ only by the order of the
 // floating-point atomics).
-constexpr int kStepMaskChunks(int nt) { return nt >= 384 ? 1 : 384 / nt < 6 ? 384 / nt : 6; }
+//
+// More chunks save cover passes and cost L1 cache.  16 x 1080p of the sheets in
+// 16 x 8 quads (one warp): 4 / 6 / 8 / 12 / 16 / 24 chunks 2826 / 2801 / 2790 /
+// 2786 / 2799 / 2839 us; 8 x 4K 20.27 / 20.17 / 20.07 / 19.92 / 19.95 / 20.19
+// ms.  3M mixed views in 8 x 8 pairs (one warp): 7972 / 7954 / 7945 / 7978 /
+// 8004 / 8088 us.  8 x 4K in 16 x 16 quads (two warps): 6 / 8 chunks 21.70 /
+// 21.57 ms.
+constexpr int kStepMaskChunks(int nt, int np) {
+  return nt <= 32 ? (np == 2 ? 12 : 8) : np == 2 && nt <= 64 ? 8 : nt <= 64 ? 6 : nt >= 384 ? 1 : 384 / nt;
+}
 
 template <int TW, int TH, int S, int NP, bool PERSIST>
 __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_step2(
@@ -1494,7 +1503,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
   __shared__ uint32_t s_ridx[2][S];
   __shared__ float s_l1[NW];
   __shared__ uint32_t s_wmax[NW];
-  __shared__ uint32_t s_hm[kStepMaskChunks(NT) * (NT + NW)];   // cover masks, hit-mask slot layout
+  __shared__ uint32_t s_hm[kStepMaskChunks(NT, NP) * (NT + NW)];   // cover masks, hit-mask slot layout
   __shared__ int s_item;
   if (*status != 0) return;
   const int lane = threadIdx.x & 31;
@@ -1511,7 +1520,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
     const float xf = (float)x, yf = (float)y, bxf = (float)bx, byf = (float)by;
     const uint32_t start = ranges[g], end = ranges[g + 1];
     PairFwdState<NP> fs;
-    pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT), xf, yf, bxf,
+    pair_fwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, &s_ridx[0][0], rec, vals, start, end, s_hm, kStepMaskChunks(NT, NP), xf, yf, bxf,
                              byf, in, t_eps, amax, fs);
     float gv[6 * NP];
     const float l1 = pair_fwd_out<NP>(fs, vt, v, x, y, in, target, color, Tout, ncontrib, dLdC, gv);
@@ -1537,7 +1546,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
       bs.gy[i] = pack2(gv[6 * i + 1], gv[6 * i + 4]);
       bs.gz[i] = pack2(gv[6 * i + 2], gv[6 * i + 5]);
     }
-    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT), grad2d, xf, yf,
+    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, true)>(s_rec, s_ridx, s_wmax, rec, vals + start, s_hm, kStepMaskChunks(NT, NP), grad2d, xf, yf,
                              bxf, byf, amax, my_field, bs, fs.walked_batch, fs.walked_buf);
   }
   leave<PERSIST>(ctr);
