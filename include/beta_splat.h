@@ -93,7 +93,7 @@ typedef struct {
 /* Render options (host struct).  beta_default_opts() fills the defaults. */
 typedef struct {
   int32_t tile_w, tile_h; /* pixel tile: 8x4, 8x8, 16x8, 16x16 (default) or 32x16 */
-  int32_t batch_s;        /* records staged per raster batch: 64, 128 or 256 */
+  int32_t batch_s;        /* records staged per raster batch, at most: 64, 128 or 256 */
   int32_t color_mode;     /* 0: c0 + lobes, 1: c0 only (diffuse), 2: lobes only (specular) */
   float t_eps;            /* stop before a primitive once T < t_eps (2^-19)   */
   float alpha_max;        /* alpha = min(alpha_max, o B)   (0.99)             */
@@ -223,9 +223,9 @@ int beta_schedule(const beta_camera* cams, int32_t n_views, const beta_opts* opt
  * 2 x 2 quad, or one pixel in 8x4 tiles) and one per warp (which cover more
  * than 12 of its threads' pixels, 16 with pairs, 24 with quads): ((pair_capacity >> 5) +
  * total_tiles + 1) x (L x 33/32) x 4 bytes, L = tile pixels / 2 (/ 4 with quads;
- * tile pixels for 8x4 tiles).  Quads are used for 16 x 8 and larger tiles with
- * batches of at most tile pixels / 2 records when the views hold at least 16000
- * blocks of 128 pixels.  0 for invalid arguments. */
+ * tile pixels for 8x4 tiles).  Quads are used for 16 x 8 and larger tiles
+ * when the views hold at least 16000 blocks of 128 pixels, 64000 with batches of
+ * more than tile pixels / 2 records.  0 for invalid arguments. */
 size_t beta_hit_mask_bytes(const beta_camera* cams /* host */, int32_t n_views, const beta_opts* opt,
                            int64_t pair_capacity);
 

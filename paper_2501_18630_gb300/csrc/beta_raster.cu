@@ -686,21 +686,38 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
 // others (8 x 4) the one-pixel-per-lane ones; the hit-mask layout follows.
 constexpr bool pair_tiles(int tw, int th) { return th % (tw % 16 == 0 ? 4 : 8) == 0; }
 
-// Pairs a lane owns.  Two need 16 x 8 blocks and record batches of at most two
-// records per thread (larger ones leave room for too few CTAs: 16x16 / 256
-// forward 1.38 -> 1.59 ms at 1M Betas x 16 x 1080p), and enough blocks to fill
-// the chip with half the warps.  At 16x8 / 64 the one launch takes, NP 1 / 2: 9840
+// Pairs a lane owns.  Two need 16 x 8 blocks and enough of them to fill the chip
+// with half the warps.  At 16x8 / 64 the one launch takes, NP 1 / 2: 9840
 // blocks (4 x 641x479, clustered lists) 130 / 151 us; 16200 (one 1080p view)
 // 253 / 223; 32400 466 / 407; 64800 877 / 752; at 32x16 / 128, 10080 blocks
-// 199 / 220 us, 16320 392 / 333.
-constexpr int kQuadBlocks = 16000;
-constexpr bool quad_shape(int tw, int th, int S) {
-  return tw % 16 == 0 && th % 8 == 0 && S <= 2 * (tw * th / 4);
-}
+// 199 / 220 us, 16320 392 / 333.  Batches of more than two records per quad
+// thread, asked for where lists are long, need four times as many, for a
+// forward by itself to gain too: 16x16 / 256, 16320 blocks, forward and one
+// launch 108 / 113 and 272 / 247 us; 32640 200 / 206 and 521 / 464 (3.1M Betas
+// 550 / 592 and 1615 / 1512); 64800 (6M Betas x 4K) 1108 / 1106 and 3666 / 2981;
+// 65280, persistent, 420 / 370 and 1006 / 803; 129600 2128 / 2088 and 7166 / 5733.
+constexpr int kQuadBlocks = 16000, kQuadBlocksLarge = 64000;
+constexpr bool quad_shape(int tw, int th) { return tw % 16 == 0 && th % 8 == 0; }
 inline int lane_pairs(const RenderOpts& ro, int total_tiles) {
-  return quad_shape(ro.tile_w, ro.tile_h, ro.batch_s) &&
-                 (int64_t)total_tiles * (ro.tile_w * ro.tile_h / 128) >= kQuadBlocks
+  const int px = ro.tile_w * ro.tile_h;
+  return quad_shape(ro.tile_w, ro.tile_h) &&
+                 (int64_t)total_tiles * (px / 128) >= (ro.batch_s <= px / 2 ? kQuadBlocks : kQuadBlocksLarge)
              ? 2 : 1;
+}
+
+// Records the kernels stage at a time for batches of S: fewer than S where the
+// shared memory does more good as L1 cache.  One warp stages 32 (16 x 1080p in
+// 16x8 quads, forward 1157 -> 1124 us; 3M mixed views in 8x8 pairs, forward
+// 2565 -> 2449, one launch 7949 -> 7785, backward 6141 -> 6119), except where
+// quads walk backwards (backward 1970 -> 1991 us, one launch of 8 x 4K 19.9 ->
+// 20.1 ms: 64).  Larger CTAs of quads stage two records per thread at most: with
+// 256-record batches too few fit (16x16 forward 1.38 -> 1.59 ms against pairs);
+// one per thread is slower (16x16 / 128, 8 x 4K one launch 21.5 -> 22.0 ms).
+// Pairs keep S (16x16 / 256 at 128, 64: 4 x 641x479 120 -> 123, 129 us).
+constexpr int staged(int tw, int th, int S, int np, bool forward_only) {
+  const int nt = tw * th / (2 * np);
+  const int most = nt <= 32 ? (np == 1 || forward_only ? 32 : 64) : np == 1 ? S : 2 * nt;
+  return S < most ? S : most;
 }
 
 template <int TW, int TH, int NP>
@@ -1778,9 +1795,9 @@ cudaError_t fwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
                       uint32_t* n_contrib, const int32_t* status, uint32_t* sched, const float* target,
                       float* dL_dcolor, float* l1_partial, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    if constexpr (quad_shape(TW, TH, S))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return fwd_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
-    return fwd_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
+    if constexpr (quad_shape(TW, TH))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return fwd_pairs<TW, TH, staged(TW, TH, S, 2, true), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
+    return fwd_pairs<TW, TH, staged(TW, TH, S, 1, true), 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
   } else {
     if (sched) {
       auto k = k_raster_fwd<TW, TH, S, true>;
@@ -1817,9 +1834,9 @@ cudaError_t bwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
                       const uint32_t* n_contrib, const float* dL_dcolor, float* grad2d,
                       const int32_t* status, uint32_t* sched, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    if constexpr (quad_shape(TW, TH, S))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return bwd_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
-    return bwd_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
+    if constexpr (quad_shape(TW, TH))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return bwd_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
+    return bwd_pairs<TW, TH, staged(TW, TH, S, 1, false), 1>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
   } else {
     if (sched) {
       auto k = k_raster_bwd<TW, TH, S, true>;
@@ -1857,9 +1874,9 @@ cudaError_t step_shape(const ViewTable& vt, const RenderOpts& ro, const float4* 
                        const int32_t* status, uint32_t* sched, const float* target, float* dL_dcolor,
                        float* l1_partial, float* grad2d, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
-    if constexpr (quad_shape(TW, TH, S))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return step_pairs<TW, TH, S, 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
-    return step_pairs<TW, TH, S, 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
+    if constexpr (quad_shape(TW, TH))
+      if (lane_pairs(ro, vt.total_tiles) == 2) return step_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
+    return step_pairs<TW, TH, staged(TW, TH, S, 1, false), 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
   } else {
     return cudaErrorInvalidValue;   // 8 x 4 tiles have no pixel-pair kernels
   }

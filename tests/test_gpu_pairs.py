@@ -106,6 +106,37 @@ def test_quad_kernels_equal_one_pixel_kernels(odd, tile, s, fused, persistent):
         assert np.max(np.abs(np.where(fin, g1 - g0, 0.0)) / scale) < 1e-4
 
 
+@pytest.mark.parametrize("tile,s,fused,persistent", [((16, 8), 128, True, False), ((16, 8), 256, False, True),
+                                                     ((16, 16), 256, True, True), ((16, 16), 256, False, False)])
+def test_quads_of_large_batches_equal_pairs_of_one_warp(tile, s, fused, persistent):
+    """Batches of more records than a quad CTA stages at a time, on views large
+    enough for quads with them; 8x8 tiles (one warp, pairs) as the reference."""
+    cam = scenes.pinhole(*scenes.look_at((0.0, 0.0, -3.0)), 4097, 2041)
+    assert -(-4097 // 16) * -(-2041 // 8) >= 64000
+    rng = np.random.Generator(np.random.PCG64(12))
+    p = torch.from_numpy(scenes.random_scene(400, 1, rng, mean_lo=-0.6, mean_hi=0.6, logscale=(-2.6, 0.5))).cuda()
+    target = torch.from_numpy(scenes.target_images([cam], seed=3)[0].reshape(-1)).cuda()
+    gc.ensure_built()
+    out = []
+    for t, b, per in (((8, 8), 64, False), (tile, s, persistent)):
+        r = render.Rasterizer(400, p.shape[1], 1, [cam], _lib.default_opts(tile_w=t[0], tile_h=t[1], batch_s=b),
+                              persistent=per, hit_masks=True)
+        r.forward(p)
+        grad = torch.zeros_like(p)
+        if fused:
+            r.raster_fwd_bwd_l1(p, target)
+        else:
+            r.raster_fwd_l1(p, target)
+            r.raster_bwd(p, r.dL_dcolor)
+        r.project_bwd(p, grad)
+        torch.cuda.synchronize()
+        out.append((r.color.cpu().numpy(), grad.cpu().numpy()))
+    np.testing.assert_array_equal(out[1][0], out[0][0])
+    g0, g1 = out[0][1], out[1][1]
+    # fp32 terms summed in another order
+    assert np.max(np.abs(g1 - g0) / (np.max(np.abs(g0), axis=1, keepdims=True) + 1e-30)) < 1e-4
+
+
 @pytest.mark.parametrize("w,h,tile", [(1, 1, (8, 4)), (257, 129, (16, 16)), (1024, 512, (8, 4)), (1032, 512, (8, 4))])
 def test_schedule_orders_every_tile_longest_first(w, h, tile):
     """One CTA up to 16384 tiles, three launches above: a permutation of the tiles
