@@ -875,10 +875,11 @@ __device__ __forceinline__ f32x2 rec_om(float4 f0, float4 f1, f32x2 dx, f32x2 u,
   return fma2(r2, both2(-1.0f), both2(1.0f));
 }
 
-// Is a record's colour free of infinities and NaN?  (A finite sum that
-// overflows reads as not finite, which only costs the slower path.)
-__device__ __forceinline__ bool finite_colour(float4 f2) {
-  return fabsf((f2.y + f2.z) + f2.w) < __int_as_float(0x7f800000);
+// Is |x| + |y| + |z| below 2^60 (no infinity, no NaN)?  Products of a colour and a
+// dL/dC for which it is cannot overflow, nor can their sums over a list, so a zero
+// alpha or weight takes them out; anything else is selected out, pixel by pixel.
+__device__ __forceinline__ bool tame(float x, float y, float z) {
+  return fabsf(x) + fabsf(y) + fabsf(z) < 1152921504606846976.0f;
 }
 
 // Per-lane state of the pixel-pair forward after a tile's walk: transmittance,
@@ -889,7 +890,7 @@ struct PairFwdState {
   float T[2 * NP], C[2 * NP][3];
   uint32_t last[2 * NP];
   int walked_batch, walked_buf;   // the last batch the walk composited and its s_rec buffer (-1: none)
-  bool odd_colours;               // a record the warp walked has a non-finite colour (warp-uniform)
+  bool odd_colours;               // a record the warp walked has a colour that is not tame (warp-uniform)
 };
 
 // Forward walk of one tile's list [start, end) at the lane's pixel pairs (xf,
@@ -974,7 +975,7 @@ __device__ __forceinline__ void pair_fwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
       bool odd = false;
       if (idx < cnt) {
         cov = pair_cover<PB::BW, NP>(s_rec[buf][idx][0], s_rec[buf][idx][1], bxf, byf);
-        odd = !finite_colour(s_rec[buf][idx][2]);
+        odd = !tame(s_rec[buf][idx][2].y, s_rec[buf][idx][2].z, s_rec[buf][idx][2].w);
       }
       uint32_t mine = transpose32(cov, lane);
       odd = __any_sync(0xffffffffu, odd);
@@ -1201,15 +1202,17 @@ template <int NP>
 struct PairBwdState {
   f32x2 T2[NP], NG2[NP], gx[NP], gy[NP], gz[NP];
   uint32_t nl[2 * NP];
-  int odd_colours;   // 1 / 0: some / none of the records has a non-finite colour; -1: not known
+  int odd_colours;   // 1 / 0: some / none of the records has a colour that is not tame; -1: not known
 };
 
 // The lane's pixels' terms (bwd_terms with ZERO) of a staged record, summed over
 // them into G; T2 and NG2 move on at the pixels where the record lies before the
 // last contributor (pos < nl, and `mine`) and covers the pixel.  There alpha
-// takes its value, elsewhere zero, so that 1 / (1 - alpha) = 1 leaves T and a
-// zero weight leaves NG2 and the colour terms (with a non-finite colour, `odd`,
-// g . c is dropped there).  Returns whether any pixel is covered.
+// takes its value, elsewhere zero, so that 1 / (1 - alpha) = 1 leaves T (the
+// approximate reciprocal of 1 is 1 on sm_103a: the tests walk a pixel past 1500
+// records; T + wgt or a select in its place take 1.4 to 2% of the one launch) and a
+// zero weight leaves NG2 and the colour terms (dL/dC is tame; with a colour that is
+// not, `odd`, g . c is dropped there).  Returns whether any pixel is covered.
 template <int NP>
 __device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x2 x2, float yf, float amax, bool odd,
                                            bool mine, uint32_t pos, PairBwdState<NP>& st, float G[kGrad2d]) {
@@ -1265,9 +1268,10 @@ __device__ __forceinline__ bool pair_terms(float4 f0, float4 f1, float4 f2, f32x
 }
 
 // Reverse walk of one tile's list lst at the lane's pixel pairs, from the CTA's
-// largest last-contributor position down: batches of S records staged as the
-// forward staged them (so chunks start at multiples of 32), the list entries
-// of the next batch down loaded one batch ahead; per chunk the cover masks
+// largest last-contributor position down: batches of S records from the list's
+// start (S is a multiple of 32 in every kernel, so that chunks are the same 32
+// positions in all of them), the list entries of the next batch down loaded one
+// batch ahead; per chunk the cover masks
 // (the forward's from hslot for the list's first hm_chunks chunks, else the
 // cover pass again), then every lane's
 // walk of its records in reverse list order at its pixels with three vector
@@ -1298,9 +1302,8 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
 #pragma unroll
   for (int w = 0; w < NW; ++w) bmax = max(bmax, (int)s_wmax[w]);
 
-  // Batch b covers list positions [b S, min(b S + S, bmax)), b = nb - 1 .. 0
-  // (the forward's batches, so chunks start at multiples of 32).  The last
-  // goes to buffer 0 now (or is already in reuse_buf); the list entries of
+  // Batch b covers list positions [b S, min(b S + S, bmax)), b = nb - 1 .. 0.
+  // The last goes to buffer 0 now (or is already in reuse_buf); the list entries of
   // the one before it are loaded ahead so that its copies issue without
   // waiting.
   const int nb = (bmax + S - 1) / S;
@@ -1373,7 +1376,9 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
         pf_chunk = j - 1;
       }
       bool odd = st.odd_colours > 0;
-      if (st.odd_colours < 0) odd = __any_sync(0xffffffffu, c + lane < cnt && !finite_colour(s_rec[buf][c + lane][2]));
+      if (st.odd_colours < 0)
+        odd = __any_sync(0xffffffffu, c + lane < cnt && !tame(s_rec[buf][c + lane][2].y, s_rec[buf][c + lane][2].z,
+                                                             s_rec[buf][c + lane][2].w));
       const int lim = (int)nlm - (lo + c);           // only positions before a pixel's last contributor
       mine &= lim >= 32 ? 0xffffffffu : (lim <= 0 ? 0u : (1u << lim) - 1u);
       // pass 2, in reverse list order: between wide records every lane walks
@@ -1417,6 +1422,46 @@ __device__ __forceinline__ void pair_bwd_walk(float4 (&s_rec)[2][S][kRecordF4], 
   __syncthreads();
 }
 
+// The reverse walk of a lane's pixels `which` (bit q) of tile g, one by one and record
+// by record from memory.  The separate backward takes the pixels whose dL/dC is not
+// tame through it, so that whatever is there reaches the records that cover that pixel
+// and no other.  Everything is worked out again from the tile's index, so that the
+// common walk before it keeps nothing for it in registers (0 to 1% of the backward, 1 to
+// 5% in persistent 8x8 tiles; with its state kept, up to 6%; selecting at every pixel of
+// the common walk 5 to 9%; a second common walk for such tiles 3%).
+template <int TW, int TH, int NP>
+__device__ __forceinline__ void pixels_alone(const ViewTable& vt, int g, uint32_t which, const float4* __restrict__ rec,
+                                             const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
+                                             const float* __restrict__ Tfin, const uint32_t* __restrict__ ncontrib,
+                                             const float* __restrict__ dLdC, float amax, float* __restrict__ grad2d) {
+  asm volatile("" : "+r"(g));
+  const ViewDev& V = vt.v[view_of_tile(vt, g)];
+  int tx, ty, bx, by, x, y;
+  bool in[2 * NP];
+  tile_xy(V, g, tx, ty);
+  lane_pixels<TW, TH, NP>(V, tx, ty, bx, by, x, y, in);
+  const uint32_t* lst = vals + ranges[g];
+#pragma unroll 1
+  for (; which; which &= which - 1u) {
+    const int q = __ffs(which) - 1, px = x + (q & 1), py = y + q / 2;
+    const int64_t HW = (int64_t)V.width * V.height, at = (int64_t)py * V.width + px;
+    const float* gb = dLdC + 3 * V.pix_off + at;
+    const float gx = gb[0], gy = gb[HW], gz = gb[2 * HW];
+    float T = Tfin[V.pix_off + at], GS = T * (gx * V.bg[0] + gy * V.bg[1] + gz * V.bg[2]);
+#pragma unroll 1
+    for (uint32_t pos = ncontrib[V.pix_off + at]; pos-- > 0u;) {
+      const uint32_t r = lst[pos];
+      const float4* f = rec + (size_t)r * kRecordF4;
+      float G[kGrad2d];
+      if (!bwd_terms<false>(f[0], f[1], f[2], (float)px, (float)py, amax, true, gx, gy, gz, T, GS, G)) continue;
+      float* gdst = grad2d + (size_t)r * kGrad2dStride;
+      red_add_v4(gdst + 0, G[0], G[1], G[2], G[3]);
+      red_add_v4(gdst + 4, G[4], G[5], G[6], G[7]);
+      red_add_v2(gdst + 8, G[8], G[9]);
+    }
+  }
+}
+
 template <int TW, int TH, int S, int NP, bool PERSIST>
 __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW, TH, S, NP)) k_raster_bwd2(
     ViewTable vt, RenderOpts ro, const float4* __restrict__ rec, const uint32_t* __restrict__ vals,
@@ -1430,6 +1475,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
   __shared__ __align__(16) float4 s_rec[2][S][kRecordF4];
   __shared__ uint32_t s_ridx[2][S];
   __shared__ uint32_t s_wmax[NW];
+  __shared__ uint8_t s_alone[NT];   // each lane's pixels whose dL/dC is not tame (bit q)
   __shared__ int s_item;
   if (*status != 0) return;
   const int lane = threadIdx.x & 31;
@@ -1448,6 +1494,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
 
     PairBwdState<NP> bs;
     bs.odd_colours = -1;
+    uint32_t alone = 0u;
     {
       const int W = vt.v[v].width;
       const int64_t HW = (int64_t)W * vt.v[v].height;
@@ -1466,6 +1513,11 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
           gy[h] = inside ? gb[HW + at] : 0.0f;
           gz[h] = inside ? gb[2 * HW + at] : 0.0f;
           bs.nl[2 * i + h] = inside ? ncontrib[pix + at] : 0u;
+          if (!tame(gx[h], gy[h], gz[h])) {   // no records in this walk
+            alone |= 1u << (2 * i + h);
+            gx[h] = gy[h] = gz[h] = 0.0f;
+            bs.nl[2 * i + h] = 0u;
+          }
           ng[h] = inside ? -(T[h] * (gx[h] * bg[0] + gy[h] * bg[1] + gz[h] * bg[2])) : 0.0f;
         }
         bs.T2[i] = pack2(T[0], T[1]);
@@ -1475,8 +1527,12 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
         bs.gz[i] = pack2(gz[0], gz[1]);
       }
     }
-    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, false)>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX, grad2d, (float)x, (float)y,
-                             (float)bx, (float)by, amax, my_field, bs, -1, 0);
+    s_alone[threadIdx.x] = (uint8_t)alone;
+    pair_bwd_walk<TW, TH, S, NP, wide_lanes(NP, false)>(s_rec, s_ridx, s_wmax, rec, vals + range0, hslot, INT_MAX,
+                                                        grad2d, (float)x, (float)y, (float)bx, (float)by, amax,
+                                                        my_field, bs, -1, 0);
+    if (s_alone[threadIdx.x])
+      pixels_alone<TW, TH, NP>(vt, g, s_alone[threadIdx.x], rec, vals, ranges, Tfin, ncontrib, dLdC, amax, grad2d);
   }
   leave<PERSIST>(ctr);
 }
@@ -1547,7 +1603,7 @@ __global__ void __launch_bounds__(PairBlock<TW, TH, NP>::NT, pair_ctas_per_sm(TW
 
     const float* bg = vt.v[v].bg;
     PairBwdState<NP> bs;
-    bs.odd_colours = fs.odd_colours ? 1 : 0;
+    bs.odd_colours = fs.odd_colours ? 1 : 0;   // dL/dC, the L1 term's, is at most 1 / 3
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       float ng[2];
