@@ -696,13 +696,14 @@ constexpr bool pair_tiles(int tw, int th) { return th % (tw % 16 == 0 ? 4 : 8) =
 // launch 108 / 113 and 272 / 247 us; 32640 200 / 206 and 521 / 464 (3.1M Betas
 // 550 / 592 and 1615 / 1512); 64800 (6M Betas x 4K) 1108 / 1106 and 3666 / 2981;
 // 65280, persistent, 420 / 370 and 1006 / 803; 129600 2128 / 2088 and 7166 / 5733.
+// With hit masks the lower line holds whatever the batch: a forward's masks serve a
+// backward with another batch size, so their layout does not depend on it.
 constexpr int kQuadBlocks = 16000, kQuadBlocksLarge = 64000;
 constexpr bool quad_shape(int tw, int th) { return tw % 16 == 0 && th % 8 == 0; }
-inline int lane_pairs(const RenderOpts& ro, int total_tiles) {
+inline int lane_pairs(const RenderOpts& ro, int total_tiles, bool masks) {
   const int px = ro.tile_w * ro.tile_h;
-  return quad_shape(ro.tile_w, ro.tile_h) &&
-                 (int64_t)total_tiles * (px / 128) >= (ro.batch_s <= px / 2 ? kQuadBlocks : kQuadBlocksLarge)
-             ? 2 : 1;
+  const int blocks = masks || ro.batch_s <= px / 2 ? kQuadBlocks : kQuadBlocksLarge;
+  return quad_shape(ro.tile_w, ro.tile_h) && (int64_t)total_tiles * (px / 128) >= blocks ? 2 : 1;
 }
 
 // Records the kernels stage at a time for batches of S: fewer than S where the
@@ -1852,7 +1853,7 @@ cudaError_t fwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
                       float* dL_dcolor, float* l1_partial, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
     if constexpr (quad_shape(TW, TH))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return fwd_pairs<TW, TH, staged(TW, TH, S, 2, true), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
+      if (lane_pairs(ro, vt.total_tiles, hm.words != nullptr) == 2) return fwd_pairs<TW, TH, staged(TW, TH, S, 2, true), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
     return fwd_pairs<TW, TH, staged(TW, TH, S, 1, true), 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, hm, s);
   } else {
     if (sched) {
@@ -1891,7 +1892,7 @@ cudaError_t bwd_shape(const ViewTable& vt, const RenderOpts& ro, const float4* r
                       const int32_t* status, uint32_t* sched, HitMasks hm, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
     if constexpr (quad_shape(TW, TH))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return bwd_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
+      if (lane_pairs(ro, vt.total_tiles, hm.words != nullptr) == 2) return bwd_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
     return bwd_pairs<TW, TH, staged(TW, TH, S, 1, false), 1>(vt, ro, rec, vals, ranges, T_final, n_contrib, dL_dcolor, grad2d, status, sched, hm, s);
   } else {
     if (sched) {
@@ -1931,7 +1932,7 @@ cudaError_t step_shape(const ViewTable& vt, const RenderOpts& ro, const float4* 
                        float* l1_partial, float* grad2d, cudaStream_t s) {
   if constexpr (kPairs<TW, TH>) {
     if constexpr (quad_shape(TW, TH))
-      if (lane_pairs(ro, vt.total_tiles) == 2) return step_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
+      if (lane_pairs(ro, vt.total_tiles, false) == 2) return step_pairs<TW, TH, staged(TW, TH, S, 2, false), 2>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
     return step_pairs<TW, TH, staged(TW, TH, S, 1, false), 1>(vt, ro, rec, vals, ranges, color, T_final, n_contrib, status, sched, target, dL_dcolor, l1_partial, grad2d, s);
   } else {
     return cudaErrorInvalidValue;   // 8 x 4 tiles have no pixel-pair kernels
@@ -1981,7 +1982,7 @@ cudaError_t launch_raster_fwd(const ViewTable& vt, const RenderOpts& ro, const f
 size_t hit_mask_bytes(const ViewTable& vt, const RenderOpts& ro, int64_t cap) {
   // one word per lane (per pixel pair in the pixel-pair kernels) and one per warp
   const bool pairs = pair_tiles(ro.tile_w, ro.tile_h);
-  const int64_t nt = (int64_t)ro.tile_w * ro.tile_h / (pairs ? 2 * lane_pairs(ro, vt.total_tiles) : 1);
+  const int64_t nt = (int64_t)ro.tile_w * ro.tile_h / (pairs ? 2 * lane_pairs(ro, vt.total_tiles, true) : 1);
   const int64_t slots = (std::max<int64_t>(cap, 0) >> 5) + vt.total_tiles + 1;
   return (size_t)slots * (size_t)(nt + nt / 32) * sizeof(uint32_t);
 }
