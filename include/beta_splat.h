@@ -224,7 +224,7 @@ int beta_schedule(const beta_camera* cams, int32_t n_views, const beta_opts* opt
  * than 12 of its threads' pixels, 16 with pairs, 24 with quads): ((pair_capacity >> 5) +
  * total_tiles + 1) x (L x 33/32) x 4 bytes, L = tile pixels / 2 (/ 4 with quads;
  * tile pixels for 8x4 tiles).  Quads are used for 16 x 8 and larger tiles
- * when the views hold at least 16000 blocks of 128 pixels (without hit masks 64000
+ * when the views hold at least 31000 blocks of 128 pixels (without hit masks 64000
  * with batches of more than tile pixels / 2 records).  The layout does not depend on
  * the batch size.  0 for invalid arguments. */
 size_t beta_hit_mask_bytes(const beta_camera* cams /* host */, int32_t n_views, const beta_opts* opt,

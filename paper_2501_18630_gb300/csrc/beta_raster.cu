@@ -686,19 +686,29 @@ __global__ void __launch_bounds__(TW * TH, min_blocks(TW * TH, 1280)) k_raster_b
 // others (8 x 4) the one-pixel-per-lane ones; the hit-mask layout follows.
 constexpr bool pair_tiles(int tw, int th) { return th % (tw % 16 == 0 ? 4 : 8) == 0; }
 
-// Pairs a lane owns.  Two need 16 x 8 blocks and enough of them to fill the chip
-// with half the warps.  At 16x8 / 64 the one launch takes, NP 1 / 2: 9840
-// blocks (4 x 641x479, clustered lists) 130 / 151 us; 16200 (one 1080p view)
-// 253 / 223; 32400 466 / 407; 64800 877 / 752; at 32x16 / 128, 10080 blocks
-// 199 / 220 us, 16320 392 / 333.  Batches of more than two records per quad
-// thread, asked for where lists are long, need four times as many, for a
-// forward by itself to gain too: 16x16 / 256, 16320 blocks, forward and one
-// launch 108 / 113 and 272 / 247 us; 32640 200 / 206 and 521 / 464 (3.1M Betas
-// 550 / 592 and 1615 / 1512); 64800 (6M Betas x 4K) 1108 / 1106 and 3666 / 2981;
-// 65280, persistent, 420 / 370 and 1006 / 803; 129600 2128 / 2088 and 7166 / 5733.
+// Pairs a lane owns.  Two need 16 x 8 blocks and enough of them: half the warps walk
+// the longest lists half as fast.  Forward / backward / one launch at 16x8 / 64 with
+// one pair -> two, us (sheets spread over the views, mixtures cluster in long lists):
+//   16200 blocks, sheets 1M x 1080p        106 / 183 / 252 -> 105 / 158 / 234
+//                 narrow mixture 200k      138 / 216 / 309 -> 198 / 242 / 393
+//   19680, mixture 500k x 8 x 641x479      319 / 517 / 751 -> 402 / 611 / 920
+//   29520, the same x 12                   401 / 674 / 964 -> 487 / 762 / 1164
+//   32400, sheets 1M x 2 x 1080p           187 / 345 / 464 -> 183 / 293 / 424
+//          narrow mixture 200k             177 / 290 / 396 -> 231 / 309 / 484
+//   64800, sheets 1M x 4 x 1080p           340 / 659 / 865 -> 311 / 530 / 751
+//          narrow mixture 1M               459 / 850 / 1118 -> 566 / 832 / 1265
+// The line decides between them: at 16000 / 31000 / 46000 / 64000 blocks the geometric
+// mean over 30 scenes of 12300 to 64800 blocks and eight shapes is, of the time of one
+// pair in scalar arithmetic, backward .821 / .812 / .818 / .829, one launch .830 / .812
+// / .807 / .808, forward .876 / .840 / .821 / .812 (persistent .848 / .845 / .860 /
+// .879, .840 / .825 / .828 / .838, .876 / .851 / .846 / .847), and the worst backward
+// 1.26 / 1.02 / 1.03 / 1.04, the worst one launch 1.21 / 1.04 / 1.00 / 1.00.
+// Batches of more than two records per quad thread, asked for where lists are long,
+// need twice as many, for a forward by itself to gain too (16x16 / 256, 32640 blocks
+// of sheets 200 / 206 us, 64800 of 6M Betas 1108 / 1106, 129600 2128 / 2088).
 // With hit masks the lower line holds whatever the batch: a forward's masks serve a
 // backward with another batch size, so their layout does not depend on it.
-constexpr int kQuadBlocks = 16000, kQuadBlocksLarge = 64000;
+constexpr int kQuadBlocks = 31000, kQuadBlocksLarge = 64000;
 constexpr bool quad_shape(int tw, int th) { return tw % 16 == 0 && th % 8 == 0; }
 inline int lane_pairs(const RenderOpts& ro, int total_tiles, bool masks) {
   const int px = ro.tile_w * ro.tile_h;
