@@ -27,18 +27,16 @@ namespace beta {
 
 // Layout of the projection buffer: records, rectangles, keys and tile masks
 // per (view, primitive), then the rule-B2 worklist (kProjRegion x V entries
-// per projection block) and one entry count per block.
+// per projection block); its size counts one more word per block, unused.
 ProjBuffers proj_layout(void* proj, int32_t pitch, int32_t n_views) {
   ProjBuffers b;
   char* p = (char*)proj;
   const size_t nrec = (size_t)pitch * n_views;
-  const size_t nwork = (size_t)proj_blocks(pitch) * kProjRegion * n_views;
   b.rec = (float4*)p;
   b.rect = (uint2*)(p + nrec * 16 * kRecordF4);
   b.key = (uint32_t*)(p + nrec * (16 * kRecordF4 + 8));
   b.tiles = (uint32_t*)(p + nrec * (16 * kRecordF4 + 12));
   b.work = (uint32_t*)(p + nrec * (16 * kRecordF4 + 16));
-  b.n_work = (uint32_t*)(p + nrec * (16 * kRecordF4 + 16) + nwork * 4);
   return b;
 }
 
@@ -176,7 +174,7 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_blocks_per_sm(M)) k_project(c
                                                  ViewTable vt, RenderOpts ro,
                                                  float4* __restrict__ rec, uint2* __restrict__ rect,
                                                  uint32_t* __restrict__ key, uint32_t* tiles,
-                                                 uint32_t* work, uint32_t* __restrict__ n_work) {
+                                                 uint32_t* work) {
   chain_begin();
   __shared__ uint32_t s_nw;
   if (threadIdx.x == 0) s_nw = 0u;
@@ -266,7 +264,6 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_blocks_per_sm(M)) k_project(c
   for (uint64_t m = need; m; m &= m - 1ull) region[base++] = (uint32_t)(__ffsll((long long)m) - 1) * (uint32_t)pitch + (uint32_t)i;
   __syncthreads();   // the list, and the tile masks of the view loop, which are written again
   const uint32_t nw = s_nw;
-  if (threadIdx.x == 0) n_work[blockIdx.x] = nw;
   for (uint32_t k = threadIdx.x; k < nw; k += blockDim.x) narrow_tiles(planes, pitch, vt, ro, region[k], tiles);
 }
 
@@ -299,23 +296,33 @@ __device__ __forceinline__ void view_geo_bwd(const PrimGeo& pg, const ViewDev& V
 // rotation matrix, the scales and the lobe directions are summed over views
 // first and taken through the view-independent maps once.
 // ---------------------------------------------------------------------------
+constexpr int kBwdThreads = 128;
 // 3 CTAs per SM, up to 170 registers a thread (4 of them: 128 registers, spills,
-// 535 against 380 us on 1M primitives x 16 views)
-constexpr int kBwdThreads = 128, kBwdBlocksPerSM = 3;
-// parameters of two blocks of primitives and 2D gradients of two (block, view) pairs
-constexpr size_t bwd_smem(int lobes) {
-  return (size_t)kBwdThreads * (2 * (15 + 6 * lobes) * sizeof(float) + 2 * 3 * sizeof(float4));
-}
+// 535 against 380 us on 1M primitives x 16 views with 3 lobes); 8 lobes 2, which
+// spill nothing (500k x 8 views 304 against 358 us; 7 lobes 291 with 3, 290 with 2,
+// 1M x 1 view 230 and 255).
+constexpr int bwd_blocks_per_sm(int lobes) { return lobes <= 7 ? 3 : 2; }
 
-// A persistent grid takes blocks of 128 primitives: while a block's last view is
-// chained back and its gradients are stored, the next block's parameters and its
-// first view's 2D gradients are copied into shared memory (within a block, view
-// v + 1's 2D gradients while view v is processed).  With one block per CTA and
+// Up to four lobes a persistent grid takes blocks of 128 primitives: while a block's
+// last view is chained back and its gradients are stored, the next block's parameters
+// and its first view's 2D gradients are copied into shared memory (within a block,
+// view v + 1's 2D gradients while view v is processed).  With one block per CTA and
 // the parameters loaded at its start, the 12 warps an SM holds waited for them:
 // 1M primitives x 1 view 100 -> 62 us (its 350 MB at the copy rate: 51), x 16
-// views 409 -> 380, 6M x 8 x 4K 1.39 -> 1.25 ms.
+// views 409 -> 380, 6M x 8 x 4K 1.39 -> 1.25 ms; with 4 lobes 146 -> 111 at 1M x 1,
+// 199 -> 181 at 500k x 8.  More lobes keep one block per CTA: the shared memory for
+// two blocks' parameters costs CTAs or L1 cache (5 lobes 151 with against 163 us at
+// 1M x 1 but 245 / 219 at 500k x 8; 6 lobes 197 / 196 and 310 / 252; 8 lobes 422 /
+// 260 and 690 / 304).
+constexpr bool bwd_ahead(int lobes) { return lobes <= 4; }
+// parameters of two blocks of primitives (copied ahead) and 2D gradients of two
+// (block, view) pairs
+constexpr size_t bwd_smem(int lobes) {
+  return (size_t)kBwdThreads * ((bwd_ahead(lobes) ? 2 * (15 + 6 * lobes) * sizeof(float) : 0) + 2 * 3 * sizeof(float4));
+}
+
 template <int M>
-__global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(const float* __restrict__ planes, int n,
+__global__ void __launch_bounds__(kBwdThreads, bwd_blocks_per_sm(M)) k_project_bwd(const float* __restrict__ planes, int n,
                                                      int pitch, ViewTable vt, RenderOpts ro,
                                                      float* __restrict__ grad2d,
                                                      float* __restrict__ gout,
@@ -326,6 +333,7 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
   float* const s_p = s_dyn + 2 * 3 * 4 * kBwdThreads;                    // [2][NP][kBwdThreads]
   constexpr int NP = 15 + 6 * M;
   constexpr int MM = M > 0 ? M : 1;
+  constexpr bool AHEAD = bwd_ahead(M);
   const int tid = threadIdx.x;
   const int nblk = (n + kBwdThreads - 1) / kBwdThreads;
   const bool bad = *status != 0;
@@ -347,15 +355,17 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
   };
   int slot = 0, pbuf = 0;
   if ((int)blockIdx.x < nblk) {
-    fetch_params(blockIdx.x, 0);
+    if (AHEAD) fetch_params(blockIdx.x, 0);
     fetch_g(blockIdx.x, 0, 0);
   }
   cp_async_commit();
   for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x, pbuf ^= 1) {
     const int i = blk * kBwdThreads + tid;
     const int next = blk + gridDim.x;
-    cp_async_wait<0>();
-    __syncthreads();   // this block's parameters have landed; the other buffer is free
+    if (AHEAD) {
+      cp_async_wait<0>();
+      __syncthreads();   // this block's parameters have landed; the other buffer is free
+    }
     float gp[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) gp[k] = 0.0f;
@@ -363,7 +373,8 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
     bool ok = i < n;
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-      p[k] = s_p[(pbuf * NP + k) * kBwdThreads + tid];
+      if (AHEAD) p[k] = s_p[(pbuf * NP + k) * kBwdThreads + tid];
+      else p[k] = i < n ? planes[(size_t)k * pitch + i] : 0.0f;
       ok = ok && isfinite(p[k]);
     }
     if (ok) ok = (p[11] >= ro.b_lo) && (p[11] < ro.b_hi);
@@ -384,14 +395,14 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocksPerSM) k_project_bwd(co
       for (int v = 0; v < vt.n_views; ++v) {
         const ViewDev& V = vt.v[v];
         float4* g2 = reinterpret_cast<float4*>(grad2d + ((size_t)v * pitch + i) * kGrad2dStride);
-        if (v > 0) cp_async_wait<0>();   // the thread's own copies
+        if (v > 0 || !AHEAD) cp_async_wait<0>();   // the thread's own copies
         const float4 ga4 = s_g[(slot * 3 + 0) * kBwdThreads + tid], gb4 = s_g[(slot * 3 + 1) * kBwdThreads + tid],
                      gc4 = s_g[(slot * 3 + 2) * kBwdThreads + tid];
         slot ^= 1;
         if (v + 1 < vt.n_views) {
           fetch_g(blk, v + 1, slot);
         } else if (next < nblk) {
-          fetch_params(next, pbuf ^ 1);
+          if (AHEAD) fetch_params(next, pbuf ^ 1);
           fetch_g(next, 0, slot);
         }
         cp_async_commit();
@@ -572,7 +583,7 @@ static cudaError_t launch_project_m(const float* planes, int n, int pitch, const
   if (grid < 1) return cudaSuccess;
   static_assert(kFwdThreads == kProjRegion, "a projection block owns one worklist region");
   launch_chained(k_project<M>, grid, kFwdThreads, 0, s, planes, n, pitch, vt, ro, pb.rec, pb.rect, pb.key, pb.tiles,
-                                            pb.work, pb.n_work);
+                                            pb.work);
   return cudaGetLastError();
 }
 
@@ -585,9 +596,7 @@ static cudaError_t launch_project_bwd_m(const float* planes, int n, int pitch, c
   constexpr size_t smem = bwd_smem(M);
   const cudaError_t e = cudaFuncSetAttribute(k_project_bwd<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // CTAs an SM's 227 KB of shared memory hold (8 lobes: two)
-  constexpr int per_sm = (int)std::min<size_t>(kBwdBlocksPerSM, 227 * 1024 / (smem + 1024));
-  const int grid = std::min(nblk, device_sm_count() * per_sm);
+  const int grid = bwd_ahead(M) ? std::min(nblk, device_sm_count() * bwd_blocks_per_sm(M)) : nblk;
   launch_chained(k_project_bwd<M>, grid, kBwdThreads, smem, s, planes, n, pitch, vt, ro, grad2d, gout, status);
   return cudaGetLastError();
 }
