@@ -223,19 +223,22 @@ cudaError_t launch_adam(int n_lobes, float* planes, const float* grad, float* m,
 // random word r of a dead primitive picks t = floor(r W_total / 2^32), the
 // source being the first i with W_i > t.
 //
-//   k_reloc_weights  weights (bit 31: dead), old logits, zeroed copy counts,
-//                    per-block weight sums and dead counts
+//   k_reloc_weights  weights summed up inside blocks of 256, old logits, zero copy
+//                    counts (bit 31: dead), per-block weight sums and dead counts
 //   k_reloc_scan     exclusive scan of the block sums, totals (one CTA)
-//   k_reloc_sample   a warp per dead primitive: its source (a 32-way search of
-//                    the block offsets, then the block's 256 weights), copy counts
+//   k_reloc_sample   the source of every dead primitive (a search of the block
+//                    offsets, then one inside the block) and copy counts
 //   k_reloc_copy     the copies, kCopyPlanes planes of one primitive a thread,
 //                    and the new opacity logits of sources and copies (from the
 //                    old logits, so in any order)
 // Bound by scattered 4-byte reads and writes: 3% dead among 1M touch a fifth of
 // all 32-byte sectors of parameters and moments, 260 MB of DRAM traffic.  A
 // thread per dead primitive walking all 33 planes x 3 arrays took 92 us, a warp
-// per dead one (lane = plane) 113; one counter for the number of dead and a
-// binary search of 1M cumulative weights per dead thread took 38.
+// per dead one (lane = plane) 113.  The sources (the whole call on 1M with 3% dead
+// anywhere / 3% in a row / half anywhere): a binary search of 1M cumulative 64-bit
+// weights per dead thread and one counter for the number of dead 122 / 62 / 206 us;
+// a warp per dead one with 32-way searches 86 / 64 / 274; a thread per dead one with
+// two binary searches, of 31 KB of block offsets and of the block's 1 KB, 84 / 37 / 135.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -248,42 +251,45 @@ __device__ __forceinline__ float rule_opacity(float x) {
   return __fdiv_rn(1.0f, __fadd_rn(1.0f, e));
 }
 
-__device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long x, unsigned long long* s_w) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  if (lane == 0) s_w[warp] = x;
-  __syncthreads();
-  unsigned long long t = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_w[w];
-  __syncthreads();
-  return t;
-}
-
 constexpr int kRelocBlock = 256;   // primitives per block of weights
 
 __global__ void __launch_bounds__(kRelocBlock) k_reloc_weights(const float* __restrict__ planes, int n, int pitch,
-                                                               float min_opacity, uint32_t* __restrict__ w,
+                                                               float min_opacity, uint32_t* __restrict__ before,
                                                                uint32_t* __restrict__ copies,
                                                                float* __restrict__ logit,
                                                                unsigned long long* __restrict__ bsum,
                                                                uint32_t* __restrict__ bdead) {
   chain_begin();
-  __shared__ unsigned long long s_w[8];
+  __shared__ uint32_t s_w[kRelocBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t wi = 0;
+  uint32_t wi = 0, mark = 0;
   if (i < n) {
     const float x = planes[(size_t)10 * pitch + i];
     logit[i] = x;
     const float o = rule_opacity(x);
-    wi = o < min_opacity ? kDeadBit : (uint32_t)__fmul_rn(o, 16777216.0f);
-    w[i] = wi;
-    copies[i] = 0u;
+    if (o < min_opacity) mark = kDeadBit;
+    else wi = (uint32_t)__fmul_rn(o, 16777216.0f);
+    copies[i] = mark;
   }
-  const int dead = __syncthreads_count((wi & kDeadBit) != 0u);
-  const unsigned long long t = block_sum_u64(wi & ~kDeadBit, s_w);
+  uint32_t inc = wi;   // at most 2^24 each
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) s_w[warp] = inc;
+  const int dead = __syncthreads_count(mark != 0u);
+  uint32_t pre = 0;
+  unsigned long long total = 0;
+#pragma unroll
+  for (int w = 0; w < kRelocBlock / 32; ++w) {
+    if (w < warp) pre += s_w[w];
+    total += s_w[w];
+  }
+  if (i < n) before[i] = pre + inc - wi;   // below 2^32: 255 weights at most
   if (threadIdx.x == 0) {
-    bsum[blockIdx.x] = t;
+    bsum[blockIdx.x] = total;
     bdead[blockIdx.x] = (uint32_t)dead;
   }
 }
@@ -345,60 +351,38 @@ __global__ void __launch_bounds__(1024) k_reloc_scan(unsigned long long* __restr
   }
 }
 
-__global__ void __launch_bounds__(kRelocBlock) k_reloc_sample(const uint32_t* __restrict__ w, int n,
+// The source of draw t is the last primitive with at most t before it: the last block
+// whose offset is <= t (t < T, so its weights reach past t), then the last place in it.
+__global__ void __launch_bounds__(kRelocBlock) k_reloc_sample(const uint32_t* __restrict__ before, int n,
                                                               const unsigned long long* __restrict__ boff, int nb,
                                                               const unsigned long long* __restrict__ total,
                                                               const uint32_t* __restrict__ rnd,
-                                                              int32_t* __restrict__ src,
-                                                              uint32_t* __restrict__ copies) {
+                                                              int32_t* __restrict__ src, uint32_t* copies) {
   chain_begin();
-  const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned long long T = *total;
-  const bool dead = i < n && (w[i] & kDeadBit) && T > 0;
+  const bool dead = i < n && (copies[i] & kDeadBit) && T > 0;
   int32_t mine = -1;
-  for (uint32_t todo = __ballot_sync(0xffffffffu, dead); todo; todo &= todo - 1u) {
-    const int from = __ffs(todo) - 1;
-    const int d = __shfl_sync(0xffffffffu, i, from);
+  if (dead) {
     // t = floor(r T / 2^32), exactly: T = hi 2^32 + lo
-    const unsigned long long r = rnd[d];
+    const unsigned long long r = rnd[i];
     const unsigned long long t = r * (T >> 32) + ((r * (T & 0xffffffffull)) >> 32);
-    // the last block whose offset is <= t: t < T, so its weights reach past t
-    int lo = 0, len = nb;
-    while (len > 1) {
-      const int step = (len + 31) >> 5;
-      const bool le = lane * step < len && boff[lo + lane * step] <= t;
-      const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
-      lo += k * step;
-      len = min(step, len - k * step);
+    int lo = 0;
+    for (int len = nb; len > 1;) {
+      const int half = len >> 1;
+      const bool up = boff[lo + half] <= t;
+      lo += up ? half : 0;
+      len = up ? len - half : half;
     }
-    // first primitive of the block whose inclusive sum exceeds t
-    const unsigned long long rem = t - boff[lo];
-    const int base = lo * kRelocBlock + lane * (kRelocBlock / 32);
-    uint32_t x[kRelocBlock / 32];
-    unsigned long long sum = 0;
-#pragma unroll
-    for (int q = 0; q < kRelocBlock / 32; ++q) {
-      x[q] = base + q < n ? w[base + q] & ~kDeadBit : 0u;
-      sum += x[q];
+    const uint32_t rem = (uint32_t)(t - boff[lo]);   // inside the block: below 2^32
+    mine = lo * kRelocBlock;
+    for (int len = min(kRelocBlock, n - mine); len > 1;) {
+      const int half = len >> 1;
+      const bool up = before[mine + half] <= rem;
+      mine += up ? half : 0;
+      len = up ? len - half : half;
     }
-    unsigned long long inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    const int who = __ffs(__ballot_sync(0xffffffffu, inc > rem)) - 1;
-    unsigned long long run = inc - sum;
-    int at = 0;
-#pragma unroll
-    for (int q = 0; q < kRelocBlock / 32; ++q) {
-      run += x[q];
-      at += run <= rem ? 1 : 0;
-    }
-    const int s = __shfl_sync(0xffffffffu, base + at, who);
-    if (lane == 0) atomicAdd(&copies[s], 1u);
-    if (lane == from) mine = s;
+    atomicAdd(&copies[mine], 1u);
   }
   if (i < n) src[i] = mine;
 }
@@ -419,7 +403,7 @@ __global__ void __launch_bounds__(256) k_reloc_copy(float* __restrict__ planes, 
   const int32_t s = src[i];
   if (blockIdx.y + 1 == gridDim.y) {
     const int from = s >= 0 ? s : i;
-    const uint32_t c = copies[from];
+    const uint32_t c = copies[from] & ~kDeadBit;
     if (c != 0u) {
       const float inv_n = 1.0f / (float)(c + 1u);
       // -log(1 - o) = softplus(logit), from the logit (1 - o by subtraction loses
@@ -453,7 +437,7 @@ __global__ void __launch_bounds__(256) k_reloc_copy(float* __restrict__ planes, 
 
 }  // namespace
 
-// workspace carve-up: weights u32[n], old logits f32[n], block sums u64[nb], dead
+// workspace carve-up: weight sums u32[n], old logits f32[n], block sums u64[nb], dead
 // counts u32[nb], total u64, copies u32[n], sources i32[n] (256-byte aligned pieces)
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -468,16 +452,17 @@ cudaError_t launch_relocate(int n, int pitch, int n_planes, float* planes, float
   if (n <= 0) return cudaSuccess;
   const int nb = (n + kRelocBlock - 1) / kRelocBlock;
   char* p = (char*)ws;
-  uint32_t* w = (uint32_t*)p;                   p += al256((size_t)n * 4);
+  uint32_t* before = (uint32_t*)p;              p += al256((size_t)n * 4);
   float* logit = (float*)p;                     p += al256((size_t)n * 4);
   unsigned long long* bsum = (unsigned long long*)p; p += al256((size_t)nb * 8);
   uint32_t* bdead = (uint32_t*)p;               p += al256((size_t)nb * 4);
   unsigned long long* total = (unsigned long long*)p; p += al256(8);
   uint32_t* copies = (uint32_t*)p;              p += al256((size_t)n * 4);
   int32_t* src = src_out ? src_out : (int32_t*)p;
-  launch_chained(k_reloc_weights, nb, kRelocBlock, 0, s, planes, n, pitch, min_opacity, w, copies, logit, bsum, bdead);
+  launch_chained(k_reloc_weights, nb, kRelocBlock, 0, s, planes, n, pitch, min_opacity, before, copies, logit, bsum,
+                 bdead);
   launch_chained(k_reloc_scan, 1, 1024, 0, s, bsum, bdead, nb, total, d_count);
-  launch_chained(k_reloc_sample, nb, kRelocBlock, 0, s, w, n, bsum, nb, total, rnd, src, copies);
+  launch_chained(k_reloc_sample, nb, kRelocBlock, 0, s, before, n, bsum, nb, total, rnd, src, copies);
   const dim3 grid((n + 255) / 256, (n_planes + kCopyPlanes - 1) / kCopyPlanes + 1);
   launch_chained(k_reloc_copy, grid, 256, 0, s, planes, m, v, n, pitch, n_planes, src, copies, logit);
   return cudaGetLastError();
