@@ -1690,8 +1690,11 @@ __global__ void k_sched_scatter(const uint32_t* __restrict__ ranges, int total_t
 
 // The whole schedule in one CTA, for few tiles: three launches of 2.5 to 5 us each
 // were 10 us of a 208 us step over 4 x 641x479 (4920 tiles).  Lanes of a warp in
-// the same bucket count, and take their places, together.
-constexpr int kSchedOneTiles = 16384, kSchedThreads = 1024;
+// the same bucket count, and take their places, together.  One launch / three, on
+// lists of all lengths 3.6 / 4.2 us at 1920 tiles, 6.7 / 6.4 at 8192, 8.5 / 7.0 at
+// 10240, 11.3 / 8.9 at 16384; where most lists are empty, one atomic address, 5.6 / 7.6
+// at 8192, 7.3 / 8.5 at 10240.
+constexpr int kSchedOneTiles = 8192, kSchedThreads = 1024;
 __global__ void __launch_bounds__(kSchedThreads) k_sched_one(const uint32_t* __restrict__ ranges, int total_tiles,
                                                              uint32_t* sched, const int32_t* __restrict__ status) {
   chain_begin();
