@@ -1776,27 +1776,27 @@ __global__ void __launch_bounds__(256) k_l1(ViewTable vt, const float* __restric
 
 // One CTA per view.  Its loads are the time, so eight are in flight per thread
 // (256 threads with one each: 35 us for 16 views of 1080p at 16x8 tiles, 127 us
-// for 8 of 4K; now 10 and 35); absent values are not added, the FP64 pipe being
-// narrow.
+// for 8 of 4K; now 15 and 42); no more threads than that takes (512 for a 64x64 view:
+// 1.3 us longer), and absent values are not added, the FP64 pipe being narrow.
 constexpr int kReduceThreads = 512, kReduceLoads = 8;
 __global__ void __launch_bounds__(kReduceThreads) k_l1_reduce(ViewTable vt, const float* __restrict__ partial,
                                                               int total_blocks, float* __restrict__ loss) {
   chain_begin();
-  __shared__ double s_w[32];
-  const int v = blockIdx.x;
+  __shared__ double s_w[kReduceThreads / 32];
+  const int v = blockIdx.x, nt = blockDim.x;
   const int b0 = vt.v[v].pad0;
   const int b1 = (v + 1 < vt.n_views) ? vt.v[v + 1].pad0 : total_blocks;
   double acc = 0.0;
-  for (int64_t c = b0; c < b1; c += kReduceThreads * kReduceLoads) {
+  for (int64_t c = b0; c < b1; c += nt * kReduceLoads) {
     float x[kReduceLoads];
 #pragma unroll
     for (int q = 0; q < kReduceLoads; ++q) {
-      const int64_t b = c + q * kReduceThreads + threadIdx.x;
+      const int64_t b = c + q * nt + threadIdx.x;
       x[q] = b < b1 ? partial[b] : 0.0f;
     }
 #pragma unroll
     for (int q = 0; q < kReduceLoads; ++q)
-      if (c + q * kReduceThreads < b1) acc += (double)x[q];
+      if (c + q * nt < b1) acc += (double)x[q];
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
@@ -1804,10 +1804,20 @@ __global__ void __launch_bounds__(kReduceThreads) k_l1_reduce(ViewTable vt, cons
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_w[w];
+    for (int w = 0; w < nt / 32; ++w) t += s_w[w];
     const double HW = (double)vt.v[v].width * vt.v[v].height;
     loss[v] = (float)(t / (3.0 * HW));
   }
+}
+
+// The sums of every view's partials [pad0 of the view, pad0 of the next).
+cudaError_t launch_l1_reduce(const ViewTable& vt, const float* partial, int total_blocks, float* loss, cudaStream_t s) {
+  int most = 0;
+  for (int v = 0; v < vt.n_views; ++v)
+    most = std::max(most, (v + 1 < vt.n_views ? vt.v[v + 1].pad0 : total_blocks) - vt.v[v].pad0);
+  const int threads = std::min(kReduceThreads, std::max(1, (most + 32 * kReduceLoads - 1) / (32 * kReduceLoads)) * 32);
+  launch_chained(k_l1_reduce, vt.n_views, threads, 0, s, vt, partial, total_blocks, loss);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -2018,8 +2028,7 @@ cudaError_t launch_raster_fwd_l1(const ViewTable& vt_in, const RenderOpts& ro, c
   if (e != cudaSuccess) return e;
   ViewTable vt = vt_in;   // the reduce finds view v's partials from tile_off[v]
   for (int v = 0; v < vt.n_views; ++v) vt.v[v].pad0 = vt.v[v].tile_off;
-  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, vt.total_tiles, loss);
-  return cudaGetLastError();
+  return launch_l1_reduce(vt, ws, vt.total_tiles, loss, s);
 }
 
 bool raster_step_supported(const RenderOpts& ro) { return pair_tiles(ro.tile_w, ro.tile_h); }
@@ -2040,8 +2049,7 @@ cudaError_t launch_raster_step_l1(const ViewTable& vt_in, const RenderOpts& ro, 
   if (e != cudaSuccess) return e;
   ViewTable vt = vt_in;   // the reduce finds view v's partials from tile_off[v]
   for (int v = 0; v < vt.n_views; ++v) vt.v[v].pad0 = vt.v[v].tile_off;
-  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, vt.total_tiles, loss);
-  return cudaGetLastError();
+  return launch_l1_reduce(vt, ws, vt.total_tiles, loss, s);
 }
 
 cudaError_t launch_raster_bwd(const ViewTable& vt, const RenderOpts& ro, const float4* rec,
@@ -2075,8 +2083,7 @@ cudaError_t launch_l1(const ViewTable& vt_in, const float* color, const float* t
   int nb = l1_blocks(vt);
   if (nb <= 0) return cudaSuccess;
   launch_chained(k_l1, nb, 256, 0, s, vt, color, target, dL_dcolor, ws);
-  launch_chained(k_l1_reduce, vt.n_views, kReduceThreads, 0, s, vt, ws, nb, loss);
-  return cudaGetLastError();
+  return launch_l1_reduce(vt, ws, nb, loss, s);
 }
 
 }  // namespace beta
