@@ -249,6 +249,10 @@ class Rasterizer:
         self._composite(planes)
         self._state_read.synchronize()
         st, k = int(self._host_status[0]), int(self._host_count[0])
+        if st != _lib.BETA_OK:
+            # the raster kernels in flight write nothing, but read the status word:
+            # they end before a buffer is replaced or the caller may drop them all
+            torch.cuda.current_stream().synchronize()
         if st == _lib.BETA_ERR_CAPACITY:
             self._alloc_pairs(int(math.ceil(k * 1.25)) + 1024)
             self.bin_sort(planes)
