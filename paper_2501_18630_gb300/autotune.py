@@ -4,7 +4,8 @@ raster forward + backward as one launch or two, by timing each candidate's
 captured CUDA graph on the actual workload.
 
 Results are cached in a JSON file keyed by (primitive count, lobes, view
-resolutions, device name), so a workload is tuned once per machine.
+resolutions, device name, library sources), so a workload is tuned once per
+machine and again when a kernel has changed.
 """
 from __future__ import annotations
 
@@ -14,7 +15,7 @@ import time
 
 import torch
 
-from . import _lib
+from . import _lib, build
 from .batched import BatchedStep
 
 # (tile_w, tile_h, batch_s, persistent[, fused]): fused (default True) runs the
@@ -40,7 +41,8 @@ def cache_path() -> str:
 
 def workload_key(n: int, n_lobes: int, cameras, device) -> str:
     res = ",".join(f"{c.width}x{c.height}" for c in cameras)
-    return f"v5;n={n};M={n_lobes};views={res};dev={torch.cuda.get_device_name(device)}"
+    return (f"v6;src={build.source_hash()};n={n};M={n_lobes};views={res}"
+            f";dev={torch.cuda.get_device_name(device)}")
 
 
 def _load():
