@@ -520,7 +520,6 @@ struct ProjBuffers {
   uint32_t* tiles;   // [V * pitch]  rule B2 tiles of the rectangle (bit r w + q; all ones: every tile)
   uint32_t* work;    // records rule B2 applies to: projection block b owns entries
                      // [b kProjRegion V, (b + 1) kProjRegion V), in arbitrary order
-  uint32_t* n_work;  // [projection blocks] entries of each block's region
 };
 
 constexpr int kProjRegion = 256;   // primitives per projection block (its worklist region)
