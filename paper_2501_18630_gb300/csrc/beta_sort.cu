@@ -543,12 +543,20 @@ __device__ __forceinline__ void warp_bitonic(K (&k)[E], int lane) {
   }
 }
 
-// How many of the warp's items (lane L: items L E .. L E + E - 1) are less than the
-// one before them?
+// Are the warp's items (lane L: items L E .. L E + E - 1) in ascending order?
 template <int E>
-__device__ __forceinline__ int warp_inversions(const u64 (&k)[E], int lane) {
+__device__ __forceinline__ bool warp_sorted(const u64 (&k)[E], int lane) {
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j + 1 < E; ++j) ok = ok && k[j] <= k[j + 1];
   const u64 prev = __shfl_up_sync(0xffffffffu, k[E - 1], 1);
-  int bad = lane > 0 && k[0] < prev ? 1 : 0;
+  return __all_sync(0xffffffffu, ok && (lane == 0 || prev <= k[0]));
+}
+
+// How many of a lane's items are less than the one before them, over the warp?
+template <int E>
+__device__ __forceinline__ int warp_inversions(const u64 (&k)[E]) {
+  int bad = 0;
 #pragma unroll
   for (int j = 0; j + 1 < E; ++j) bad += k[j + 1] < k[j] ? 1 : 0;
   return __reduce_add_sync(0xffffffffu, bad);
@@ -562,11 +570,13 @@ __device__ __forceinline__ int warp_inversions(const u64 (&k)[E], int lane) {
 // 64-bit one (1156 instructions a list before, at 98 items on average).  The
 // items are gathered by position and checked: keys that the shift (or the
 // scene) made equal can be out of order, and a few odd-even passes over
-// neighbours put such pairs right.  Where they are too many for that the items
-// are sorted outright; at once where the keys are all the same or, in the larger
-// sorts, twelve of a sample of 32 have an equal among three others of it (bin_sort
-// of lists of 1082 with one depth or three: 64-bit items 460 us, words and all the
-// passes first 526, this 404 to 408; with distinct depths 456, 389, 364).
+// neighbours put such pairs right; if that is not enough the items are sorted
+// outright.  Lists of more than 128 are sorted outright as soon as they are
+// seen to need it: where the keys are all the same, where twelve of a sample of
+// 32 have an equal among three others of it, and where too many neighbours are
+// out of order for the passes (bin_sort of lists of 1082 with one depth or
+// three: 64-bit items 460 us, words and all the passes first 526, this 400 to
+// 404; with distinct depths 456, 386, 360).
 template <int E>
 __device__ __forceinline__ void warp_sort_items(u64 (&k)[E], const u64* sm, int s0, int lane) {
   constexpr int kPosBits = 5 + (E >= 2) + (E >= 4) + (E >= 8) + (E >= 16);
@@ -581,15 +591,16 @@ __device__ __forceinline__ void warp_sort_items(u64 (&k)[E], const u64* sm, int 
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  bool words = lo < hi;
-  if (E >= 8) {
+  constexpr bool kTies = E >= 8;             // (in the smaller sorts the test costs more than it saves)
+  bool words = true;
+  if (kTies) {
     const uint32_t x1 = __shfl_xor_sync(0xffffffffu, c[0], 1), x2 = __shfl_xor_sync(0xffffffffu, c[0], 2),
                    x4 = __shfl_xor_sync(0xffffffffu, c[0], 4);
     const bool tied = c[0] == x1 || c[0] == x2 || c[0] == x4;
-    words = words && __popc(__ballot_sync(0xffffffffu, tied)) < 12;
+    words = lo < hi && __popc(__ballot_sync(0xffffffffu, tied)) < 12;
   }
   if (words) {
-    const int shift = max(0, kPosBits - __clz(hi - lo));
+    const int shift = hi > lo ? max(0, kPosBits - __clz(hi - lo)) : 0;
 #pragma unroll
     for (int j = 0; j < E; ++j)
       c[j] = c[j] == 0xffffffffu ? c[j] : ((c[j] - lo) >> shift) << kPosBits | (uint32_t)(j * 32 + lane);
@@ -598,10 +609,10 @@ __device__ __forceinline__ void warp_sort_items(u64 (&k)[E], const u64* sm, int 
     // a pad's word has all position bits set: the last position, itself a pad
 #pragma unroll
     for (int j = 0; j < E; ++j) k[j] = sm[sidx(s0 + (int)(c[j] & (32 * E - 1)))];
-    int bad = warp_inversions<E>(k, lane);
-    if (bad == 0) return;
+    if (warp_sorted<E>(k, lane)) return;
+    const int passes = E < 2 || (kTies && warp_inversions<E>(k) > 4 * E) ? 0 : 3;
 #pragma unroll 1
-    for (int pass = 0; E >= 2 && bad <= 4 * E && pass < 3; ++pass) {   // warp-uniform
+    for (int pass = 0; pass < passes; ++pass) {
 #pragma unroll
       for (int odd = 0; odd < 2; ++odd)
 #pragma unroll
@@ -614,8 +625,7 @@ __device__ __forceinline__ void warp_sort_items(u64 (&k)[E], const u64* sm, int 
       const u64 next = __shfl_down_sync(0xffffffffu, k[0], 1), prev = __shfl_up_sync(0xffffffffu, k[E - 1], 1);
       if (lane < 31 && next < k[E - 1]) k[E - 1] = next;
       if (lane > 0 && k[0] < prev) k[0] = prev;
-      bad = warp_inversions<E>(k, lane);
-      if (bad == 0) return;
+      if (warp_sorted<E>(k, lane)) return;
     }
   } else {
 #pragma unroll
