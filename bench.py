@@ -592,8 +592,8 @@ def main():
             torch.cuda.synchronize()
             n_dead = int(cnt.item())
         extras["relocation"] = {"ms": e0.elapsed_time(e1), "n_betas": sc.n, "relocated": n_dead,
-                                "what": "beta_relocate: fixed-rule opacities, 64-bit cumulative weights, one "
-                                        "binary search per dead primitive, opacity-only update, copies"}
+                                "what": "beta_relocate: fixed-rule opacities, cumulative weights by blocks, two "
+                                        "binary searches per dead primitive, opacity-only update, copies"}
         del opt_planes, adam, flush, reloc_planes, radam
 
         # ---- the composite loss with the DSSIM term (Sec. 3.4), HBM-bound ---
